@@ -71,9 +71,21 @@ struct DevMem {
 
 struct ObjBufs {
     DevMem R, Rx, Rt, C;      // C stays empty when the collision cloud is R itself
+    DevMem nodes, leaves;     // matching cells of R
     int M = 0, Mpad = 0, Mc = 0;
-    bool set = false;
+    bool set = false, cells_built = false;
 };
+
+// Matching through cells (k_cells.cu): for clouds of kCellMinM points and more (the screening
+// reads the same eight tiles for any smaller one) up to kCellMaxM (the build's 32-bit
+// counters cannot overflow below it), once the passes known of on the present objects (those of
+// an asicp_run, or the asicp_step calls so far) would take longer through the screening than
+// the build: screening and exact choice take 1 us per kCellRate pairs, the build 100 us + 1 us
+// per kCellRatePts points (measured: 0.27 ms at 8192 points, 1.4 ms at 65536), the matching
+// through the cells little beside either.
+constexpr int kCellMinM = 1024, kCellMaxM = 1 << 18;
+constexpr double kCellRate = 1.65e7, kCellRatePts = 50.0;
+constexpr size_t kCellScratch = (size_t)256 << 20;   // scratch of one build launch (at least one object)
 
 enum { kTimeMatch = 0, kTimeCollide = 1, kTimeCollideNN = 2, kTimeFinalize = 3, kTimeStein = 4, kTimeExact = 5,
        kTimeKinds = 6 };
@@ -103,6 +115,9 @@ struct asicp_ctx {
 
     int fwd_variant = 0;              // forward-matching kernel shape (autotuner's choice)
     bool tuned = false;
+    bool cells_oom = false;           // no room for matching cells: the screening is used
+    bool cells_on = false;            // the passes being launched match through the cells
+    double cells_owed = 0.0;          // microseconds of screening on the present objects so far
     bool expire_test = false;         // the float32 matching kernels' first copy waits expire (testing)
 
     // layout (rebuilt when objects, particle counts or N change)
@@ -112,7 +127,7 @@ struct asicp_ctx {
     std::vector<int> grp_off_h;
     std::vector<ObjMeta> objmeta_h;
 
-    DevMem partgrp, grpoff, objmeta, items, ctaoff, com, frame, colitems, collist, box, stage, S, pconst, dmeta, theta, fsums,
+    DevMem partgrp, grpoff, objmeta, items, ctaoff, com, frame, colitems, collist, box, stage, S, Ssort, cellwork, pconst, dmeta, theta, fsums,
         csums, ncol, colidx, cost, grad, prev, frozen, phi, h, order, errw, out7, outc, outi, nnidx, tccand, dbg_d2, dbg_sp,
         dbg_colnn;
 
@@ -297,6 +312,8 @@ void build_layout(asicp_ctx *c)
         m.R = b.R.as<float4>();
         m.Rx = b.Rx.as<ulonglong2>();
         m.Rt = b.Rt.as<float>();
+        m.nodes = b.nodes.as<int2>();
+        m.leaves = b.leaves.as<int>();
         m.C = b.C.p ? b.C.as<float4>() : b.R.as<float4>();
         m.M = b.M;
         m.Mpad = b.Mpad;
@@ -441,6 +458,90 @@ void select_minibatch(asicp_ctx *c, int k)
     ck(launch_store_meta(c->objmeta.as<ObjMeta>(), m, st), "object table");
 }
 
+// Decide whether the next `passes` passes of kernel shape v match through the cells, and build
+// those of every object whose points are new (outside any capture).  The objects of a
+// launch share it, so many small clouds cost little more than one.
+void ensure_cells(asicp_ctx *c, int v, int passes)
+{
+    c->cells_on = false;
+    if (v != kFwdVariants - 1 || c->cells_oom) return;
+    std::vector<int> todo;
+    int most = 0;
+    double pairs = 0.0, points = 0.0;
+    for (int o = 0; o < c->nobj; ++o) {
+        most = std::max(most, c->objs[o].M);
+        pairs += (double)c->objmeta_h[o].np * c->N * c->objs[o].M;
+        if (c->objs[o].cells_built) continue;
+        todo.push_back(o);
+        points += c->objs[o].M;
+    }
+    if (most < kCellMinM || most > kCellMaxM) return;
+    if (!todo.empty()) {
+        c->cells_owed += passes * pairs / kCellRate;
+        if (c->cells_owed <= 100.0 + points / kCellRatePts) return;
+    }
+    c->cells_on = true;
+    if (todo.empty()) return;
+    auto scratch = [](const CellSizes &s) { return 2 * sizeof(int) * (size_t)s.list_cap + s.rec_bytes; };
+    constexpr size_t kCtr = sizeof(int) * kCellCounters * kCellBatch;
+    size_t need = 0;
+    bool moved = false;
+    try {
+        size_t sum = 0;
+        for (size_t i = 0, first = 0; i < todo.size(); ++i) {
+            ObjBufs &b = c->objs[todo[i]];
+            const CellSizes s = cell_sizes(b.M);
+            const void *was[2] = {b.nodes.p, b.leaves.p};
+            b.nodes.ensure(sizeof(int2) * (size_t)s.node_cap, "matching cells");
+            b.leaves.ensure(sizeof(int) * (size_t)s.leaf_cap, "matching cells");
+            moved = moved || b.nodes.p != was[0] || b.leaves.p != was[1];
+            if (i > first && (sum + scratch(s) > kCellScratch || i - first == kCellBatch)) { sum = 0; first = i; }
+            sum += scratch(s);
+            need = std::max(need, sum);
+        }
+        c->cellwork.ensure(kCtr + need, "matching cells' scratch");
+    } catch (const Err &e) {
+        if (e.st != ASICP_ERR_OOM) throw;
+        c->cells_oom = true;
+        c->cells_on = false;
+        c->cellwork.release();
+        return;
+    }
+    if (moved) {
+        for (int o = 0; o < c->nobj; ++o) {
+            c->objmeta_h[o].nodes = c->objs[o].nodes.as<int2>();
+            c->objmeta_h[o].leaves = c->objs[o].leaves.as<int>();
+        }
+        ck(cudaMemcpyAsync(c->objmeta.p, c->objmeta_h.data(), sizeof(ObjMeta) * c->nobj, cudaMemcpyHostToDevice, c->st),
+           "object table");
+        ck(cudaStreamSynchronize(c->st), "object table");
+    }
+    for (size_t i = 0; i < todo.size();) {
+        CellBuildBatch batch{};
+        unsigned char *at = c->cellwork.as<unsigned char>() + kCtr, *end = c->cellwork.as<unsigned char>() + c->cellwork.bytes;
+        int n = 0;
+        for (; i < todo.size() && n < kCellBatch; ++i, ++n) {
+            ObjBufs &o = c->objs[todo[i]];
+            const CellSizes s = cell_sizes(o.M);
+            if (n > 0 && (size_t)(end - at) < scratch(s)) break;
+            CellBuild &b = batch.b[n];
+            b.R = o.R.as<float4>();
+            b.frame = c->frame.as<float4>() + todo[i];
+            b.nodes = o.nodes.as<int2>();
+            b.leaves = o.leaves.as<int>();
+            b.recs = at;
+            b.lists = reinterpret_cast<int *>(at + s.rec_bytes);
+            b.ctr = c->cellwork.as<int>() + kCellCounters * n;
+            b.M = o.M;
+            b.leaf_cap = s.leaf_cap; b.list_cap = s.list_cap; b.cell_cap = s.cell_cap; b.node_cap = s.node_cap;
+            at += scratch(s);
+        }
+        ck(cudaMemsetAsync(c->cellwork.p, 0, kCtr, c->st), "matching cells");
+        ck(launch_cells_build(batch, n, c->st), "matching cells");
+    }
+    for (int o : todo) c->objs[o].cells_built = true;
+}
+
 void iterate(asicp_ctx *c, int mode, float gamma, int k)
 {
     select_minibatch(c, k);
@@ -456,13 +557,15 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
     fa.nn_idx = c->nnidx.as<int>();
     fa.cand = c->tccand.as<int4>();
     fa.variant = c->fwd_variant;
+    fa.Ssort = c->Ssort.as<float4>();
+    fa.cells = c->cells_on;
     fa.expire_test = c->expire_test ? 1 : 0;
     if (c->cfg.debug) {
         fa.dbg_d2 = c->dbg_d2.as<float>();
         fa.dbg_sp = c->dbg_sp.as<float>();
     }
     timed(c, kTimeMatch, [&](cudaStream_t st) { return launch_fwd_match(fa, st); }, "forward matching kernel");
-    if (fwd_has_exact_kernel(fa.variant))
+    if (fwd_has_exact_kernel(fa))
         timed(c, kTimeExact, [&](cudaStream_t st) { return launch_fwd_exact(fa, st); }, "exact choice kernel");
 
     CollideArgs ca{};
@@ -548,7 +651,8 @@ std::vector<const void *> loop_key(const asicp_ctx *c)
             reinterpret_cast<const void *>((size_t)c->mb_version), reinterpret_cast<const void *>((size_t)c->T),
             reinterpret_cast<const void *>((size_t)c->G), reinterpret_cast<const void *>((size_t)c->n_items),
             reinterpret_cast<const void *>((size_t)c->N), reinterpret_cast<const void *>((size_t)c->fwd_variant),
-            reinterpret_cast<const void *>((size_t)c->expire_test)};
+            reinterpret_cast<const void *>((size_t)c->expire_test), c->Ssort.p,
+            reinterpret_cast<const void *>((size_t)c->cells_on)};
 }
 
 // Replay the captured loop on the caller's stream, capturing it first when the
@@ -645,12 +749,15 @@ void autotune_impl(asicp_ctx *c, float *ms_out)
         fa.nn_idx = c->nnidx.as<int>();
         fa.cand = c->tccand.as<int4>();
         fa.variant = v;
+        ensure_cells(c, v, c->cfg.k_max + 1);
+        fa.Ssort = c->Ssort.as<float4>();
+        fa.cells = c->cells_on;
         ck(launch_fwd_match(fa, c->st), "autotune warm-up");
-        if (fwd_has_exact_kernel(v)) ck(launch_fwd_exact(fa, c->st), "autotune warm-up");
+        if (fwd_has_exact_kernel(fa)) ck(launch_fwd_exact(fa, c->st), "autotune warm-up");
         ck(cudaEventRecord(e0, c->st), "cudaEventRecord");
         for (int r = 0; r < reps; ++r) {
             ck(launch_fwd_match(fa, c->st), "autotune launch");
-            if (fwd_has_exact_kernel(v)) ck(launch_fwd_exact(fa, c->st), "autotune launch");
+            if (fwd_has_exact_kernel(fa)) ck(launch_fwd_exact(fa, c->st), "autotune launch");
         }
         ck(cudaEventRecord(e1, c->st), "cudaEventRecord");
         ck(cudaEventSynchronize(e1), "cudaEventSynchronize");
@@ -684,6 +791,8 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
     const void *was[4] = {b.R.p, b.Rx.p, b.Rt.p, b.C.p};
     const int was_M = b.M, was_Mc = b.Mc, was_Mpad = b.Mpad;
     b.set = false;
+    b.cells_built = false;
+    ctx->cells_owed = 0.0;
     ctx->run_done = false;
     ctx->stage.ensure(sizeof(float) * 3 * (size_t)(M > mc ? M : mc), "staging");
     b.R.ensure(sizeof(float4) * M, "object cloud");
@@ -779,6 +888,7 @@ asicp_status asicp_create(const asicp_config *cfg, asicp_ctx **out)
         fwd_grid_size();
         ck(init_collision_attributes(), "collision kernel attributes");
         ck(init_update_attributes(), "update kernel attributes");
+        ck(init_cells_attributes(), "cell kernel attributes");
         c->com.ensure(sizeof(double) * 3 * c->nobj, "com");
         c->frame.ensure(sizeof(float4) * c->nobj, "screening frames");
         c->pconst.ensure(sizeof(double) * 12 * cfg->P, "pconst");
@@ -891,6 +1001,8 @@ asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_
         ck(cudaMemcpyAsync(ctx->stage.p, S_xyz, sizeof(float) * 3 * (size_t)N, cudaMemcpyDefault, ctx->st), "copy S");
         float4 *Sp = ctx->S.as<float4>() + (size_t)preshape * N;
         ck(launch_pack_points(ctx->stage.as<float>(), N, Sp, ctx->errw.as<int>(), ctx->st), "pack S");
+        ctx->Ssort.ensure(sizeof(float4) * (size_t)ctx->cfg.P * N, "gripper clouds, sorted");
+        ck(launch_sort_points(Sp, N, ctx->Ssort.as<float4>() + (size_t)preshape * N, ctx->st), "sort S");
         ck(launch_preshape_consts(Sp, N, ctx->pconst.as<double>() + 12 * preshape, ctx->st), "preshape sums");
         const size_t nv = (size_t)nx * ny * nz;
         ctx->grids[preshape].ensure(sizeof(float) * nv, "sdf grid");
@@ -972,6 +1084,7 @@ asicp_status asicp_step(asicp_ctx *ctx, int k)
         if (!ctx->inputs_ready() || !ctx->theta_set) fail(ASICP_ERR_STATE, "step: inputs and poses must be set first");
         if (ctx->layout_dirty) fail(ASICP_ERR_STATE, "step: inputs changed since the poses were set");
         if (k < 0 || k >= ctx->cfg.k_max) fail(ASICP_ERR_INVALID_ARG, "step: k out of [0, k_max)");
+        ensure_cells(ctx, ctx->fwd_variant, 1);
         step_impl(ctx, k);
         ctx->run_done = false;
     });
@@ -997,6 +1110,7 @@ asicp_status asicp_run(asicp_ctx *ctx, const float *theta0)
         }
         ctx->theta_set = true;
         if (ctx->cfg.autotune && !ctx->tuned) autotune_impl(ctx, nullptr);
+        ensure_cells(ctx, ctx->fwd_variant, ctx->cfg.k_max + 1);
         run_loop_graph(ctx);
         ctx->k_next = ctx->cfg.k_max;
         ctx->stepped = true;

@@ -198,6 +198,8 @@ struct ObjMeta {
     const float4 *R;          // [M] object points
     const ulonglong2 *Rx;     // [Mpad] screening layout (pairs of (-2r, |r|^2)), Mpad = whole tiles
     const float *Rt;          // [Mpad / 128] augmented tiles of the tensor-core kernel (8 KB each)
+    const int2 *nodes;        // matching cells (k_cells.cu): tables and nodes, and the
+    const int *leaves;        // points that can be nearest per cell; null where not built
     const float4 *C;          // [Mc] collision points (may alias R)
     int M, Mpad, Mc, chunks;  // chunks = ceil(Mc / kColChunk)
     int pfirst, np;           // first particle and number of particles of this object
@@ -225,6 +227,7 @@ struct FwdItem {
 struct FwdArgs {
     Layout L;
     const float4 *S;         // [P][N] gripper points (gripper frame)
+    const float4 *Ssort;     // [P][N] the same along a space-filling curve, w = own index (cells only)
     const float *theta;      // [T][8]
     const FwdItem *items;    // [n_items] work items (null: object 0, consecutive 1024-query items)
     const int *cta_off;      // [grid + 1]: CTA b runs items cta_off[b] .. cta_off[b+1]-1 (null: round-robin)
@@ -235,6 +238,7 @@ struct FwdArgs {
     float *dbg_sp;           // [T][N][3] or null
     int4 *cand;              // [T][N] tensor-core shape only: candidate chunks per query
     int variant;             // kernel shape (0 .. kFwdVariants - 1), chosen by the autotuner
+    int cells;               // tensor-core shape only: match through the objects' cells instead
     int expire_test;         // float32 shapes: the first copy wait of a CTA waits on an mbarrier
                              // that nothing arrives at, for kTestWaitCycles (tests the timeout path)
 };
@@ -243,7 +247,7 @@ constexpr int kFwdVariants = 8;        // kernel shapes of the forward matching 
 cudaError_t launch_fwd_match(const FwdArgs &a, cudaStream_t st);
 // The tensor-core shape leaves the exact choice to a second kernel (launch it after
 // launch_fwd_match on the same stream); the float32 shapes make it themselves.
-inline bool fwd_has_exact_kernel(int v) { return v == kFwdVariants - 1; }
+inline bool fwd_has_exact_kernel(const FwdArgs &a) { return a.variant == kFwdVariants - 1 && !a.cells; }
 cudaError_t launch_fwd_exact(const FwdArgs &a, cudaStream_t st);
 int fwd_grid_size();                   // first call sets the kernels' attributes
 int fwd_shape_grid(int v);             // CTAs of kernel shape v (a whole number per SM)
@@ -263,6 +267,33 @@ cudaError_t launch_fwd_match_tc(const FwdArgs &a, cudaStream_t st);
 cudaError_t launch_tc_exact(const FwdArgs &a, cudaStream_t st);
 int fwd_tc_grid();
 int fwd_tc_threads();
+
+// Matching cells (k_cells.cu).  One object's build: its points and frame, the tables it
+// leaves behind (nodes, leaves) and the scratch of the build (lists and records of two
+// levels in turn, counters cleared by the caller).
+constexpr int kCellCounters = 64;      // ints per object
+constexpr int kCellBatch = 32;         // objects per launch
+struct CellBuild {
+    const float4 *R;
+    const float4 *frame;
+    int2 *nodes;
+    int *leaves, *lists;
+    void *recs;
+    int *ctr;
+    int M, leaf_cap, list_cap, cell_cap, node_cap;
+};
+struct CellBuildBatch {
+    CellBuild b[kCellBatch];
+};
+struct CellSizes {
+    int leaf_cap, list_cap, cell_cap, node_cap;   // ints, ints per level, records per level, nodes
+    size_t rec_bytes;                             // records of both levels
+};
+CellSizes cell_sizes(int M);
+cudaError_t launch_cells_build(const CellBuildBatch &batch, int n, cudaStream_t st);
+cudaError_t launch_cells_match(const FwdArgs &a, cudaStream_t st);
+cudaError_t launch_sort_points(const float4 *S, int N, float4 *out, cudaStream_t st);
+cudaError_t init_cells_attributes();
 
 constexpr int kColChunk = 64;          // colliding points per reverse-matching work item
 

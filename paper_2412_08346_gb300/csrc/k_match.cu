@@ -367,7 +367,7 @@ const char *fwd_variant_name(int v)
 
 cudaError_t launch_fwd_match(const FwdArgs &a, cudaStream_t st)
 {
-    if (a.variant == kTcVariant) return launch_fwd_match_tc(a, st);
+    if (a.variant == kTcVariant) return a.cells ? launch_cells_match(a, st) : launch_fwd_match_tc(a, st);
     return with_shape(a.variant, [&](auto sh) { return launch_shape<decltype(sh)>(a, st); });
 }
 

@@ -1,0 +1,83 @@
+"""Matching through the objects' cells (the tensor-core shape on clouds of 1024 points and more)
+against the float32 kernel and the FP64 nearest neighbour, on clouds where a cell's list is hard to
+keep short (exact planes, a sphere seen from its centre, duplicates), at the smallest size that uses
+cells and one below, and on queries near, far and beyond the outermost cells."""
+import numpy as np
+import pytest
+
+import asicp_testlib as tl
+from paper_2412_08346_gb300 import asicp, synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+
+def _cloud(kind, M):
+    g = np.random.default_rng(M)
+    if kind == "plane":
+        R = np.concatenate([g.uniform(-0.05, 0.05, (M, 2)), np.zeros((M, 1))], 1)
+    elif kind == "grid":
+        R = np.stack(np.meshgrid(*[np.arange(int(np.ceil(M ** (1 / 3)))) * 0.004] * 3), -1).reshape(-1, 3)[:M]
+    elif kind == "sphere":
+        R = g.normal(size=(M, 3))
+        R *= 0.05 / np.linalg.norm(R, axis=1, keepdims=True)
+    elif kind == "duplicates":
+        R = g.uniform(-0.05, 0.05, (64, 3))[g.integers(0, 64, M)]
+    elif kind == "shifted":
+        R = synth.partial_object(M, 5).points + np.float32([3.0, -2.0, 8.0])
+    else:
+        R = synth.partial_object(M, 7).points
+    return np.ascontiguousarray(R, dtype=np.float32)
+
+
+def _indices(R, S, theta, P, shape):
+    N = S.shape[1]
+    cfg = asicp.asicp_config_default(P=P, K=len(theta) // P, k_max=2, k_stein=0, conv_tol=-1.0, debug=1, fwd_shape=shape,
+                                     cuda_stream=torch.cuda.current_stream().cuda_stream)
+    ctx = asicp.asicp_create(cfg)
+    try:
+        asicp.asicp_set_object(ctx, R)
+        for p in range(P):
+            asicp.asicp_set_gripper_sdf(ctx, p, S[p], -np.ones((8, 8, 8), np.float32), np.full(3, -0.1, np.float32),
+                                        np.float32(0.2 / 7))
+        for _ in range(100 if shape else 1):         # the build waits until the steps would have paid for it
+            asicp.asicp_set_state(ctx, theta, 0)
+            asicp.asicp_step(ctx, 0)
+        return tl.read_state(ctx, P, len(theta) // P, N, len(R))
+    finally:
+        asicp.asicp_destroy(ctx)
+
+
+@pytest.mark.parametrize("kind,M", [("partial", 1023), ("partial", 1024), ("partial", 9001), ("shifted", 4099),
+                                    ("plane", 2000), ("grid", 1728), ("sphere", 1500), ("duplicates", 1100)])
+def test_cells_find_the_nearest_points(kind, M):
+    R = _cloud(kind, M)
+    g = np.random.default_rng(3)
+    P, N, K = 2, 203, 64
+    S = g.uniform(-0.05, 0.05, (P, N, 3)).astype(np.float32)
+    S[:, :40] = R[g.integers(0, M, (P, 40))] - R.mean(0)       # on object points (when the pose is the identity)
+    S[:, 40] = 0.0
+    c = (R.max(0) + R.min(0)) / 2
+    t = np.stack([R.mean(0), c, c + [0.1, 0, 0], c - [0, 0.3, 0.1], c + [0, 0, 1.5], c + [4, 4, -4], c - [9, 0, 30],
+                  c + [0.02, 0.03, -0.01]])
+    t = np.tile(t, (K // 8, 1))
+    q = g.normal(size=(K, 4))
+    q[::8] = q[1::8] = [1, 0, 0, 0]
+    theta = np.tile(np.concatenate([t, q / np.linalg.norm(q, axis=1, keepdims=True)], 1), (P, 1)).astype(np.float32)
+    a, b = (_indices(R, S, theta, P, v) for v in (0, asicp.FWD_SHAPES - 1))
+    assert np.array_equal(a["s_prime"], b["s_prime"])
+    tl.check_nn(b["s_prime"].reshape(-1, 3), R, b["nn_idx"].reshape(-1), {})
+    d = b["s_prime"].astype(np.float64) - R[b["nn_idx"]]
+    assert np.allclose(b["nn_d2"], (d ** 2).sum(-1), rtol=1e-6, atol=0)
+    # the cells give the lowest index of the smallest float32 distance over the whole cloud; the float32
+    # kernel the same, but for points whose distances differ by less than their rounding
+    for pk in range(P * K):
+        diff = np.nonzero(a["nn_idx"][pk] != b["nn_idx"][pk])[0]
+        assert np.all(b["nn_d2"][pk][diff] <= a["nn_d2"][pk][diff])
+        tie = diff[b["nn_d2"][pk][diff] == a["nn_d2"][pk][diff]]
+        assert np.all(b["nn_idx"][pk][tie] < a["nn_idx"][pk][tie])
+        if np.abs(t[pk % K] - c).max() < 1.0:
+            assert len(diff) == 0
