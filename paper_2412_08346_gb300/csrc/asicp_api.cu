@@ -118,6 +118,9 @@ struct asicp_ctx {
     bool cells_oom = false;           // no room for matching cells: the screening is used
     bool cells_on = false;            // the passes being launched match through the cells
     double cells_owed = 0.0;          // microseconds of screening on the present objects so far
+    bool pre_oom = false;             // no room for the gripper clouds' cells
+    bool pre_built = false;           // the gripper clouds' cells are built (all preshapes together)
+    double pre_owed = 0.0;            // microseconds of reverse matching without them so far
     bool expire_test = false;         // the float32 matching kernels' first copy waits expire (testing)
 
     // layout (rebuilt when objects, particle counts or N change)
@@ -127,7 +130,7 @@ struct asicp_ctx {
     std::vector<int> grp_off_h;
     std::vector<ObjMeta> objmeta_h;
 
-    DevMem partgrp, grpoff, objmeta, items, ctaoff, com, frame, colitems, collist, box, stage, S, Ssort, cellwork, pconst, dmeta, theta, fsums,
+    DevMem partgrp, grpoff, objmeta, items, ctaoff, com, frame, colitems, collist, box, stage, S, Ssort, preframe, prenodes, preleaves, cellwork, pconst, dmeta, theta, fsums,
         csums, ncol, colidx, cost, grad, prev, frozen, phi, h, order, errw, out7, outc, outi, nnidx, tccand, dbg_d2, dbg_sp,
         dbg_colnn;
 
@@ -458,6 +461,46 @@ void select_minibatch(asicp_ctx *c, int k)
     ck(launch_store_meta(c->objmeta.as<ObjMeta>(), m, st), "object table");
 }
 
+// Build the cells of the given clouds (at most kCellBatch of them, or as many as the scratch
+// holds, per launch).
+size_t cell_scratch(const CellSizes &s) { return 2 * sizeof(int) * (size_t)s.list_cap + s.rec_bytes; }
+constexpr size_t kCellCtrBytes = sizeof(int) * kCellCounters * kCellBatch;
+
+void ensure_cell_scratch(asicp_ctx *c, const std::vector<CellBuild> &todo)
+{
+    size_t need = 0, sum = 0;
+    for (size_t i = 0, first = 0; i < todo.size(); ++i) {
+        const size_t w = cell_scratch(cell_sizes(todo[i].M));
+        if (i > first && (sum + w > kCellScratch || i - first == kCellBatch)) { sum = 0; first = i; }
+        sum += w;
+        need = std::max(need, sum);
+    }
+    c->cellwork.ensure(kCellCtrBytes + need, "matching cells' scratch");
+}
+
+void build_cells(asicp_ctx *c, const std::vector<CellBuild> &todo)
+{
+    for (size_t i = 0; i < todo.size();) {
+        CellBuildBatch batch{};
+        unsigned char *at = c->cellwork.as<unsigned char>() + kCellCtrBytes,
+                      *end = c->cellwork.as<unsigned char>() + c->cellwork.bytes;
+        int n = 0;
+        for (; i < todo.size() && n < kCellBatch; ++i, ++n) {
+            const CellSizes s = cell_sizes(todo[i].M);
+            if (n > 0 && (size_t)(end - at) < cell_scratch(s)) break;
+            CellBuild &b = batch.b[n];
+            b = todo[i];
+            b.recs = at;
+            b.lists = reinterpret_cast<int *>(at + s.rec_bytes);
+            b.ctr = c->cellwork.as<int>() + kCellCounters * n;
+            b.leaf_cap = s.leaf_cap; b.list_cap = s.list_cap; b.cell_cap = s.cell_cap; b.node_cap = s.node_cap;
+            at += cell_scratch(s);
+        }
+        ck(cudaMemsetAsync(c->cellwork.p, 0, kCellCtrBytes, c->st), "matching cells");
+        ck(launch_cells_build(batch, n, c->st), "matching cells");
+    }
+}
+
 // Decide whether the next `passes` passes of kernel shape v match through the cells, and build
 // those of every object whose points are new (outside any capture).  The objects of a
 // launch share it, so many small clouds cost little more than one.
@@ -482,30 +525,31 @@ void ensure_cells(asicp_ctx *c, int v, int passes)
     }
     c->cells_on = true;
     if (todo.empty()) return;
-    auto scratch = [](const CellSizes &s) { return 2 * sizeof(int) * (size_t)s.list_cap + s.rec_bytes; };
-    constexpr size_t kCtr = sizeof(int) * kCellCounters * kCellBatch;
-    size_t need = 0;
+    std::vector<CellBuild> builds;
     bool moved = false;
     try {
-        size_t sum = 0;
-        for (size_t i = 0, first = 0; i < todo.size(); ++i) {
-            ObjBufs &b = c->objs[todo[i]];
-            const CellSizes s = cell_sizes(b.M);
-            const void *was[2] = {b.nodes.p, b.leaves.p};
-            b.nodes.ensure(sizeof(int2) * (size_t)s.node_cap, "matching cells");
-            b.leaves.ensure(sizeof(int) * (size_t)s.leaf_cap, "matching cells");
-            moved = moved || b.nodes.p != was[0] || b.leaves.p != was[1];
-            if (i > first && (sum + scratch(s) > kCellScratch || i - first == kCellBatch)) { sum = 0; first = i; }
-            sum += scratch(s);
-            need = std::max(need, sum);
+        for (int i : todo) {
+            ObjBufs &o = c->objs[i];
+            const CellSizes s = cell_sizes(o.M);
+            const void *was[2] = {o.nodes.p, o.leaves.p};
+            o.nodes.ensure(sizeof(int2) * (size_t)s.node_cap, "matching cells");
+            o.leaves.ensure(sizeof(int) * (size_t)s.leaf_cap, "matching cells");
+            moved = moved || o.nodes.p != was[0] || o.leaves.p != was[1];
+            CellBuild b{};
+            b.R = o.R.as<float4>();
+            b.frame = c->frame.as<float4>() + i;
+            b.nodes = o.nodes.as<int2>();
+            b.leaves = o.leaves.as<int>();
+            b.M = o.M;
+            b.factor = kObjectCells;
+            builds.push_back(b);
         }
-        c->cellwork.ensure(kCtr + need, "matching cells' scratch");
+        ensure_cell_scratch(c, builds);
     } catch (const Err &e) {
         if (e.st != ASICP_ERR_OOM) throw;
         c->cells_oom = true;
         c->cells_on = false;
         c->cellwork.release();
-        return;
     }
     if (moved) {
         for (int o = 0; o < c->nobj; ++o) {
@@ -516,30 +560,53 @@ void ensure_cells(asicp_ctx *c, int v, int passes)
            "object table");
         ck(cudaStreamSynchronize(c->st), "object table");
     }
-    for (size_t i = 0; i < todo.size();) {
-        CellBuildBatch batch{};
-        unsigned char *at = c->cellwork.as<unsigned char>() + kCtr, *end = c->cellwork.as<unsigned char>() + c->cellwork.bytes;
-        int n = 0;
-        for (; i < todo.size() && n < kCellBatch; ++i, ++n) {
-            ObjBufs &o = c->objs[todo[i]];
-            const CellSizes s = cell_sizes(o.M);
-            if (n > 0 && (size_t)(end - at) < scratch(s)) break;
-            CellBuild &b = batch.b[n];
-            b.R = o.R.as<float4>();
-            b.frame = c->frame.as<float4>() + todo[i];
-            b.nodes = o.nodes.as<int2>();
-            b.leaves = o.leaves.as<int>();
-            b.recs = at;
-            b.lists = reinterpret_cast<int *>(at + s.rec_bytes);
-            b.ctr = c->cellwork.as<int>() + kCellCounters * n;
-            b.M = o.M;
-            b.leaf_cap = s.leaf_cap; b.list_cap = s.list_cap; b.cell_cap = s.cell_cap; b.node_cap = s.node_cap;
-            at += scratch(s);
-        }
-        ck(cudaMemsetAsync(c->cellwork.p, 0, kCtr, c->st), "matching cells");
-        ck(launch_cells_build(batch, n, c->st), "matching cells");
-    }
+    if (!c->cells_on) return;
+    build_cells(c, builds);
     for (int o : todo) c->objs[o].cells_built = true;
+}
+
+// Decide whether the reverse matching of the next `passes` passes goes through the cells of the
+// gripper clouds, and build those (all preshapes together) once the passes so far and to
+// come would take longer without them: a pass of collide_nn_kernel takes 5 us more than
+// one through the cells, and 1 us per kPreRate pairs, a colliding point in 32 assumed.
+constexpr int kPreMinN = 512;
+constexpr double kPreRate = 5.7e6;
+
+void ensure_pre_cells(asicp_ctx *c, int passes)
+{
+    if (c->pre_built || c->pre_oom || c->N < kPreMinN) return;
+    double tests = 0.0;
+    for (const ObjMeta &m : c->objmeta_h) tests += (double)m.np * m.Mc;
+    c->pre_owed += passes * (5.0 + tests / 32.0 * c->N / kPreRate);
+    const int P = c->cfg.P;
+    if (c->pre_owed <= 150.0 + (double)P * c->N / kCellRatePts) return;
+    std::vector<CellBuild> builds;
+    const CellSizes s = cell_sizes(c->N);
+    try {
+        c->prenodes.ensure(sizeof(int2) * (size_t)s.node_cap * P, "gripper cells");
+        c->preleaves.ensure(sizeof(int) * (size_t)s.leaf_cap * P, "gripper cells");
+        for (int p = 0; p < P; ++p) {
+            CellBuild b{};
+            b.R = c->S.as<float4>() + (size_t)p * c->N;
+            b.frame = c->preframe.as<float4>() + p;
+            b.nodes = c->prenodes.as<int2>() + (size_t)p * s.node_cap;
+            b.leaves = c->preleaves.as<int>() + (size_t)p * s.leaf_cap;
+            b.M = c->N;
+            b.factor = kGripperCells;
+            b.tol = kGripperTol;
+            b.near_only = 1;
+            builds.push_back(b);
+        }
+        ensure_cell_scratch(c, builds);
+    } catch (const Err &e) {
+        if (e.st != ASICP_ERR_OOM) throw;
+        c->pre_oom = true;
+        c->prenodes.release();
+        c->preleaves.release();
+        return;
+    }
+    build_cells(c, builds);
+    c->pre_built = true;
 }
 
 void iterate(asicp_ctx *c, int mode, float gamma, int k)
@@ -582,6 +649,16 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
     ca.col_list = c->collist.as<int>();
     ca.err = c->errw.as<int>();
     if (c->cfg.debug) ca.dbg_colnn = c->dbg_colnn.as<int>();
+    ca.cells = c->pre_built;
+    if (ca.cells) {
+        const CellSizes s = cell_sizes(c->N);
+        ca.pre_nodes = c->prenodes.as<int2>();
+        ca.pre_leaves = c->preleaves.as<int>();
+        ca.pre_frame = c->preframe.as<float4>();
+        ca.pre_node_cap = s.node_cap;
+        ca.pre_leaf_cap = s.leaf_cap;
+        ca.most_items = (int)std::min<long long>(std::max<long long>(1, c->csum_total), INT_MAX);
+    }
     timed(c, kTimeCollide, [&](cudaStream_t st) { return launch_collide(ca, st); }, "collision kernel");
     timed(c, kTimeCollideNN, [&](cudaStream_t st) { return launch_collide_nn(ca, st); }, "collision matching kernel");
 
@@ -652,7 +729,8 @@ std::vector<const void *> loop_key(const asicp_ctx *c)
             reinterpret_cast<const void *>((size_t)c->G), reinterpret_cast<const void *>((size_t)c->n_items),
             reinterpret_cast<const void *>((size_t)c->N), reinterpret_cast<const void *>((size_t)c->fwd_variant),
             reinterpret_cast<const void *>((size_t)c->expire_test), c->Ssort.p,
-            reinterpret_cast<const void *>((size_t)c->cells_on)};
+            reinterpret_cast<const void *>((size_t)c->cells_on), c->prenodes.p, c->preleaves.p, c->preframe.p,
+            reinterpret_cast<const void *>((size_t)c->pre_built), reinterpret_cast<const void *>((size_t)c->csum_total)};
 }
 
 // Replay the captured loop on the caller's stream, capturing it first when the
@@ -1002,7 +1080,11 @@ asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_
         float4 *Sp = ctx->S.as<float4>() + (size_t)preshape * N;
         ck(launch_pack_points(ctx->stage.as<float>(), N, Sp, ctx->errw.as<int>(), ctx->st), "pack S");
         ctx->Ssort.ensure(sizeof(float4) * (size_t)ctx->cfg.P * N, "gripper clouds, sorted");
-        ck(launch_sort_points(Sp, N, ctx->Ssort.as<float4>() + (size_t)preshape * N, ctx->st), "sort S");
+        ctx->preframe.ensure(sizeof(float4) * ctx->cfg.P, "gripper frames");
+        ck(launch_sort_points(Sp, N, ctx->Ssort.as<float4>() + (size_t)preshape * N, ctx->preframe.as<float4>() + preshape,
+                              ctx->st), "sort S");
+        ctx->pre_built = false;
+        ctx->pre_owed = 0.0;
         ck(launch_preshape_consts(Sp, N, ctx->pconst.as<double>() + 12 * preshape, ctx->st), "preshape sums");
         const size_t nv = (size_t)nx * ny * nz;
         ctx->grids[preshape].ensure(sizeof(float) * nv, "sdf grid");
@@ -1085,6 +1167,7 @@ asicp_status asicp_step(asicp_ctx *ctx, int k)
         if (ctx->layout_dirty) fail(ASICP_ERR_STATE, "step: inputs changed since the poses were set");
         if (k < 0 || k >= ctx->cfg.k_max) fail(ASICP_ERR_INVALID_ARG, "step: k out of [0, k_max)");
         ensure_cells(ctx, ctx->fwd_variant, 1);
+        ensure_pre_cells(ctx, 1);
         step_impl(ctx, k);
         ctx->run_done = false;
     });
@@ -1111,6 +1194,7 @@ asicp_status asicp_run(asicp_ctx *ctx, const float *theta0)
         ctx->theta_set = true;
         if (ctx->cfg.autotune && !ctx->tuned) autotune_impl(ctx, nullptr);
         ensure_cells(ctx, ctx->fwd_variant, ctx->cfg.k_max + 1);
+        ensure_pre_cells(ctx, ctx->cfg.k_max + 1);
         run_loop_graph(ctx);
         ctx->k_next = ctx->cfg.k_max;
         ctx->stepped = true;

@@ -281,7 +281,13 @@ struct CellBuild {
     void *recs;
     int *ctr;
     int M, leaf_cap, list_cap, cell_cap, node_cap;
+    float factor;             // near cells reach this many times the power of two above the radius
+    float tol;                // positions looked up may be off by 0.4 tol times the radius
+    int near_only;            // no cells beyond the near ones
 };
+// Cells of objects, and of gripper clouds in the gripper frame (colliding points lie in the
+// gripper's body, not far from its surface; see collide_cells_kernel for the tolerance).
+constexpr float kObjectCells = 4.f, kGripperCells = 2.f, kGripperTol = 1.25e-4f;
 struct CellBuildBatch {
     CellBuild b[kCellBatch];
 };
@@ -292,7 +298,7 @@ struct CellSizes {
 CellSizes cell_sizes(int M);
 cudaError_t launch_cells_build(const CellBuildBatch &batch, int n, cudaStream_t st);
 cudaError_t launch_cells_match(const FwdArgs &a, cudaStream_t st);
-cudaError_t launch_sort_points(const float4 *S, int N, float4 *out, cudaStream_t st);
+cudaError_t launch_sort_points(const float4 *S, int N, float4 *out, float4 *frame, cudaStream_t st);
 cudaError_t init_cells_attributes();
 
 constexpr int kColChunk = 64;          // colliding points per reverse-matching work item
@@ -308,6 +314,12 @@ struct CollideArgs {
     double *fsums;            // [T][kFwdSums]
     double *csums;            // chunk sums (see ObjMeta::csum_base) [.][kColSums]
     int *dbg_colnn;           // like colidx, or null
+    int cells;                // reverse matching through the gripper clouds' cells
+    const int2 *pre_nodes;    // [P][pre_node_cap]
+    const int *pre_leaves;    // [P][pre_leaf_cap]
+    const float4 *pre_frame;  // [P]
+    int pre_node_cap, pre_leaf_cap;
+    int most_items;           // work-list entries at most
     int *col_items;           // (count, next) of the reverse-matching work list
     int *col_list;            // [2 * items] (particle, chunk) pairs
     const int *err;           // error word: a kernel of the pass found an error, skip the work

@@ -41,7 +41,7 @@
 // (table, two or three nodes, list, points), all from L2 and L1; queries in the gripper
 // cloud's own order take 68 us.  The build (ten rounds of few and uneven cells, latency again)
 // takes 0.10 ms at 1024 points, 0.27 at 8192, 1.4 at 65536.
-#include "asicp_internal.cuh"
+#include "cells.cuh"
 
 namespace asicp {
 
@@ -49,10 +49,8 @@ namespace {
 
 constexpr int kLeaf = 12;                  // a list of at most this many points is not halved
 constexpr int kNearLevels = 9, kFarLevels = 5;   // halvings at most (near cells: h = J / 4096 at the end)
-constexpr int kTable = 32;                 // near table: kTable^3 cells
 constexpr int kStartNear = 8;              // the near grid the lists start from
-constexpr int kShells = 6;
-constexpr int kFarBase = kTable * kTable * kTable;
+constexpr int kTable = kCellTable, kShells = kCellShells, kFarBase = kCellFarBase;
 constexpr int kFixedNodes = kFarBase + kShells * 64;
 constexpr int kStartCells = kStartNear * kStartNear * kStartNear + kShells * 64;
 constexpr int kStaged = 512;               // parent lists up to this length are staged in shared memory
@@ -60,20 +58,13 @@ constexpr int kBatch = 4;                  // points per lane and round
 constexpr int kMaskPts = 4096;             // points per warp whose verdicts are kept between the two passes
 constexpr int kStartMask = 256;            // words of a warp's mask in the start kernel (65536 points)
 constexpr int kIterBits = 10;              // see nearest9
-constexpr int kSubBits = 10;               // cell coordinates below a table or shell cell
-enum { kInner = -1, kWhole = -2 };         // node.y: children at node.x .. + 7 / the whole cloud; else list length
+static_assert(kNearLevels - 2 <= kCellSubBits && kFarLevels <= kCellSubBits, "cell coordinates");
+constexpr int kInner = kCellInner, kWhole = kCellWhole;
 constexpr int kRounds = kNearLevels + 1;   // rounds of the build: the start lists' second pass, then the halvings
 // counters: leaf entries, nodes, and per round the cells with short lists (recorded from the
 // front of the round's records), with long ones (from the back) and the list entries
 enum { kCtrLeaf = 0, kCtrNode = 1, kCtrShort = 2, kCtrLong = kCtrShort + kRounds, kCtrList = kCtrLong + kRounds };
 static_assert(kCtrList + kRounds <= kCellCounters, "counters");
-
-__device__ __forceinline__ float near_half(float B)      // J
-{
-    int ex;
-    frexpf(fmaxf(B, 1e-30f), &ex);
-    return ldexpf(4.f, ex);
-}
 
 __device__ __forceinline__ float sqrt_about(float x)
 {
@@ -83,11 +74,12 @@ __device__ __forceinline__ float sqrt_about(float x)
 }
 
 // The rounding bound above, doubled and split into the part of the point and the part of the
-// point it is held against: p is dropped when need(p) > 2 h |p - p'|_1 + have(p').
-__device__ __forceinline__ float need_of(float d, float B) { return d - 2e-6f * d - 5e-7f * B * sqrt_about(d); }
-__device__ __forceinline__ float have_of(float d, float h, float B)
+// point it is held against: p is dropped when need(p) > 2 h |p - p'|_1 + have(p').  k is
+// 5e-7 B, more where positions are less exact (CellBuild::tol).
+__device__ __forceinline__ float need_of(float d, float k) { return d - 2e-6f * d - k * sqrt_about(d); }
+__device__ __forceinline__ float have_of(float d, float h, float k)
 {
-    return d + 2e-6f * d + 5e-7f * B * (sqrt_about(d) + 4.f * h) + 8e-6f * h * h;
+    return d + 2e-6f * d + k * (sqrt_about(d) + 4.f * h) + 8e-6f * h * h;
 }
 
 // q = (p', have(p')): whether p cannot be nearest anywhere in the cell (h2: twice its widened
@@ -190,7 +182,7 @@ __global__ void __launch_bounds__(256) cells_start_kernel(const CellBuildBatch b
     __shared__ int s_cnt[8], s_leaf, s_base;
     __shared__ unsigned s_mask[8][kStartMask];
     const float4 fr = *b.frame;
-    const float B = fr.w, J = near_half(B);
+    const float J = cell_half(fr.w, b.factor), k = (5e-7f + b.tol) * fr.w;
     int cell = blockIdx.x;
     CellRef r;
     r.shell = -1;
@@ -207,7 +199,8 @@ __global__ void __launch_bounds__(256) cells_start_kernel(const CellBuildBatch b
         r.c.w = 0.25f * H;
         r.c.x = (2 * x + 1) * r.c.w - H; r.c.y = (2 * y + 1) * r.c.w - H; r.c.z = (2 * z + 1) * r.c.w - H;
         r.at = kFarBase + cell;
-        if (x % 3 != 0 && y % 3 != 0 && z % 3 != 0) {     // inside: the near grid or a smaller shell covers it
+        // inside (the near grid or a smaller shell covers it), or no far cells wanted
+        if ((x % 3 != 0 && y % 3 != 0 && z % 3 != 0) || b.near_only) {
             if (threadIdx.x == 0) b.nodes[r.at] = make_int2(0, kWhole);
             return;
         }
@@ -236,13 +229,13 @@ __global__ void __launch_bounds__(256) cells_start_kernel(const CellBuildBatch b
     float4 q;
     {
         const float d = rel((int)(unsigned)best, q.x, q.y, q.z);
-        q.w = have_of(d, c.w, B);
+        q.w = have_of(d, c.w, k);
     }
     const float h2 = 2.f * widened(c.w, r.shell, J);
     auto kept = [&](int i) {
         float x, y, z;
         const float d = rel(min(i, M - 1), x, y, z);
-        return i < hi && !dropped_by(q, x, y, z, need_of(d, B), h2);
+        return i < hi && !dropped_by(q, x, y, z, need_of(d, k), h2);
     };
     const bool masks = hi - lo <= 32 * kStartMask;
     int cnt = 0;
@@ -343,7 +336,7 @@ __device__ __forceinline__ void reduce9(const unsigned (&keys)[9], int lo, int h
 // The distinct points of the warp's lanes 0 .. 8 as the points to hold the others against, the
 // centre's first; returns their number.
 template <class P>
-__device__ __forceinline__ int make_doms(P point, int pos, float4 c, float B, float4 *dom)
+__device__ __forceinline__ int make_doms(P point, int pos, float4 c, float k, float4 *dom)
 {
     const int lane = threadIdx.x & 31;
     const unsigned same = __match_any_sync(0xffffffffu, lane < 9 ? pos : -1 - lane);
@@ -352,7 +345,7 @@ __device__ __forceinline__ int make_doms(P point, int pos, float4 c, float B, fl
     if (first) {
         float4 p = point(pos);
         const float ex = p.x - c.x, ey = p.y - c.y, ez = p.z - c.z;
-        p.w = have_of(ex * ex + ey * ey + ez * ez, c.w, B);
+        p.w = have_of(ex * ex + ey * ey + ez * ez, c.w, k);
         dom[__popc(firsts & ((1u << lane) - 1u))] = p;
     }
     __syncwarp();
@@ -362,7 +355,7 @@ __device__ __forceinline__ int make_doms(P point, int pos, float4 c, float B, fl
 // Which of the points [i0, i0 + 32 kBatch) below hi no point of dom drops: bit lane of m[j] for
 // point i0 + 32 j + lane.
 template <class P>
-__device__ __forceinline__ void keeps(P point, int i0, int hi, float4 c, const float4 *dom, int nd, float h2, float B,
+__device__ __forceinline__ void keeps(P point, int i0, int hi, float4 c, const float4 *dom, int nd, float h2, float k,
                                       unsigned (&m)[kBatch])
 {
     const int lane = threadIdx.x & 31;
@@ -372,13 +365,13 @@ __device__ __forceinline__ void keeps(P point, int i0, int hi, float4 c, const f
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
         const float ex = p[j].x - c.x, ey = p[j].y - c.y, ez = p[j].z - c.z;
-        p[j].w = need_of(ex * ex + ey * ey + ez * ez, B);
+        p[j].w = need_of(ex * ex + ey * ey + ez * ez, k);
     }
     bool out[kBatch];
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) out[j] = i0 + 32 * j + lane >= hi;
-    for (int k = 0; k < nd; ++k) {
-        const float4 q = dom[k];
+    for (int e = 0; e < nd; ++e) {
+        const float4 q = dom[e];
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) out[j] = out[j] || dropped_by(q, p[j].x, p[j].y, p[j].z, p[j].w, h2);
     }
@@ -453,7 +446,7 @@ __global__ void __launch_bounds__(256) cells_level_kernel(const CellBuildBatch b
     __shared__ int s_pos[8][9], s_cnt[8];
     __shared__ Place s_place;
     const float4 fr = *b.frame;
-    const float B = fr.w, J = near_half(B);
+    const float J = cell_half(fr.w, b.factor), k = (5e-7f + b.tol) * fr.w;
     for (int u = blockIdx.x; u < n_long * children; u += gridDim.x) {
         const CellRef r = recs(b, round)[b.cell_cap - 1 - u / children];
         if (r.len <= 0) continue;
@@ -474,13 +467,13 @@ __global__ void __launch_bounds__(256) cells_level_kernel(const CellBuildBatch b
         __syncthreads();
         for (int w = 0; w < 8; ++w)
             if (lane < 9 && s_key[w][lane] < key) { key = s_key[w][lane]; pos = s_pos[w][lane]; }
-        const int nd = make_doms(load, min(pos, r.len - 1), q.c, B, s_dom[warp]);
+        const int nd = make_doms(load, min(pos, r.len - 1), q.c, k, s_dom[warp]);
         const float h2 = 2.f * widened(q.c.w, r.shell, J);
         const bool masks = hi - lo <= kMaskPts;
         int cnt = 0;
         for (int i0 = lo; i0 < hi; i0 += 32 * kBatch) {
             unsigned m[kBatch];
-            keeps(load, i0, hi, q.c, s_dom[warp], nd, h2, B, m);
+            keeps(load, i0, hi, q.c, s_dom[warp], nd, h2, k, m);
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) {
                 if (masks && lane == 0) s_mask[warp][((i0 - lo) >> 5) + j] = m[j];
@@ -504,7 +497,7 @@ __global__ void __launch_bounds__(256) cells_level_kernel(const CellBuildBatch b
         int *out = (p.leaf ? b.leaves : lists(b, round + 1)) + p.base;
         for (int i0 = lo; i0 < hi; i0 += 32 * kBatch) {
             unsigned m[kBatch];
-            if (!masks) keeps(load, i0, hi, q.c, s_dom[warp], nd, h2, B, m);
+            if (!masks) keeps(load, i0, hi, q.c, s_dom[warp], nd, h2, k, m);
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) {
                 if (masks) m[j] = s_mask[warp][((i0 - lo) >> 5) + j];
@@ -537,12 +530,12 @@ __global__ void __launch_bounds__(256) cells_level_kernel(const CellBuildBatch b
         int pos;
         nearest9(point, 0, r.len, q.c, keys);
         reduce9(keys, 0, r.len, key, pos);
-        const int nd = make_doms(point, pos, q.c, B, s_dom[warp]);
+        const int nd = make_doms(point, pos, q.c, k, s_dom[warp]);
         const float h2 = 2.f * widened(q.c.w, r.shell, J);
         int n = 0;
         for (int i0 = 0; i0 < r.len; i0 += 32 * kBatch) {
             unsigned m[kBatch];
-            keeps(point, i0, r.len, q.c, s_dom[warp], nd, h2, B, m);
+            keeps(point, i0, r.len, q.c, s_dom[warp], nd, h2, k, m);
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) {
                 if (lane == 0) s_mask[warp][(i0 >> 5) + j] = m[j];
@@ -592,41 +585,15 @@ __global__ void __launch_bounds__(256) cells_match_kernel(const FwdArgs a)
     const float3 o = xform_f32(Rm, th[0], th[1], th[2], s.x, s.y, s.z);
     const ObjMeta &om = a.L.obj[obj];
     const float4 *__restrict__ R = om.R;
-    const int2 *__restrict__ nodes = om.nodes;
     const float4 fr = a.L.frame[obj];
 
-    // the query's cell
-    const float ax = __fsub_rn(o.x, fr.x), ay = __fsub_rn(o.y, fr.y), az = __fsub_rn(o.z, fr.z);
-    const float J = near_half(fr.w), v = fmaxf(fabsf(ax), fmaxf(fabsf(ay), fabsf(az))) * (1.f / J);
-    int2 nd = make_int2(0, kWhole);
-    if (fabsf(ax) + fabsf(ay) + fabsf(az) < __int_as_float(0x7f800000) && v < (float)(1 << kShells)) {
-        int x, y, z, at;
-        if (v < 1.f) {
-            const float k = (float)(kTable << kSubBits) / (2.f * J);
-            const int top = (kTable << kSubBits) - 1;
-            x = min(max((int)((ax + J) * k), 0), top);
-            y = min(max((int)((ay + J) * k), 0), top);
-            z = min(max((int)((az + J) * k), 0), top);
-            at = ((z >> kSubBits) * kTable + (y >> kSubBits)) * kTable + (x >> kSubBits);
-        } else {
-            const int shell = (int)(__float_as_uint(v) >> 23) - 127;
-            const float k = 1.f / ldexpf(J, shell + 1), f = (float)(2 << kSubBits);
-            const int top = (4 << kSubBits) - 1;
-            x = min(max((int)((ax * k + 1.f) * f), 0), top);
-            y = min(max((int)((ay * k + 1.f) * f), 0), top);
-            z = min(max((int)((az * k + 1.f) * f), 0), top);
-            at = kFarBase + 64 * shell + ((z >> kSubBits) * 4 + (y >> kSubBits)) * 4 + (x >> kSubBits);
-        }
-        nd = __ldg(nodes + at);
-        for (int bit = kSubBits - 1; nd.y == kInner && bit >= 0; --bit)
-            nd = __ldg(nodes + nd.x + (((x >> bit) & 1) | (((y >> bit) & 1) << 1) | (((z >> bit) & 1) << 2)));
-    }
+    const float J = cell_half(fr.w, kObjectCells);
+    const int2 nd = find_cell(om.nodes, J, __fsub_rn(o.x, fr.x), __fsub_rn(o.y, fr.y), __fsub_rn(o.z, fr.z));
 
     // its list, four points at a time
     float best = __int_as_float(0x7f800000);
     int bi = 0x7fffffff;
-    constexpr int kOwn = 128;              // longer lists are scanned by the warp together
-    if (nd.y <= kOwn) {
+    if (nd.y <= kCellOwn) {
         const int4 *l = reinterpret_cast<const int4 *>(om.leaves + nd.x);
         for (int e = 0; e < nd.y; e += 4, ++l) {
             const int4 id = __ldg(l);
@@ -640,7 +607,7 @@ __global__ void __launch_bounds__(256) cells_match_kernel(const FwdArgs a)
             if (d3 < best) { best = d3; bi = id.w; }
         }
     }
-    unsigned pending = __ballot_sync(0xffffffffu, valid && (nd.y == kWhole || nd.y > kOwn));
+    unsigned pending = __ballot_sync(0xffffffffu, valid && (nd.y == kWhole || nd.y > kCellOwn));
     while (pending) {
         const int src = __ffs(pending) - 1;
         pending &= pending - 1;
@@ -702,8 +669,9 @@ cudaError_t launch_cells_match(const FwdArgs &a, cudaStream_t st)
 }
 
 // Spatial order of a gripper cloud (one CTA): a bitonic sort of (Morton code, index) keys,
-// then the points in that order with their own index in w.
-__global__ void __launch_bounds__(1024) sort_points_kernel(const float4 *S, int N, int Npow, float4 *out)
+// then the points in that order with their own index in w.  *frame: the centre of the bounding
+// box and the largest distance from it, rounded up.
+__global__ void __launch_bounds__(1024) sort_points_kernel(const float4 *S, int N, int Npow, float4 *out, float4 *frame)
 {
     extern __shared__ unsigned long long s_key[];
     __shared__ float s_lo[3][32], s_hi[3][32];
@@ -725,6 +693,21 @@ __global__ void __launch_bounds__(1024) sort_points_kernel(const float4 *S, int 
     __syncthreads();
     for (int k = 0; k < 3; ++k)
         for (int w = 0; w < 32; ++w) { lo[k] = fminf(lo[k], s_lo[k][w]); hi[k] = fmaxf(hi[k], s_hi[k][w]); }
+    const float cx = 0.5f * lo[0] + 0.5f * hi[0], cy = 0.5f * lo[1] + 0.5f * hi[1], cz = 0.5f * lo[2] + 0.5f * hi[2];
+    float far2 = 0.f;
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+        const float4 p = S[i];
+        const float x = p.x - cx, y = p.y - cy, z = p.z - cz;
+        far2 = fmaxf(far2, x * x + y * y + z * z);
+    }
+    for (int o = 16; o > 0; o >>= 1) far2 = fmaxf(far2, __shfl_xor_sync(0xffffffffu, far2, o));
+    __syncthreads();                       // s_lo has been read
+    if (lane == 0) s_lo[0][warp] = far2;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 0; w < 32; ++w) far2 = fmaxf(far2, s_lo[0][w]);
+        *frame = make_float4(cx, cy, cz, sqrtf(far2) * (1.f + 1e-5f) + 1e-30f);
+    }
     const float ext = fmaxf(fmaxf(hi[0] - lo[0], hi[1] - lo[1]), fmaxf(hi[2] - lo[2], 1e-30f));
     auto spread = [](unsigned v) {         // ten bits, two zeros after each
         v = (v | (v << 16)) & 0x030000ffu;
@@ -767,12 +750,12 @@ cudaError_t init_cells_attributes()
                                 8192 * (int)sizeof(unsigned long long));
 }
 
-cudaError_t launch_sort_points(const float4 *S, int N, float4 *out, cudaStream_t st)
+cudaError_t launch_sort_points(const float4 *S, int N, float4 *out, float4 *frame, cudaStream_t st)
 {
     static_assert(kMaxN <= 8192, "shared-memory sort");
     int Npow = 2;
     while (Npow < N) Npow <<= 1;
-    sort_points_kernel<<<1, 1024, (size_t)Npow * sizeof(unsigned long long), st>>>(S, N, Npow, out);
+    sort_points_kernel<<<1, 1024, (size_t)Npow * sizeof(unsigned long long), st>>>(S, N, Npow, out, frame);
     return cudaGetLastError();
 }
 

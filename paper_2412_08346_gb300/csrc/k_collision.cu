@@ -2,7 +2,7 @@
 // collision cloud in every particle's gripper frame (Eq. 12, Section IV-C) and
 // the reverse matching of the colliding points onto the transformed contact
 // cloud (Eq. 18).
-#include "asicp_internal.cuh"
+#include "cells.cuh"
 
 #include <climits>
 
@@ -473,6 +473,137 @@ __global__ void __launch_bounds__(kColThreads) collide_nn_kernel(const CollideAr
     }
 }
 
+// Reverse matching through the cells of the gripper clouds: the nearest gripper point of a
+// colliding point c among the transformed cloud, by the same float32 distances |c - s'| in the
+// object frame as collide_nn_kernel, but only of the points that can be nearest.  The
+// cells belong to the gripper cloud in its own frame (built once per gripper), where c is
+// at x = R^T (c - t).  What that mapping and the rounding of s' can change, u = 2^-24: x is off
+// by at most 20 u |x| (a rounded c - t, three products and sums per coordinate, R
+// orthonormal up to 8 u), s' by 6 u (|t|_1 + 2 max |s|) and by 8 u |s| for R again; distances
+// all scale by |q|^2 alike.  The lists hold for positions off by kGripperTol / 2.5 of the
+// cloud's radius; a colliding point beyond that bound (an object metres from its frame's origin)
+// compares the whole cloud.  64 threads per item, one per colliding point; the item's sums
+// are added in collide_nn_kernel's order, so they are the same to the last bit.
+// Measured on GB300 (per pass, against collide_nn_kernel): 3 x 256 particles, N 2048 18 us
+// against 71 (2.3e5 colliding points); 3 x 1024, N 4096 0.79 ms against 14.6 (9.8e6); 2 x 64,
+// N 1024 12 against 16.  A third goes into the item's sums, the rest is the latency of
+// the chain item, particle, point, table, nodes, list, gripper points.
+constexpr int kRec = 9;                // floats per record (8 used: the odd stride spreads the banks)
+__global__ void __launch_bounds__(kColChunk) collide_cells_kernel(const CollideArgs a)
+{
+    if (a.err && *a.err != kDevOk) return;
+    __shared__ float sRec[kColChunk][kRec];
+    const int tid = threadIdx.x, lane = tid & 31, N = a.L.N;
+    const int count = a.col_items[0];
+    for (int item = blockIdx.x; item < count; item += gridDim.x) {
+        const int2 it = reinterpret_cast<const int2 *>(a.col_list)[item];
+        const int pk = it.x, slot = it.y * kColChunk + tid;
+        const int grp = a.L.part_grp[pk], p = grp % a.L.P;
+        const ObjMeta &om = a.L.obj[grp / a.L.P];
+        const bool valid = slot < a.ncol[pk];
+        const long long at = om.colidx_base + (long long)(pk - om.pfirst) * om.Mc + slot;
+        const float4 c = valid ? __ldg(om.C + a.colidx[at]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float *th = a.theta + (size_t)pk * 8;
+        const float tx = th[0], ty = th[1], tz = th[2];
+        float Rm[9];
+        quat_rot_f32(th[3], th[4], th[5], th[6], Rm);
+        const float4 *__restrict__ S = a.S + (size_t)p * N;
+        const int *__restrict__ leaves = a.pre_leaves + (size_t)p * a.pre_leaf_cap;
+        const float4 fr = __ldg(a.pre_frame + p);
+        auto dist = [&](int i, float cx, float cy, float cz) {
+            const float4 s = __ldg(S + i);
+            const float3 o = xform_f32(Rm, tx, ty, tz, s.x, s.y, s.z);
+            return dist2_f32(o.x, o.y, o.z, cx, cy, cz);
+        };
+
+        int2 nd = make_int2(0, 0);
+        if (valid) {
+            const float dx = __fsub_rn(c.x, tx), dy = __fsub_rn(c.y, ty), dz = __fsub_rn(c.z, tz);
+            const float x = fmaf(Rm[0], dx, fmaf(Rm[3], dy, Rm[6] * dz)), y = fmaf(Rm[1], dx, fmaf(Rm[4], dy, Rm[7] * dz)),
+                        z = fmaf(Rm[2], dx, fmaf(Rm[5], dy, Rm[8] * dz));
+            const float reach = fabsf(fr.x) + fabsf(fr.y) + fabsf(fr.z) + fr.w;      // >= max |s|
+            const float off = 1.2e-6f * (fabsf(x) + fabsf(y) + fabsf(z) + reach) + 4e-7f * (fabsf(tx) + fabsf(ty) + fabsf(tz));
+            nd = off <= 0.4f * kGripperTol * fr.w
+                     ? find_cell(a.pre_nodes + (size_t)p * a.pre_node_cap, cell_half(fr.w, kGripperCells), x - fr.x, y - fr.y,
+                                 z - fr.z)
+                     : make_int2(0, kCellWhole);
+        }
+        float best = __int_as_float(0x7f800000);
+        int bi = 0x7fffffff;
+        if (nd.y <= kCellOwn) {
+            const int4 *l = reinterpret_cast<const int4 *>(leaves + nd.x);
+            for (int e = 0; e < nd.y; e += 4, ++l) {
+                const int4 id = __ldg(l);
+                const float d0 = dist(id.x, c.x, c.y, c.z), d1 = dist(id.y, c.x, c.y, c.z), d2 = dist(id.z, c.x, c.y, c.z),
+                            d3 = dist(id.w, c.x, c.y, c.z);
+                if (d0 < best) { best = d0; bi = id.x; }
+                if (d1 < best) { best = d1; bi = id.y; }
+                if (d2 < best) { best = d2; bi = id.z; }
+                if (d3 < best) { best = d3; bi = id.w; }
+            }
+        }
+        unsigned pending = __ballot_sync(0xffffffffu, nd.y == kCellWhole || nd.y > kCellOwn);
+        while (pending) {
+            const int src = __ffs(pending) - 1;
+            pending &= pending - 1;
+            const float qx = __shfl_sync(0xffffffffu, c.x, src), qy = __shfl_sync(0xffffffffu, c.y, src),
+                        qz = __shfl_sync(0xffffffffu, c.z, src);
+            const int base = __shfl_sync(0xffffffffu, nd.x, src), len = __shfl_sync(0xffffffffu, nd.y, src);
+            float wb = __int_as_float(0x7f800000);
+            int wi = 0x7fffffff;
+            for (int e = lane; e < (len == kCellWhole ? N : len); e += 32) {
+                const int i = len == kCellWhole ? e : __ldg(leaves + base + e);
+                const float d = dist(i, qx, qy, qz);
+                if (d < wb || (d == wb && i < wi)) { wb = d; wi = i; }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) argmin_xor(wb, wi, o);
+            if (lane == src) { best = wb; bi = wi; }
+        }
+        {
+            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (valid) {
+                bi = bi < N ? bi : 0;      // no finite distance at all (not reached with finite inputs)
+                s = __ldg(S + bi);
+                if (a.dbg_colnn) a.dbg_colnn[at] = bi;
+            }
+            float *rec = sRec[tid];
+            rec[0] = s.x; rec[1] = s.y; rec[2] = s.z;
+            rec[3] = c.x; rec[4] = c.y; rec[5] = c.z;
+            rec[6] = valid ? 1.f : 0.f;
+        }
+        __syncthreads();
+        // the item's sums, as in collide_nn_kernel: (sum e, part) adds colliding points part + 8 u
+        for (int e0 = 0; e0 < kColSums; e0 += kColChunk / 8) {
+            const int e = e0 + (tid >> 3), part = tid & 7;
+            dfloat acc{0.f, 0.f};
+            if (e < kColSums) {
+                const int ia = kColSel[e][0], ib = kColSel[e][1];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const float *rec = sRec[part + 8 * u];
+                    df_add_prod(acc, rec[ia], rec[ib]);
+                    if (e == kColSums - 1) {
+                        df_add_prod(acc, rec[4], rec[4]);
+                        df_add_prod(acc, rec[5], rec[5]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                dfloat y;
+                y.hi = __shfl_xor_sync(0xffffffffu, acc.hi, o);
+                y.lo = __shfl_xor_sync(0xffffffffu, acc.lo, o);
+                df_merge(acc, y);
+            }
+            if (part == 0 && e < kColSums)
+                a.csums[(om.csum_base + (long long)(pk - om.pfirst) * om.chunks + it.y) * kColSums + e] =
+                    (double)acc.hi + (double)acc.lo;
+        }
+        __syncthreads();
+    }
+}
+
 cudaError_t launch_collide(const CollideArgs &a, cudaStream_t st)
 {
     collide_kernel<<<a.L.T, kTestThreads, 0, st>>>(a);
@@ -495,6 +626,10 @@ cudaError_t launch_collide_nn(const CollideArgs &a, cudaStream_t st)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         return 4 * sms;
     });
+    if (a.cells) {          // 24 small CTAs per SM, no more than the work list can hold
+        collide_cells_kernel<<<a.most_items < 6 * grid ? a.most_items : 6 * grid, kColChunk, 0, st>>>(a);
+        return cudaGetLastError();
+    }
     const size_t smem = 2 * sizeof(float4) * (size_t)((a.L.N + 63) / 64 * 64) + 32 * sizeof(float4);
     collide_nn_kernel<<<grid, kColThreads, smem, st>>>(a);
     return cudaGetLastError();

@@ -81,3 +81,36 @@ def test_cells_find_the_nearest_points(kind, M):
         assert np.all(b["nn_idx"][pk][tie] < a["nn_idx"][pk][tie])
         if np.abs(t[pk % K] - c).max() < 1.0:
             assert len(diff) == 0
+
+
+@pytest.mark.parametrize("N,offset", [(511, 0.0), (512, 0.0), (2047, 0.0), (1000, 3.0), (1000, 30.0)])
+def test_gripper_cells_give_the_same_reverse_matches(N, offset):
+    """Reverse matching through the gripper clouds' cells (512 points and more, once the steps have paid for
+    their build; an object metres away is beyond their tolerance and compares the whole cloud)
+    against the brute-force kernel of a context's first step: every output of the step the same."""
+    w = synth.custom_case(P=2, K=24, N=N, M=1500, grid=40, k_max=4, seed=83, k_stein=0)
+    w.objects[0].points = (w.objects[0].points + np.float32(offset)).astype(np.float32)
+    g = np.random.default_rng(N)
+    t = w.objects[0].points.mean(0, dtype=np.float64) + g.normal(size=(48, 3)) * 0.02
+    q = g.normal(size=(48, 4))
+    theta = np.concatenate([t, q / np.linalg.norm(q, axis=1, keepdims=True)], 1).astype(np.float32)
+    states = []
+    for steps in (1, 80):
+        ctx = asicp.asicp_create(tl.make_config(w, torch.cuda.current_stream().cuda_stream))
+        try:
+            keep = tl.upload(ctx, w)
+            for _ in range(steps):
+                asicp.asicp_set_state(ctx, theta, 0)
+                asicp.asicp_step(ctx, 0)
+            states.append(tl.read_state(ctx, 2, 24, N, 1500))
+            del keep
+        finally:
+            asicp.asicp_destroy(ctx)
+    a, b = states
+    assert a["ncol"].max() > 64
+    for pk in range(48):
+        n = a["ncol"][pk]
+        assert np.array_equal(a["col_list"][pk, :n], b["col_list"][pk, :n])
+        assert np.array_equal(a["col_nn"][pk, :n], b["col_nn"][pk, :n])
+    for key in ("theta", "cost", "grad", "ncol"):
+        assert np.array_equal(a[key], b[key]), key
