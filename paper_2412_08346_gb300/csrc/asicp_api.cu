@@ -72,8 +72,9 @@ struct DevMem {
 struct ObjBufs {
     DevMem R, Rx, Rt, C;      // C stays empty when the collision cloud is R itself
     DevMem nodes, leaves;     // matching cells of R
+    DevMem Csort, Cball;      // the collision cloud in spatial order
     int M = 0, Mpad = 0, Mc = 0;
-    bool set = false, cells_built = false;
+    bool set = false, cells_built = false, sorted = false;
 };
 
 // Matching through cells (k_cells.cu): for clouds of kCellMinM points and more (the screening
@@ -106,6 +107,7 @@ struct asicp_ctx {
     std::vector<SdfMeta> meta;
     std::vector<DevMem> grids;
     std::vector<DevMem> cells;         // corner-packed grids
+    std::vector<DevMem> clear;         // their cells' clearances
     int k_next = 0;
 
     // mini-batches of the object cloud per iteration (Table I), one object only
@@ -130,7 +132,7 @@ struct asicp_ctx {
     std::vector<int> grp_off_h;
     std::vector<ObjMeta> objmeta_h;
 
-    DevMem partgrp, grpoff, objmeta, items, ctaoff, com, frame, colitems, collist, box, stage, S, Ssort, preframe, prenodes, preleaves, cellwork, pconst, dmeta, theta, fsums,
+    DevMem partgrp, grpoff, objmeta, items, ctaoff, com, frame, colitems, collist, stage, S, Ssort, preframe, prenodes, preleaves, cellwork, pconst, dmeta, theta, fsums,
         csums, ncol, colidx, cost, grad, prev, frozen, phi, h, order, errw, out7, outc, outi, nnidx, tccand, dbg_d2, dbg_sp,
         dbg_colnn;
 
@@ -317,6 +319,8 @@ void build_layout(asicp_ctx *c)
         m.Rt = b.Rt.as<float>();
         m.nodes = b.nodes.as<int2>();
         m.leaves = b.leaves.as<int>();
+        m.Csort = b.Csort.as<float4>();
+        m.Cball = b.Cball.as<float4>();
         m.C = b.C.p ? b.C.as<float4>() : b.R.as<float4>();
         m.M = b.M;
         m.Mpad = b.Mpad;
@@ -541,7 +545,7 @@ void ensure_cells(asicp_ctx *c, int v, int passes)
             b.nodes = o.nodes.as<int2>();
             b.leaves = o.leaves.as<int>();
             b.M = o.M;
-            b.factor = kObjectCells;
+            b.log_factor = kObjectCells;
             builds.push_back(b);
         }
         ensure_cell_scratch(c, builds);
@@ -563,6 +567,28 @@ void ensure_cells(asicp_ctx *c, int v, int passes)
     if (!c->cells_on) return;
     build_cells(c, builds);
     for (int o : todo) c->objs[o].cells_built = true;
+}
+
+// Sort the collision clouds that are new into their spatial order (before the kernels run, and
+// outside any capture), those of all objects together.
+void ensure_sorted(asicp_ctx *c)
+{
+    CloudBatch batch{};
+    int n = 0;
+    for (ObjBufs &o : c->objs) {
+        if (o.sorted) continue;
+        const float4 *src = o.C.p ? o.C.as<float4>() : o.R.as<float4>();
+        for (int seg = 0; seg < o.Mc; seg += kColSegment) {
+            batch.b[n++] = {src + seg, o.Csort.as<float4>() + seg, o.Cball.as<float4>() + seg / 32,
+                            std::min(kColSegment, o.Mc - seg)};
+            if (n == kCloudBatch) {
+                ck(launch_sort_clouds(batch, n, c->st), "collision cloud order");
+                n = 0;
+            }
+        }
+        o.sorted = true;
+    }
+    if (n > 0) ck(launch_sort_clouds(batch, n, c->st), "collision cloud order");
 }
 
 // Decide whether the reverse matching of the next `passes` passes goes through the cells of the
@@ -592,7 +618,7 @@ void ensure_pre_cells(asicp_ctx *c, int passes)
             b.nodes = c->prenodes.as<int2>() + (size_t)p * s.node_cap;
             b.leaves = c->preleaves.as<int>() + (size_t)p * s.leaf_cap;
             b.M = c->N;
-            b.factor = kGripperCells;
+            b.log_factor = kGripperCells;
             b.tol = kGripperTol;
             b.near_only = 1;
             builds.push_back(b);
@@ -866,10 +892,10 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
     }
     // what the layout (object table, work plan) and the captured loop depend on
     const bool was_set = b.set;
-    const void *was[4] = {b.R.p, b.Rx.p, b.Rt.p, b.C.p};
+    const void *was[6] = {b.R.p, b.Rx.p, b.Rt.p, b.C.p, b.Csort.p, b.Cball.p};
     const int was_M = b.M, was_Mc = b.Mc, was_Mpad = b.Mpad;
     b.set = false;
-    b.cells_built = false;
+    b.cells_built = b.sorted = false;
     ctx->cells_owed = 0.0;
     ctx->run_done = false;
     ctx->stage.ensure(sizeof(float) * 3 * (size_t)(M > mc ? M : mc), "staging");
@@ -883,6 +909,8 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
     } else {
         b.C.release();
     }
+    b.Csort.ensure(sizeof(float4) * (size_t)mc, "collision cloud, sorted");
+    b.Cball.ensure(sizeof(float4) * (((size_t)mc + 31) / 32), "collision cloud, balls");
     ck(launch_centroid(b.R.as<float4>(), M, ctx->com.as<double>() + 3 * o, ctx->st), "centroid");
     const int Mpad = (M + kRefTilePts - 1) / kRefTilePts * kRefTilePts;
     b.Rx.ensure(sizeof(float4) * (size_t)Mpad, "screening layout");
@@ -898,7 +926,7 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
     // a new object of the same sizes in the same buffers keeps the layout, the poses
     // and the captured loop (whose kernels read the object's data at replay)
     if (!was_set || M != was_M || mc != was_Mc || Mpad != was_Mpad || b.R.p != was[0] || b.Rx.p != was[1] ||
-        b.Rt.p != was[2] || b.C.p != was[3])
+        b.Rt.p != was[2] || b.C.p != was[3] || b.Csort.p != was[4] || b.Cball.p != was[5])
         ctx->layout_dirty = true;
 }
 
@@ -959,6 +987,7 @@ asicp_status asicp_create(const asicp_config *cfg, asicp_ctx **out)
     c->meta.assign(cfg->P, SdfMeta{});
     c->grids.resize(cfg->P);
     c->cells.resize(cfg->P);
+    c->clear.resize(cfg->P);
     c->objs.resize(c->nobj);
     c->Kg.assign((size_t)c->nobj * cfg->P, cfg->K);
     asicp_status s = guarded(c, [&] {
@@ -1093,31 +1122,19 @@ asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_
         ctx->cells[preshape].ensure(sdf_cells_bytes(nx, ny, nz), "corner-packed sdf grid");
         ck(launch_sdf_pack_cells(ctx->grids[preshape].as<float>(), nx, ny, nz, ctx->cells[preshape].as<float4>(), ctx->st),
            "pack sdf cells");
-        // index box of the positive nodes -> gripper-frame box holding every cell that
-        // has a positive corner (trilinear values outside it cannot be > 0)
-        ctx->box.ensure(sizeof(int) * 6, "sdf box");
-        const int box_init[6] = {INT_MAX, INT_MAX, INT_MAX, INT_MIN, INT_MIN, INT_MIN};
-        ck(cudaMemcpyAsync(ctx->box.p, box_init, sizeof(box_init), cudaMemcpyHostToDevice, ctx->st), "init sdf box");
-        ck(launch_sdf_box(ctx->grids[preshape].as<float>(), nx, ny, nz, ctx->box.as<int>(), ctx->st), "sdf box");
-        int box6[6];
-        ck(cudaMemcpyAsync(box6, ctx->box.p, sizeof(box6), cudaMemcpyDeviceToHost, ctx->st), "read sdf box");
+        const size_t nc = sdf_cells_bytes(nx, ny, nz) / (2 * sizeof(float4));
+        ctx->clear[preshape].ensure(nc, "sdf clearances");
+        ctx->stage.ensure(nc, "staging");
+        ck(launch_sdf_clear(ctx->cells[preshape].as<float4>(), nx, ny, nz, ctx->clear[preshape].as<unsigned char>(),
+                            ctx->stage.as<unsigned char>(), ctx->st), "sdf clearances");
         sync_and_check_err(ctx, "set_gripper_sdf");
         SdfMeta m{};
         m.grid = ctx->grids[preshape].as<float>();
         m.cells = ctx->cells[preshape].as<float4>();
+        m.clear = ctx->clear[preshape].as<unsigned char>();
         m.nx = nx; m.ny = ny; m.nz = nz;
         m.ox = org[0]; m.oy = org[1]; m.oz = org[2];
         m.voxel = voxel;
-        for (int a = 0; a < 3; ++a) {
-            if (box6[a] == INT_MAX) {            // no positive node: nothing can collide
-                m.lo[a] = 1.f;
-                m.hi[a] = -1.f;
-            } else {
-                const double margin = 1e-3 * voxel;
-                m.lo[a] = (float)(org[a] + (double)voxel * (box6[a] - 1) - margin);
-                m.hi[a] = (float)(org[a] + (double)voxel * (box6[3 + a] + 1) + margin);
-            }
-        }
         ctx->meta[preshape] = m;
         ck(cudaMemcpyAsync(ctx->dmeta.as<SdfMeta>() + preshape, &ctx->meta[preshape], sizeof(SdfMeta),
                            cudaMemcpyHostToDevice, ctx->st), "copy sdf meta");
@@ -1168,6 +1185,7 @@ asicp_status asicp_step(asicp_ctx *ctx, int k)
         if (k < 0 || k >= ctx->cfg.k_max) fail(ASICP_ERR_INVALID_ARG, "step: k out of [0, k_max)");
         ensure_cells(ctx, ctx->fwd_variant, 1);
         ensure_pre_cells(ctx, 1);
+        ensure_sorted(ctx);
         step_impl(ctx, k);
         ctx->run_done = false;
     });
@@ -1195,6 +1213,7 @@ asicp_status asicp_run(asicp_ctx *ctx, const float *theta0)
         if (ctx->cfg.autotune && !ctx->tuned) autotune_impl(ctx, nullptr);
         ensure_cells(ctx, ctx->fwd_variant, ctx->cfg.k_max + 1);
         ensure_pre_cells(ctx, ctx->cfg.k_max + 1);
+        ensure_sorted(ctx);
         run_loop_graph(ctx);
         ctx->k_next = ctx->cfg.k_max;
         ctx->stepped = true;

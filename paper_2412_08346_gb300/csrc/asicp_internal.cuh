@@ -41,7 +41,8 @@ struct SdfMeta {           // one preshape's grid
     int nx, ny, nz;
     float ox, oy, oz;      // position of node (0,0,0)
     float voxel;
-    float lo[3], hi[3];    // box (gripper frame) holding every cell with a positive corner
+    const unsigned char *clear;   // per cell (same order) its distance in cells to the nearest one
+                                  // with a positive corner (largest coordinate, at most 255)
 };
 
 // Rotation of a (unit) quaternion in the homogeneous form
@@ -201,6 +202,8 @@ struct ObjMeta {
     const int2 *nodes;        // matching cells (k_cells.cu): tables and nodes, and the
     const int *leaves;        // points that can be nearest per cell; null where not built
     const float4 *C;          // [Mc] collision points (may alias R)
+    const float4 *Csort;      // [Mc] the same in spatial order per segment, w = index in the segment
+    const float4 *Cball;      // [ceil(Mc / 32)] bounding balls of 32 points of Csort (w = radius)
     int M, Mpad, Mc, chunks;  // chunks = ceil(Mc / kColChunk)
     int pfirst, np;           // first particle and number of particles of this object
     long long colidx_base;    // this object's collision lists start here ([np][Mc] ints)
@@ -281,13 +284,14 @@ struct CellBuild {
     void *recs;
     int *ctr;
     int M, leaf_cap, list_cap, cell_cap, node_cap;
-    float factor;             // near cells reach this many times the power of two above the radius
+    int log_factor;           // near cells reach 2^log_factor times the power of two above the radius
     float tol;                // positions looked up may be off by 0.4 tol times the radius
     int near_only;            // no cells beyond the near ones
 };
 // Cells of objects, and of gripper clouds in the gripper frame (colliding points lie in the
 // gripper's body, not far from its surface; see collide_cells_kernel for the tolerance).
-constexpr float kObjectCells = 4.f, kGripperCells = 2.f, kGripperTol = 1.25e-4f;
+constexpr int kObjectCells = 2, kGripperCells = 1;     // (log_factor)
+constexpr float kGripperTol = 1.25e-4f;
 struct CellBuildBatch {
     CellBuild b[kCellBatch];
 };
@@ -302,6 +306,20 @@ cudaError_t launch_sort_points(const float4 *S, int N, float4 *out, float4 *fram
 cudaError_t init_cells_attributes();
 
 constexpr int kColChunk = 64;          // colliding points per reverse-matching work item
+
+// Spatial order of the collision clouds: segments of at most kColSegment points, several
+// (of several objects) per launch.
+constexpr int kColSegment = 65536;
+struct CloudSort {
+    const float4 *src;
+    float4 *dst, *balls;
+    int n;
+};
+constexpr int kCloudBatch = 64;
+struct CloudBatch {
+    CloudSort b[kCloudBatch];
+};
+cudaError_t launch_sort_clouds(const CloudBatch &batch, int n, cudaStream_t st);
 
 struct CollideArgs {
     Layout L;
@@ -363,7 +381,8 @@ cudaError_t launch_fibonacci(const Layout &L, float radius, int mode, float *the
 cudaError_t launch_gather_points(const float4 *R, const int *idx, int n, float4 *out, cudaStream_t st);
 cudaError_t launch_store_meta(ObjMeta *dst, const ObjMeta &v, cudaStream_t st);
 cudaError_t launch_set_theta(const float *theta7, int T, float *theta8, int *err, cudaStream_t st);
-cudaError_t launch_sdf_box(const float *grid, int nx, int ny, int nz, int *box6, cudaStream_t st);
+cudaError_t launch_sdf_clear(const float4 *cells, int nx, int ny, int nz, unsigned char *clear, unsigned char *tmp,
+                             cudaStream_t st);
 cudaError_t launch_sdf_pack_cells(const float *grid, int nx, int ny, int nz, float4 *cells, cudaStream_t st);
 size_t sdf_cells_bytes(int nx, int ny, int nz);
 cudaError_t launch_select(const Layout &L, const double *cost, const int *ncol, int *order, cudaStream_t st);

@@ -35,9 +35,9 @@
 // common sphere or plane, float32 resolution far out): its queries scan it as it is.
 //
 // Measured on GB300 (per pass, against screening and exact choice on the tensor cores): 3 x 256
-// particles, N 2048, M 8192 38 us against 783; 3 x 1024, N 4096, M 65536 0.31 ms against 41.4;
-// lists of at most 12 points (16: 44 us, 24: 46, 32: 52, 48: 60; at 8 they stop shrinking
-// and the budgets run out).  What bounds the matching is the latency of its dependent loads
+// particles, N 2048, M 8192 34 us against 783; 3 x 1024, N 4096, M 65536 0.28 ms against 41.4;
+// lists of at most 12 points (with one flat grid of queries, which divided each by N: 12 38 us,
+// 16 44, 24 46, 32 52, 48 60; at 8 they stop shrinking and the budgets run out).  What bounds the matching is the latency of its dependent loads
 // (table, two or three nodes, list, points), all from L2 and L1; queries in the gripper
 // cloud's own order take 68 us.  The build (ten rounds of few and uneven cells, latency again)
 // takes 0.10 ms at 1024 points, 0.27 at 8192, 1.4 at 65536.
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(256) cells_start_kernel(const CellBuildBatch b
     __shared__ int s_cnt[8], s_leaf, s_base;
     __shared__ unsigned s_mask[8][kStartMask];
     const float4 fr = *b.frame;
-    const float J = cell_half(fr.w, b.factor), k = (5e-7f + b.tol) * fr.w;
+    const float J = cell_half(fr.w, b.log_factor), k = (5e-7f + b.tol) * fr.w;
     int cell = blockIdx.x;
     CellRef r;
     r.shell = -1;
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(256) cells_level_kernel(const CellBuildBatch b
     __shared__ int s_pos[8][9], s_cnt[8];
     __shared__ Place s_place;
     const float4 fr = *b.frame;
-    const float J = cell_half(fr.w, b.factor), k = (5e-7f + b.tol) * fr.w;
+    const float J = cell_half(fr.w, b.log_factor), k = (5e-7f + b.tol) * fr.w;
     for (int u = blockIdx.x; u < n_long * children; u += gridDim.x) {
         const CellRef r = recs(b, round)[b.cell_cap - 1 - u / children];
         if (r.len <= 0) continue;
@@ -566,19 +566,19 @@ __global__ void __launch_bounds__(256) cells_level_kernel(const CellBuildBatch b
     }
 }
 
-// The matching itself: one thread per query.  Queries are taken in the gripper cloud's
-// spatial order (S sorted along a space-filling curve, w = the point's own index), so
-// that the lanes of a warp meet in the same cells.
-__global__ void __launch_bounds__(256) cells_match_kernel(const FwdArgs a)
+// The matching itself: one thread per query, a particle's queries in CTAs of their own (its pose
+// and object are the CTA's, and no query divides by N).  Queries are taken in the gripper cloud's
+// spatial order (S sorted along a space-filling curve, w = the point's own index), so that
+// the lanes of a warp meet in the same cells.
+constexpr int kMatchThreads = 128;
+
+__global__ void __launch_bounds__(kMatchThreads) cells_match_kernel(const FwdArgs a, int ctas)
 {
-    const long long Qtot = (long long)a.L.T * a.L.N;
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31;
-    const bool valid = g < Qtot;
-    const long long gq = valid ? g : Qtot - 1;
-    const int pk = (int)(gq / a.L.N);
+    const int pk = blockIdx.x / ctas, k = (blockIdx.x - pk * ctas) * kMatchThreads + threadIdx.x;
+    const int lane = threadIdx.x & 31, N = a.L.N;
+    const bool valid = k < N;
     const int grp = a.L.part_grp[pk], obj = grp / a.L.P;
-    const float4 s = a.Ssort[(size_t)(grp % a.L.P) * a.L.N + (gq - (long long)pk * a.L.N)];
+    const float4 s = a.Ssort[(size_t)(grp - obj * a.L.P) * N + min(k, N - 1)];
     const float *th = a.theta + (size_t)pk * 8;
     float Rm[9];
     quat_rot_f32(th[3], th[4], th[5], th[6], Rm);
@@ -613,14 +613,13 @@ __global__ void __launch_bounds__(256) cells_match_kernel(const FwdArgs a)
         pending &= pending - 1;
         const float qx = __shfl_sync(0xffffffffu, o.x, src), qy = __shfl_sync(0xffffffffu, o.y, src),
                     qz = __shfl_sync(0xffffffffu, o.z, src);
-        const ObjMeta &qm = a.L.obj[__shfl_sync(0xffffffffu, obj, src)];
         const int base = __shfl_sync(0xffffffffu, nd.x, src), len = __shfl_sync(0xffffffffu, nd.y, src);
-        const int n = len == kWhole ? qm.M : len;
+        const int n = len == kWhole ? om.M : len;
         float wb = __int_as_float(0x7f800000);
         int wi = 0x7fffffff;
         for (int e = lane; e < n; e += 32) {
-            const int r = len == kWhole ? e : __ldg(qm.leaves + base + e);
-            const float4 p = __ldg(qm.R + r);
+            const int r = len == kWhole ? e : __ldg(om.leaves + base + e);
+            const float4 p = __ldg(R + r);
             const float d = dist2_f32(qx, qy, qz, p.x, p.y, p.z);
             if (d < wb || (d == wb && r < wi)) { wb = d; wi = r; }
         }
@@ -632,7 +631,7 @@ __global__ void __launch_bounds__(256) cells_match_kernel(const FwdArgs a)
         if (lane == src) { best = wb; bi = wi; }
     }
     if (!valid) return;
-    const long long q = (long long)pk * a.L.N + __float_as_int(s.w);
+    const long long q = (long long)pk * N + __float_as_int(s.w);
     a.nn_idx[q] = best < __int_as_float(0x7f800000) ? bi : 0;      // no finite distance: 0
     if (a.dbg_d2) a.dbg_d2[q] = best;
     if (a.dbg_sp) {
@@ -662,9 +661,9 @@ cudaError_t launch_cells_build(const CellBuildBatch &batch, int n, cudaStream_t 
 
 cudaError_t launch_cells_match(const FwdArgs &a, cudaStream_t st)
 {
-    const long long Qtot = (long long)a.L.T * a.L.N;
-    if (Qtot == 0) return cudaSuccess;
-    cells_match_kernel<<<(unsigned)((Qtot + 255) / 256), 256, 0, st>>>(a);
+    if (a.L.T == 0) return cudaSuccess;
+    const int ctas = (a.L.N + kMatchThreads - 1) / kMatchThreads;
+    cells_match_kernel<<<(unsigned)(a.L.T * ctas), kMatchThreads, 0, st>>>(a, ctas);
     return cudaGetLastError();
 }
 

@@ -4,24 +4,21 @@
 // cloud (Eq. 18).
 #include "cells.cuh"
 
-#include <climits>
-
 namespace asicp {
 
 namespace {
 constexpr int kColThreads = 256;       // reverse matching
-constexpr int kTestThreads = 128;      // collision test: one CTA per particle, small enough that every
-                                       // particle of a paper-scale launch is resident at once
-constexpr int kColU = 4;          // collision points per thread per compaction round
+constexpr int kTestThreads = 128;      // collision test and matching sums: one small CTA per particle each
+constexpr int kSegWords = kColSegment / 32;      // words of a segment's bit map = most chunks of a segment
+constexpr int kTestB = 4;         // chunks per warp whose loads overlap
 constexpr int kPairB = 4;         // matching pairs per thread whose loads overlap (57.5 us per paper-scale
                                   // launch against 61.8 us one pair at a time; 72 registers, 7 CTAs per SM)
 
-// Trilinear interpolation of a node-centred grid at gripper-frame point (x, y, z).
-// Returns false when the point lies outside the grid's node box (the grid covers
-// the gripper, so such a point is not inside it).  The eight corner values come
-// from the corner-packed copy of the grid: one 32-byte record per cell, read as
-// two float4 from a single 32-byte sector.
-__device__ __forceinline__ bool sdf_lookup(const SdfMeta &m, float x, float y, float z, float &val)
+// Whether point (x, y, z) of the gripper frame collides: inside the grid's node box (the grid covers
+// the gripper, so a point outside is not in it) and trilinear value > 0 (Eq. 12).  Only a
+// cell with a positive corner (clear 0) can interpolate to a positive value; its eight
+// corners come from the corner-packed copy of the grid, two float4 from one 32-byte sector.
+__device__ __forceinline__ bool sdf_hit(const SdfMeta &m, float x, float y, float z)
 {
     const float ux = __fdiv_rn(__fsub_rn(x, m.ox), m.voxel);
     const float uy = __fdiv_rn(__fsub_rn(y, m.oy), m.voxel);
@@ -32,15 +29,39 @@ __device__ __forceinline__ bool sdf_lookup(const SdfMeta &m, float x, float y, f
     const int ix = min((int)floorf(ux), m.nx - 2);
     const int iy = min((int)floorf(uy), m.ny - 2);
     const int iz = min((int)floorf(uz), m.nz - 2);
+    const size_t at = (size_t)ix + (size_t)(m.nx - 1) * ((size_t)iy + (size_t)(m.ny - 1) * iz);
+    if (__ldg(m.clear + at) != 0) return false;
     const float fx = ux - (float)ix, fy = uy - (float)iy, fz = uz - (float)iz;
-    const float4 *cell = m.cells + 2 * ((size_t)ix + (size_t)(m.nx - 1) * ((size_t)iy + (size_t)(m.ny - 1) * iz));
+    const float4 *cell = m.cells + 2 * at;
     const float4 z0 = __ldg(cell), z1 = __ldg(cell + 1);
     const float c000 = z0.x, c100 = z0.y, c010 = z0.z, c110 = z0.w;
     const float c001 = z1.x, c101 = z1.y, c011 = z1.z, c111 = z1.w;
     const float gx = 1.f - fx, gy = 1.f - fy, gz = 1.f - fz;
-    val = gx * gy * gz * c000 + fx * gy * gz * c100 + gx * fy * gz * c010 + fx * fy * gz * c110 +
-          gx * gy * fz * c001 + fx * gy * fz * c101 + gx * fy * fz * c011 + fx * fy * fz * c111;
-    return true;
+    const float val = gx * gy * gz * c000 + fx * gy * gz * c100 + gx * fy * gz * c010 + fx * fy * gz * c110 +
+                      gx * gy * fz * c001 + fx * gy * fz * c101 + gx * fy * fz * c011 + fx * fy * fz * c111;
+    return val > 0.f;
+}
+
+// clear of the cell that holds point (x, y, z), found without divisions: it may be a neighbour of the
+// cell sdf_hit finds (inv = 1 / voxel is rounded), so the point cannot collide when this is above
+// 1.  Points outside the grid get the nearest cell's.
+__device__ __forceinline__ int cell_clear(const SdfMeta &m, float inv, float x, float y, float z)
+{
+    const int ix = (int)fminf(fmaxf((x - m.ox) * inv, 0.f), (float)(m.nx - 2));
+    const int iy = (int)fminf(fmaxf((y - m.oy) * inv, 0.f), (float)(m.ny - 2));
+    const int iz = (int)fminf(fmaxf((z - m.oz) * inv, 0.f), (float)(m.nz - 2));
+    return __ldg(m.clear + (size_t)ix + (size_t)(m.nx - 1) * ((size_t)iy + (size_t)(m.ny - 1) * iz));
+}
+
+// Whether a ball of radius rho around the gripper-frame point (x, y, z) can hold a colliding point:
+// clear is the distance in cells (largest coordinate) from a cell to the nearest one with a
+// positive corner, and rho voxels reach ceil(rho) cells.  A centre outside the grid is
+// moved to the nearest cell, which only shortens the distance.  The slack covers the rounding
+// of the centre's and the points' coordinates (1e-6 of them).
+__device__ __forceinline__ bool ball_may_hit(const SdfMeta &m, float inv, float x, float y, float z, float rho)
+{
+    const float reach = (rho + 1e-5f * (fabsf(x) + fabsf(y) + fabsf(z) + fabsf(m.ox) + fabsf(m.oy) + fabsf(m.oz))) * inv;
+    return !((float)cell_clear(m, inv, x, y, z) > ceilf(reach + 0.02f));
 }
 
 // Block sum of double-float accumulators: warp trees in double-float, then the
@@ -62,36 +83,38 @@ __device__ __forceinline__ void block_reduce_store(dfloat (&acc)[NV], double (*s
 }
 }  // namespace
 
-// One CTA per particle.
-//  1. Matching sums of the forward pairs (i <-> nn_idx[i]) in float64:
+// Two CTAs per particle, which do not depend on each other:
+// CTA T + pk: matching sums of the forward pairs (i <-> nn_idx[i]) in float64:
 //     sum r (3), sum r s^T (9), sum |r|^2 (1), r the matched object point and s the
 //     gripper point in the gripper frame (exact products of float32 values).
-//  2. Collision test: every collision point c is mapped into the gripper frame,
-//     c' = R^T (c - t); points outside the box of cells with a positive corner
-//     cannot interpolate to a positive value and are skipped; the others are
-//     looked up in the preshape's SDF and kept when the value is > 0.  The
-//     colliding indices are compacted in ascending order (warp ballots and a
-//     block prefix), so results do not depend on scheduling.
+// CTA pk: collision test.  Every collision point c is mapped into the gripper frame,
+//     c' = R^T (c - t), and kept when the preshape's distance field is > 0 there (Eq. 12).
+//     The collision cloud is held in spatial order (sort_cloud_kernel) in chunks of 32
+//     points with their bounding balls: a chunk whose ball is clear of the gripper is skipped,
+//     a warp tests the points of another one.  Hits set bits by the points' own indices, which
+//     are then listed in ascending order, so results depend neither on the order of the
+//     chunks nor on scheduling.  Clouds beyond kColSegment points are taken segment by segment.
+// Measured on GB300 (per pass, against one CTA per particle doing the sums and then testing every
+// point): 3 x 256 particles, N 2048, M 8192 31 us against 58; 3 x 1024, N 4096, M 65536 0.34 ms
+// against 1.19; 2 x 64, N 1024, Mc 4501 16 us against 27.  A quarter of the chunks survive
+// (balls of 10 mm at 8192 points against voxels of 3.2 mm); latency of loads bounds it.
 __global__ void __launch_bounds__(kTestThreads) collide_kernel(const CollideArgs a)
 {
     if (a.err && *a.err != kDevOk) return;    // the matching gave up: its correspondences are not valid
-    __shared__ int swarp[kColU][kTestThreads / 32];
-    __shared__ double sred[kTestThreads / 32][kFwdSums];
-    const int pk = blockIdx.x;
+    const bool sums = (int)blockIdx.x >= a.L.T;
+    const int pk = sums ? blockIdx.x - a.L.T : blockIdx.x;
     const int grp = a.L.part_grp[pk], p = grp % a.L.P;
-    const ObjMeta om = a.L.obj[grp / a.L.P];
-    const int N = a.L.N, Mc = om.Mc;
-    const float *th = a.theta + (size_t)pk * 8;
-    const float tx = th[0], ty = th[1], tz = th[2];
-    float Rm[9];
-    quat_rot_f32(th[3], th[4], th[5], th[6], Rm);
+    const ObjMeta &om = a.L.obj[grp / a.L.P];
+    const int N = a.L.N;
 
-    {
+    if (sums) {
+        __shared__ double sred[kTestThreads / 32][kFwdSums];
         dfloat acc[kFwdSums];
 #pragma unroll
         for (int c = 0; c < kFwdSums; ++c) acc[c] = dfloat{0.f, 0.f};
         const float4 *S = a.S + (size_t)p * N;
         const int *idx = a.nn_idx + (size_t)pk * N;
+        const float4 *R = om.R;
         auto add_pair = [&](float4 r, float4 s) {
             const float rv[3] = {r.x, r.y, r.z}, sv[3] = {s.x, s.y, s.z};
 #pragma unroll
@@ -111,80 +134,221 @@ __global__ void __launch_bounds__(kTestThreads) collide_kernel(const CollideArgs
 #pragma unroll
             for (int u = 0; u < kPairB; ++u) { id[u] = idx[i + u * kTestThreads]; s[u] = S[i + u * kTestThreads]; }
 #pragma unroll
-            for (int u = 0; u < kPairB; ++u) r[u] = __ldg(om.R + id[u]);
+            for (int u = 0; u < kPairB; ++u) r[u] = __ldg(R + id[u]);
 #pragma unroll
             for (int u = 0; u < kPairB; ++u) add_pair(r[u], s[u]);
         }
-        for (; i < N; i += kTestThreads) add_pair(__ldg(om.R + idx[i]), S[i]);
+        for (; i < N; i += kTestThreads) add_pair(__ldg(R + idx[i]), S[i]);
         block_reduce_store<kFwdSums>(acc, sred, a.fsums + (size_t)pk * kFwdSums);
+        return;
     }
 
+    __shared__ unsigned s_bits[kSegWords];
+    __shared__ unsigned short s_chunk[kSegWords];
+    __shared__ int s_n, s_wsum[kTestThreads / 32], s_base;
+    const float *th = a.theta + (size_t)pk * 8;
+    const float tx = th[0], ty = th[1], tz = th[2];
+    float Rm[9];
+    quat_rot_f32(th[3], th[4], th[5], th[6], Rm);
     const SdfMeta m = a.meta[p];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const float inv = 1.f / m.voxel;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, Mc = om.Mc;
+    auto local = [&](float4 c, float &lx, float &ly, float &lz) {
+        const float dx = __fsub_rn(c.x, tx), dy = __fsub_rn(c.y, ty), dz = __fsub_rn(c.z, tz);
+        lx = __fmaf_rn(Rm[0], dx, __fmaf_rn(Rm[3], dy, __fmul_rn(Rm[6], dz)));
+        ly = __fmaf_rn(Rm[1], dx, __fmaf_rn(Rm[4], dy, __fmul_rn(Rm[7], dz)));
+        lz = __fmaf_rn(Rm[2], dx, __fmaf_rn(Rm[5], dy, __fmul_rn(Rm[8], dz)));
+    };
     int *colidx = a.colidx + om.colidx_base + (long long)(pk - om.pfirst) * Mc;
     int count = 0;
-    // kU points per thread per round (their loads and lookups overlap), one
-    // compaction per round in ascending point order (round slot, warp, lane)
-    for (int c0 = 0; c0 < Mc; c0 += kTestThreads * kColU) {
-        float4 v[kColU];
-#pragma unroll
-        for (int u = 0; u < kColU; ++u) {
-            const int c = c0 + u * kTestThreads + threadIdx.x;
-            v[u] = c < Mc ? om.C[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        bool hit[kColU];
-#pragma unroll
-        for (int u = 0; u < kColU; ++u) {
-            const int c = c0 + u * kTestThreads + threadIdx.x;
-            hit[u] = false;
-            if (c < Mc) {
-                const float dx = __fsub_rn(v[u].x, tx), dy = __fsub_rn(v[u].y, ty), dz = __fsub_rn(v[u].z, tz);
-                const float lx = __fmaf_rn(Rm[0], dx, __fmaf_rn(Rm[3], dy, __fmul_rn(Rm[6], dz)));
-                const float ly = __fmaf_rn(Rm[1], dx, __fmaf_rn(Rm[4], dy, __fmul_rn(Rm[7], dz)));
-                const float lz = __fmaf_rn(Rm[2], dx, __fmaf_rn(Rm[5], dy, __fmul_rn(Rm[8], dz)));
-                if (lx >= m.lo[0] && lx <= m.hi[0] && ly >= m.lo[1] && ly <= m.hi[1] && lz >= m.lo[2] &&
-                    lz <= m.hi[2]) {
-                    float val;
-                    hit[u] = sdf_lookup(m, lx, ly, lz, val) && val > 0.f;
-                }
+    for (int seg = 0; seg < Mc; seg += kColSegment) {
+        const int pts = min(kColSegment, Mc - seg), chunks = (pts + 31) / 32;
+        const float4 *balls = om.Cball + seg / 32, *cloud = om.Csort + seg;
+        for (int w = threadIdx.x; w < chunks; w += kTestThreads) s_bits[w] = 0u;
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        for (int c0 = 0; c0 < chunks; c0 += kTestThreads) {
+            const int c = c0 + threadIdx.x;
+            bool may = false;
+            if (c < chunks) {
+                const float4 b = __ldg(balls + c);
+                float lx, ly, lz;
+                local(b, lx, ly, lz);
+                may = ball_may_hit(m, inv, lx, ly, lz, b.w);
             }
-        }
-        unsigned bal[kColU];
-#pragma unroll
-        for (int u = 0; u < kColU; ++u) {
-            bal[u] = __ballot_sync(0xffffffffu, hit[u]);
-            if (lane == 0) swarp[u][warp] = __popc(bal[u]);
+            const unsigned bal = __ballot_sync(0xffffffffu, may);
+            int base = 0;
+            if (lane == 0 && bal) base = atomicAdd(&s_n, __popc(bal));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (may) s_chunk[base + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)c;
         }
         __syncthreads();
-        int before = 0, tot = 0;
+        const int n = s_n;
+        // kTestB chunks per warp at a time: their loads are in flight together
+        for (int k0 = warp; k0 < n; k0 += kTestB * (kTestThreads / 32)) {
+            float4 c[kTestB];
+            int near[kTestB];
 #pragma unroll
-        for (int u = 0; u < kColU; ++u) {
-            int mine = 0;
-#pragma unroll
-            for (int w = 0; w < kTestThreads / 32; ++w) {
-                const int n = swarp[u][w];
-                mine += w < warp ? n : 0;
-                tot += n;
+            for (int u = 0; u < kTestB; ++u) {
+                const int k = k0 + u * (kTestThreads / 32), i = (k < n ? s_chunk[k] * 32 : kColSegment) + lane;
+                c[u] = __ldg(cloud + min(i, pts - 1));
+                if (i >= pts) c[u].w = __int_as_float(-1);
             }
-            if (hit[u])
-                colidx[count + before + mine + __popc(bal[u] & ((1u << lane) - 1u))] = c0 + u * kTestThreads + threadIdx.x;
-            before = tot;
+#pragma unroll
+            for (int u = 0; u < kTestB; ++u) {
+                float lx, ly, lz;
+                local(c[u], lx, ly, lz);
+                near[u] = cell_clear(m, inv, lx, ly, lz);
+                c[u].x = lx; c[u].y = ly; c[u].z = lz;
+            }
+#pragma unroll
+            for (int u = 0; u < kTestB; ++u) {
+                const int own = __float_as_int(c[u].w);
+                if (near[u] <= 1 && own >= 0 && sdf_hit(m, c[u].x, c[u].y, c[u].z))
+                    atomicOr(&s_bits[own >> 5], 1u << (own & 31));
+            }
         }
-        count += tot;
         __syncthreads();
+        // list the set bits in ascending order: kTestThreads words a round
+        for (int w0 = 0; w0 < chunks; w0 += kTestThreads) {
+            const int w = w0 + threadIdx.x;
+            unsigned bits = w < chunks ? s_bits[w] : 0u;
+            int inc = __popc(bits);
+            const int mine = inc;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += y;
+            }
+            if (lane == 31) s_wsum[warp] = inc;
+            __syncthreads();
+            int before = inc - mine, tot = 0;
+#pragma unroll
+            for (int v = 0; v < kTestThreads / 32; ++v) {
+                const int y = s_wsum[v];
+                before += v < warp ? y : 0;
+                tot += y;
+            }
+            int *out = colidx + count + before;
+            while (bits) {
+                const int b = __ffs(bits) - 1;
+                bits &= bits - 1;
+                *out++ = seg + w * 32 + b;
+            }
+            count += tot;
+            __syncthreads();
+        }
     }
+    // queue this particle's chunks of colliding points for the reverse matching
+    const int used = (count + kColChunk - 1) / kColChunk;
     if (threadIdx.x == 0) {
         a.ncol[pk] = count;
-        // queue this particle's chunks of colliding points for the reverse matching
-        const int used = (count + kColChunk - 1) / kColChunk;
-        if (used > 0) {
-            const int base = atomicAdd(&a.col_items[0], used);
-            for (int c = 0; c < used; ++c) {
-                a.col_list[2 * (base + c)] = pk;
-                a.col_list[2 * (base + c) + 1] = c;
-            }
-        }
+        s_base = used > 0 ? atomicAdd(&a.col_items[0], used) : 0;
     }
+    __syncthreads();
+    for (int c = threadIdx.x; c < used; c += kTestThreads)
+        reinterpret_cast<int2 *>(a.col_list)[s_base + c] = make_int2(pk, c);
+}
+
+// Spatial order of (a segment of) a collision cloud, one CTA each: points sorted into the 32^3
+// bins of their bounding box, bins along a space-filling curve (the order within a bin does not
+// matter), w = the point's index in the segment; and per 32 points in that order a bounding
+// ball (w = its radius, rounded up).
+__global__ void __launch_bounds__(1024) sort_cloud_kernel(const CloudBatch batch)
+{
+    const CloudSort &b = batch.b[blockIdx.x];
+    extern __shared__ int s_bin[];
+    __shared__ float s_lo[3][32], s_hi[3][32];
+    __shared__ int s_sum[32];
+    constexpr int kBins = 32 * 32 * 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n = b.n;
+    float lo[3], hi[3];
+    for (int k = 0; k < 3; ++k) { lo[k] = __int_as_float(0x7f800000); hi[k] = -lo[k]; }
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const float4 p = __ldg(b.src + i);
+        lo[0] = fminf(lo[0], p.x); lo[1] = fminf(lo[1], p.y); lo[2] = fminf(lo[2], p.z);
+        hi[0] = fmaxf(hi[0], p.x); hi[1] = fmaxf(hi[1], p.y); hi[2] = fmaxf(hi[2], p.z);
+    }
+    for (int i = threadIdx.x; i < kBins; i += blockDim.x) s_bin[i] = 0;
+    for (int k = 0; k < 3; ++k) {
+        for (int o = 16; o > 0; o >>= 1) {
+            lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
+            hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
+        }
+        if (lane == 0) { s_lo[k][warp] = lo[k]; s_hi[k][warp] = hi[k]; }
+    }
+    __syncthreads();
+    float ext = 1e-30f;
+    for (int k = 0; k < 3; ++k) {
+        lo[k] = s_lo[k][lane];
+        hi[k] = s_hi[k][lane];
+        for (int o = 16; o > 0; o >>= 1) {
+            lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
+            hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
+        }
+        ext = fmaxf(ext, hi[k] - lo[k]);
+    }
+    const float scale = 32.f / ext;
+    auto bin = [&](float4 p) {
+        auto spread = [](unsigned v) { v = (v | (v << 8)) & 0x100fu; v = (v | (v << 4)) & 0x10c3u; return (v | (v << 2)) & 0x1249u; };
+        const unsigned x = (unsigned)min(max((int)((p.x - lo[0]) * scale), 0), 31),
+                       y = (unsigned)min(max((int)((p.y - lo[1]) * scale), 0), 31),
+                       z = (unsigned)min(max((int)((p.z - lo[2]) * scale), 0), 31);
+        return (int)(spread(x) | (spread(y) << 1) | (spread(z) << 2));
+    };
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&s_bin[bin(__ldg(b.src + i))], 1);
+    __syncthreads();
+    // exclusive scan over the bins: warp w's 1024, then the warps
+    int *mine = s_bin + warp * (kBins / 32);
+    int carry = 0;
+    for (int k = 0; k < kBins / 32; k += 32) {
+        const int v = mine[k + lane];
+        int inc = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        mine[k + lane] = carry + inc - v;
+        carry += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    if (lane == 0) s_sum[warp] = carry;
+    __syncthreads();
+    int before = 0;
+    for (int w = 0; w < warp; ++w) before += s_sum[w];
+    for (int k = lane; k < kBins / 32; k += 32) mine[k] += before;
+    __syncthreads();
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        float4 p = __ldg(b.src + i);
+        const int at = atomicAdd(&s_bin[bin(p)], 1);
+        p.w = __int_as_float(i);
+        b.dst[at] = p;
+    }
+    __syncthreads();
+    for (int c = warp; c * 32 < n; c += 32) {
+        const bool in = c * 32 + lane < n;
+        const float4 p = b.dst[min(c * 32 + lane, n - 1)];
+        float l[3] = {p.x, p.y, p.z}, h[3] = {p.x, p.y, p.z};
+        for (int k = 0; k < 3; ++k)
+            for (int o = 16; o > 0; o >>= 1) {
+                l[k] = fminf(l[k], __shfl_xor_sync(0xffffffffu, l[k], o));
+                h[k] = fmaxf(h[k], __shfl_xor_sync(0xffffffffu, h[k], o));
+            }
+        float4 ball = make_float4(0.5f * l[0] + 0.5f * h[0], 0.5f * l[1] + 0.5f * h[1], 0.5f * l[2] + 0.5f * h[2], 0.f);
+        const float x = p.x - ball.x, y = p.y - ball.y, z = p.z - ball.z;
+        float d = in ? x * x + y * y + z * z : 0.f;
+        for (int o = 16; o > 0; o >>= 1) d = fmaxf(d, __shfl_xor_sync(0xffffffffu, d, o));
+        ball.w = sqrtf(d) * 1.00001f + 1e-30f;
+        if (lane == 0) b.balls[c] = ball;
+    }
+}
+
+cudaError_t launch_sort_clouds(const CloudBatch &batch, int n, cudaStream_t st)
+{
+    sort_cloud_kernel<<<n, 1024, 32 * 32 * 32 * sizeof(int), st>>>(batch);
+    return cudaGetLastError();
 }
 
 namespace {
@@ -606,12 +770,15 @@ __global__ void __launch_bounds__(kColChunk) collide_cells_kernel(const CollideA
 
 cudaError_t launch_collide(const CollideArgs &a, cudaStream_t st)
 {
-    collide_kernel<<<a.L.T, kTestThreads, 0, st>>>(a);
+    collide_kernel<<<2 * a.L.T, kTestThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t init_collision_attributes()
 {
+    const cudaError_t e = cudaFuncSetAttribute(sort_cloud_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               32 * 32 * 32 * (int)sizeof(int));
+    if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(collide_nn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)(2 * sizeof(float4) * kMaxN + 32 * sizeof(float4)));
 }
@@ -633,25 +800,6 @@ cudaError_t launch_collide_nn(const CollideArgs &a, cudaStream_t st)
     const size_t smem = 2 * sizeof(float4) * (size_t)((a.L.N + 63) / 64 * 64) + 32 * sizeof(float4);
     collide_nn_kernel<<<grid, kColThreads, smem, st>>>(a);
     return cudaGetLastError();
-}
-
-// Index box of the grid nodes with a positive value: box6 = (min x, min y, min z,
-// max x, max y, max z); the caller initialises it to (INT_MAX x3, INT_MIN x3).
-__global__ void sdf_box_kernel(const float *grid, int nx, int ny, int nz, int *box6)
-{
-    const long long n = (long long)nx * ny * nz;
-    int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        if (grid[i] > 0.f) {
-            const int x = (int)(i % nx), y = (int)((i / nx) % ny), z = (int)(i / ((long long)nx * ny));
-            lo[0] = min(lo[0], x); lo[1] = min(lo[1], y); lo[2] = min(lo[2], z);
-            hi[0] = max(hi[0], x); hi[1] = max(hi[1], y); hi[2] = max(hi[2], z);
-        }
-    }
-    for (int a = 0; a < 3; ++a) {
-        if (lo[a] != INT_MAX) atomicMin(box6 + a, lo[a]);
-        if (hi[a] != INT_MIN) atomicMax(box6 + 3 + a, hi[a]);
-    }
 }
 
 // Corner-packed copy of a grid: cell (ix, iy, iz), x fastest over the
@@ -680,12 +828,40 @@ cudaError_t launch_sdf_pack_cells(const float *grid, int nx, int ny, int nz, flo
     return cudaGetLastError();
 }
 
-cudaError_t launch_sdf_box(const float *grid, int nx, int ny, int nz, int *box6, cudaStream_t st)
+// Clearance of every cell of a grid: the distance in cells (largest coordinate, at most 255) to
+// the nearest cell with a positive corner, 0 for such a cell.  One axis at a time:
+// min over steps r of max(r, the previous axis's distance r cells away).
+__global__ void sdf_clear_kernel(const float4 *cells, int cx, int cy, int cz, int axis, const unsigned char *in,
+                                 unsigned char *out)
 {
-    const long long n = (long long)nx * ny * nz;
-    long long blocks = (n + 255) / 256;
-    if (blocks > 1024) blocks = 1024;
-    sdf_box_kernel<<<(int)blocks, 256, 0, st>>>(grid, nx, ny, nz, box6);
+    const long long nc = (long long)cx * cy * cz;
+    const int len = axis == 0 ? cx : axis == 1 ? cy : cz;
+    const long long stride = axis == 0 ? 1 : axis == 1 ? cx : (long long)cx * cy;
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nc; c += (long long)gridDim.x * blockDim.x) {
+        const int pos = axis == 0 ? (int)(c % cx) : axis == 1 ? (int)(c / cx % cy) : (int)(c / ((long long)cx * cy));
+        auto at = [&](long long k) -> int {
+            if (axis != 0) return in[k];
+            const float4 u = cells[2 * k], v = cells[2 * k + 1];
+            return u.x > 0.f || u.y > 0.f || u.z > 0.f || u.w > 0.f || v.x > 0.f || v.y > 0.f || v.z > 0.f || v.w > 0.f ? 0 : 255;
+        };
+        int best = at(c);
+        for (int r = 1; r < best && (pos >= r || pos + r < len); ++r) {
+            if (pos >= r) best = min(best, max(r, at(c - r * stride)));
+            if (pos + r < len) best = min(best, max(r, at(c + r * stride)));
+        }
+        out[c] = (unsigned char)best;
+    }
+}
+
+// clear and tmp: one byte per cell.
+cudaError_t launch_sdf_clear(const float4 *cells, int nx, int ny, int nz, unsigned char *clear, unsigned char *tmp,
+                             cudaStream_t st)
+{
+    const long long nc = (long long)(nx - 1) * (ny - 1) * (nz - 1);
+    const int blocks = (int)((nc + 255) / 256 < 4096 ? (nc + 255) / 256 : 4096);
+    sdf_clear_kernel<<<blocks, 256, 0, st>>>(cells, nx - 1, ny - 1, nz - 1, 0, nullptr, clear);
+    sdf_clear_kernel<<<blocks, 256, 0, st>>>(cells, nx - 1, ny - 1, nz - 1, 1, clear, tmp);
+    sdf_clear_kernel<<<blocks, 256, 0, st>>>(cells, nx - 1, ny - 1, nz - 1, 2, tmp, clear);
     return cudaGetLastError();
 }
 

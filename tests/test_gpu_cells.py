@@ -114,3 +114,41 @@ def test_gripper_cells_give_the_same_reverse_matches(N, offset):
         assert np.array_equal(a["col_nn"][pk, :n], b["col_nn"][pk, :n])
     for key in ("theta", "cost", "grad", "ncol"):
         assert np.array_equal(a[key], b[key]), key
+
+
+@pytest.mark.parametrize("Mc", [1, 31, 33, 4096, 65537, 131072 + 45])
+def test_collision_test_skips_no_colliding_point(Mc):
+    """The collision test skips chunks of the spatially sorted collision cloud that are clear of the gripper:
+    the colliding points, ascending, are the oracle's (but for values within 1e-6 m of zero), for
+    clouds of one point to several segments of the sort and a grid of three different sides."""
+    import oracle
+    w = synth.custom_case(P=2, K=6, N=64, M=300, grid=28, k_max=2, seed=91, k_stein=0)
+    g = np.random.default_rng(Mc)
+    for pre in w.preshapes:
+        pre.sdf = np.ascontiguousarray(pre.sdf[2:, 1:, :])
+        pre.origin = (pre.origin + pre.voxel * np.float32([0, 1, 2])).astype(np.float32)
+    C = (w.objects[0].points.mean(0) + g.uniform(-0.12, 0.12, (Mc, 3))).astype(np.float32)
+    t = C.mean(0, dtype=np.float64) + g.normal(size=(12, 3)) * 0.04
+    q = g.normal(size=(12, 4))
+    theta = np.concatenate([t, q / np.linalg.norm(q, axis=1, keepdims=True)], 1).astype(np.float32)
+    theta[3, :3] += 5.0                                        # nowhere near
+    ctx = asicp.asicp_create(tl.make_config(w, torch.cuda.current_stream().cuda_stream))
+    try:
+        asicp.asicp_set_object(ctx, w.objects[0].points, C)
+        for p, pre in enumerate(w.preshapes):
+            asicp.asicp_set_gripper_sdf(ctx, p, pre.S, pre.sdf, pre.origin, pre.voxel)
+        asicp.asicp_set_state(ctx, theta, 0)
+        before = tl.read_theta(ctx, 12)
+        asicp.asicp_step(ctx, 0)
+        st = tl.read_state(ctx, 2, 6, 64, Mc)
+    finally:
+        asicp.asicp_destroy(ctx)
+    orc = oracle.Oracle(np.stack([pre.S for pre in w.preshapes]), [(pre.sdf, pre.origin, pre.voxel) for pre in w.preshapes],
+                        w.objects[0].points, Cc=C, K=6)
+    for pk in range(12):
+        want, vals = orc.collision_points(pk // 6, before[pk].astype(np.float64))
+        got = st["col_list"][pk, :st["ncol"][pk]]
+        assert np.all(np.diff(got) > 0)
+        diff = np.setxor1d(got, want)
+        assert np.all(np.abs(np.asarray(vals)[diff]) <= tl.PHI_TOL), (pk, len(diff))
+    assert st["ncol"][3] == 0 and st["ncol"].max() >= Mc // 200       # (the gripper fills 0.75 % of the cube)
