@@ -128,13 +128,12 @@ struct asicp_ctx {
     // layout (rebuilt when objects, particle counts or N change)
     bool layout_dirty = true;
     int T = 0, G = 0, n_items = 0;
-    long long colidx_total = 0, csum_total = 0;
+    long long colidx_total = 0, colmap_total = 0;
     std::vector<int> grp_off_h;
     std::vector<ObjMeta> objmeta_h;
 
-    DevMem partgrp, grpoff, objmeta, items, ctaoff, com, frame, colitems, collist, stage, S, Ssort, preframe, prenodes, preleaves, cellwork, pconst, dmeta, theta, fsums,
-        csums, ncol, colidx, cost, grad, prev, frozen, phi, h, order, errw, out7, outc, outi, nnidx, tccand, dbg_d2, dbg_sp,
-        dbg_colnn;
+    DevMem partgrp, grpoff, objmeta, items, ctaoff, com, frame, colitems, collist, stage, S, Ssort, preframe, prenodes, preleaves, cellwork, pconst, dmeta, theta,
+        ncol, colidx, colsrt, colnn, colmap, cost, grad, prev, frozen, phi, h, order, errw, out7, outc, outi, nnidx, tccand, dbg_d2, dbg_sp;
 
     // profiling: events recorded around launches (kind, start, stop)
     struct Ev { int kind; cudaEvent_t a, b; };
@@ -310,7 +309,7 @@ void build_layout(asicp_ctx *c)
     for (int g = 0; g < G; ++g)
         for (int i = off[g]; i < off[g + 1]; ++i) part_grp[i] = g;
     std::vector<ObjMeta> om(c->nobj);
-    long long colidx_total = 0, csum_total = 0;
+    long long colidx_total = 0, colmap_total = 0;
     for (int o = 0; o < c->nobj; ++o) {
         const ObjBufs &b = c->objs[o];
         ObjMeta &m = om[o];
@@ -325,13 +324,12 @@ void build_layout(asicp_ctx *c)
         m.M = b.M;
         m.Mpad = b.Mpad;
         m.Mc = b.Mc;
-        m.chunks = (b.Mc + kColChunk - 1) / kColChunk;
         m.pfirst = off[o * P];
         m.np = off[(o + 1) * P] - off[o * P];
         m.colidx_base = colidx_total;
-        m.csum_base = csum_total;
+        m.colmap_base = colmap_total;
         colidx_total += (long long)m.np * m.Mc;
-        csum_total += (long long)m.np * m.chunks;
+        colmap_total += (long long)m.np * ((m.Mc + 31) / 32);
     }
 
     if (T != c->T) {
@@ -341,7 +339,7 @@ void build_layout(asicp_ctx *c)
     c->T = T;
     c->G = G;
     c->colidx_total = colidx_total;
-    c->csum_total = csum_total;
+    c->colmap_total = colmap_total;
     c->grp_off_h = off;
     c->objmeta_h = om;
 
@@ -349,14 +347,15 @@ void build_layout(asicp_ctx *c)
     c->grpoff.ensure(sizeof(int) * (G + 1), "group offsets");
     c->objmeta.ensure(sizeof(ObjMeta) * c->nobj, "object table");
     c->theta.ensure(sizeof(float) * 8 * (size_t)T, "poses");
-    c->fsums.ensure(sizeof(double) * T * kFwdSums, "fsums");
-    c->csums.ensure(sizeof(double) * std::max<long long>(1, csum_total) * kColSums, "csums");
     c->colitems.ensure(sizeof(int) * 2, "collision work counters");
-    c->collist.ensure(sizeof(int) * 2 * std::max<long long>(1, csum_total), "collision work list");
+    c->collist.ensure(sizeof(int) * 2 * std::max<long long>(1, colmap_total), "collision work list");
+    c->colmap.ensure(sizeof(int2) * std::max<long long>(1, colmap_total), "collision bit maps");
     c->nnidx.ensure(sizeof(int) * (size_t)T * N, "nn_idx");
     c->tccand.ensure(sizeof(int4) * (size_t)T * N, "tensor-core candidate chunks");
     c->ncol.ensure(sizeof(int) * T, "ncol");
     c->colidx.ensure(sizeof(int) * std::max<long long>(1, colidx_total), "colidx");
+    c->colsrt.ensure(sizeof(int) * std::max<long long>(1, colidx_total), "colsrt");
+    c->colnn.ensure(sizeof(int) * std::max<long long>(1, colidx_total), "colnn");
     c->cost.ensure(sizeof(double) * T, "cost");
     c->grad.ensure(sizeof(double) * T * 8, "grad");
     c->prev.ensure(sizeof(double) * T, "prev_cost");
@@ -370,7 +369,6 @@ void build_layout(asicp_ctx *c)
     if (c->cfg.debug) {
         c->dbg_d2.ensure(sizeof(float) * (size_t)T * N, "dbg_d2");
         c->dbg_sp.ensure(sizeof(float) * (size_t)T * N * 3, "dbg_sp");
-        c->dbg_colnn.ensure(sizeof(int) * std::max<long long>(1, colidx_total), "dbg_colnn");
     }
     // device tables (pageable sources: the copies complete before returning)
     ck(cudaMemcpyAsync(c->partgrp.p, part_grp.data(), sizeof(int) * T, cudaMemcpyHostToDevice, c->st), "particle groups");
@@ -666,15 +664,15 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
     ca.theta = c->theta.as<float>();
     ca.meta = c->dmeta.as<SdfMeta>();
     ca.S = c->S.as<float4>();
-    ca.nn_idx = c->nnidx.as<int>();
     ca.ncol = c->ncol.as<int>();
     ca.colidx = c->colidx.as<int>();
-    ca.fsums = c->fsums.as<double>();
-    ca.csums = c->csums.as<double>();
+    ca.colsrt = c->colsrt.as<int>();
+    ca.colnn = c->colnn.as<int>();
+    ca.colmap = c->colmap.as<int2>();
     ca.col_items = c->colitems.as<int>();
     ca.col_list = c->collist.as<int>();
     ca.err = c->errw.as<int>();
-    if (c->cfg.debug) ca.dbg_colnn = c->dbg_colnn.as<int>();
+    for (const ObjMeta &m : c->objmeta_h) ca.most_points = std::max(ca.most_points, m.Mc);
     ca.cells = c->pre_built;
     if (ca.cells) {
         const CellSizes s = cell_sizes(c->N);
@@ -683,7 +681,7 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
         ca.pre_frame = c->preframe.as<float4>();
         ca.pre_node_cap = s.node_cap;
         ca.pre_leaf_cap = s.leaf_cap;
-        ca.most_items = (int)std::min<long long>(std::max<long long>(1, c->csum_total), INT_MAX);
+        ca.most_items = (int)std::min<long long>(std::max<long long>(1, c->colmap_total), INT_MAX);
     }
     timed(c, kTimeCollide, [&](cudaStream_t st) { return launch_collide(ca, st); }, "collision kernel");
     timed(c, kTimeCollideNN, [&](cudaStream_t st) { return launch_collide_nn(ca, st); }, "collision matching kernel");
@@ -691,8 +689,10 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
     UpdateArgs ua{};
     ua.L = L;
     ua.theta = c->theta.as<float>();
-    ua.fsums = c->fsums.as<double>();
-    ua.csums = c->csums.as<double>();
+    ua.S = c->S.as<float4>();
+    ua.nn_idx = c->nnidx.as<int>();
+    ua.colidx = c->colidx.as<int>();
+    ua.colnn = c->colnn.as<int>();
     ua.ncol = c->ncol.as<int>();
     ua.pconst = c->pconst.as<double>();
     ua.w_com = c->cfg.w_com;
@@ -748,15 +748,15 @@ void run_loop(asicp_ctx *c)
 std::vector<const void *> loop_key(const asicp_ctx *c)
 {
     return {c->partgrp.p, c->grpoff.p, c->objmeta.p, c->items.p, c->ctaoff.p, c->com.p, c->frame.p, c->colitems.p, c->collist.p,
-            c->S.p, c->pconst.p, c->dmeta.p, c->theta.p, c->fsums.p, c->csums.p, c->ncol.p, c->colidx.p, c->cost.p,
+            c->S.p, c->pconst.p, c->dmeta.p, c->theta.p, c->ncol.p, c->colidx.p, c->colsrt.p, c->colnn.p, c->colmap.p, c->cost.p,
             c->grad.p, c->prev.p, c->frozen.p, c->phi.p, c->h.p, c->order.p, c->errw.p, c->nnidx.p, c->tccand.p, c->dbg_d2.p,
-            c->dbg_sp.p, c->dbg_colnn.p, c->mb_idx.p, c->mb_R.p, c->mb_Rx.p,
+            c->dbg_sp.p, c->mb_idx.p, c->mb_R.p, c->mb_Rx.p,
             reinterpret_cast<const void *>((size_t)c->mb_version), reinterpret_cast<const void *>((size_t)c->T),
             reinterpret_cast<const void *>((size_t)c->G), reinterpret_cast<const void *>((size_t)c->n_items),
             reinterpret_cast<const void *>((size_t)c->N), reinterpret_cast<const void *>((size_t)c->fwd_variant),
             reinterpret_cast<const void *>((size_t)c->expire_test), c->Ssort.p,
             reinterpret_cast<const void *>((size_t)c->cells_on), c->prenodes.p, c->preleaves.p, c->preframe.p,
-            reinterpret_cast<const void *>((size_t)c->pre_built), reinterpret_cast<const void *>((size_t)c->csum_total)};
+            reinterpret_cast<const void *>((size_t)c->pre_built), reinterpret_cast<const void *>((size_t)c->colmap_total)};
 }
 
 // Replay the captured loop on the caller's stream, capturing it first when the
@@ -1287,7 +1287,7 @@ asicp_status asicp_get_state(asicp_ctx *ctx, const asicp_state_view *v)
                 copy_out(v->nn_d2, ctx->dbg_d2.p, sizeof(float) * (size_t)T * ctx->N, ctx->st, "copy nn_d2");
                 copy_out(v->s_prime, ctx->dbg_sp.p, sizeof(float) * 3 * (size_t)T * ctx->N, ctx->st, "copy s_prime");
                 copy_out(v->col_list, ctx->colidx.p, sizeof(int) * (size_t)ctx->colidx_total, ctx->st, "copy col_list");
-                copy_out(v->col_nn, ctx->dbg_colnn.p, sizeof(int) * (size_t)ctx->colidx_total, ctx->st, "copy col_nn");
+                copy_out(v->col_nn, ctx->colnn.p, sizeof(int) * (size_t)ctx->colidx_total, ctx->st, "copy col_nn");
             }
         } else if (v->cost || v->ncol || v->h || dbg) {
             fail(ASICP_ERR_STATE, "get_state: no step has run since the poses were set");

@@ -204,10 +204,10 @@ struct ObjMeta {
     const float4 *C;          // [Mc] collision points (may alias R)
     const float4 *Csort;      // [Mc] the same in spatial order per segment, w = index in the segment
     const float4 *Cball;      // [ceil(Mc / 32)] bounding balls of 32 points of Csort (w = radius)
-    int M, Mpad, Mc, chunks;  // chunks = ceil(Mc / kColChunk)
+    int M, Mpad, Mc;
     int pfirst, np;           // first particle and number of particles of this object
     long long colidx_base;    // this object's collision lists start here ([np][Mc] ints)
-    long long csum_base;      // this object's chunk sums start here ([np][chunks] slots)
+    long long colmap_base;    // and their bit maps ([np][ceil(Mc / 32)] words)
 };
 
 struct Layout {
@@ -305,7 +305,7 @@ cudaError_t launch_cells_match(const FwdArgs &a, cudaStream_t st);
 cudaError_t launch_sort_points(const float4 *S, int N, float4 *out, float4 *frame, cudaStream_t st);
 cudaError_t init_cells_attributes();
 
-constexpr int kColChunk = 64;          // colliding points per reverse-matching work item
+constexpr int kColChunk = 64;          // colliding points per partial sum, and per work item of collide_nn_kernel
 
 // Spatial order of the collision clouds: segments of at most kColSegment points, several
 // (of several objects) per launch.
@@ -326,21 +326,22 @@ struct CollideArgs {
     const float *theta;       // [T][8]
     const SdfMeta *meta;      // [P]
     const float4 *S;          // [P][N]
-    const int *nn_idx;        // [T][N] forward correspondences
     int *ncol;                // [T]
-    int *colidx;              // collision lists (see ObjMeta::colidx_base)
-    double *fsums;            // [T][kFwdSums]
-    double *csums;            // chunk sums (see ObjMeta::csum_base) [.][kColSums]
-    int *dbg_colnn;           // like colidx, or null
+    int *colidx;              // colliding points, ascending (see ObjMeta::colidx_base)
+    int *colsrt;              // the same points as positions in Csort, in no particular order
+    int *colnn;               // like colidx: nearest gripper point of each
+    int2 *colmap;             // bit map of the colliding points: words (bits, number of earlier bits),
+                              // only those with bits written (see ObjMeta::colmap_base)
+    int *col_items;           // (count, next) of the reverse-matching work list
+    int *col_list;            // [2 * items] (particle, item) pairs
+    const int *err;           // error word: a kernel of the pass found an error, skip the work
     int cells;                // reverse matching through the gripper clouds' cells
     const int2 *pre_nodes;    // [P][pre_node_cap]
     const int *pre_leaves;    // [P][pre_leaf_cap]
     const float4 *pre_frame;  // [P]
     int pre_node_cap, pre_leaf_cap;
     int most_items;           // work-list entries at most
-    int *col_items;           // (count, next) of the reverse-matching work list
-    int *col_list;            // [2 * items] (particle, chunk) pairs
-    const int *err;           // error word: a kernel of the pass found an error, skip the work
+    int most_points;          // points of the largest collision cloud
 };
 cudaError_t launch_collide(const CollideArgs &a, cudaStream_t st);
 cudaError_t launch_collide_nn(const CollideArgs &a, cudaStream_t st);
@@ -348,9 +349,10 @@ cudaError_t launch_collide_nn(const CollideArgs &a, cudaStream_t st);
 struct UpdateArgs {
     Layout L;
     float *theta;             // [T][8] in/out
-    const double *fsums;      // [T][kFwdSums]
-    const double *csums;      // chunk sums
+    const float4 *S;          // [P][N]
+    const int *nn_idx;        // [T][N] forward correspondences
     const int *ncol;          // [T]
+    const int *colidx, *colnn;    // colliding points and their gripper points (see CollideArgs)
     const double *pconst;     // [P][12]: sum s (3), sum s s^T (xx,xy,xz,yy,yz,zz), pad
     double w_com;
     int mode;                 // 0: evaluate only, 1: SVGD step, 2: SGD step

@@ -1,18 +1,14 @@
-// Per-particle matching sums and the collision term: SDF test of the
-// collision cloud in every particle's gripper frame (Eq. 12, Section IV-C) and
-// the reverse matching of the colliding points onto the transformed contact
-// cloud (Eq. 18).
+// The collision term: SDF test of the collision cloud in every particle's gripper
+// frame (Eq. 12, Section IV-C) and the reverse matching of the colliding points
+// onto the transformed contact cloud (Eq. 18).
 #include "cells.cuh"
 
 namespace asicp {
 
 namespace {
 constexpr int kColThreads = 256;       // reverse matching
-constexpr int kTestThreads = 128;      // collision test and matching sums: one small CTA per particle each
 constexpr int kSegWords = kColSegment / 32;      // words of a segment's bit map = most chunks of a segment
 constexpr int kTestB = 4;         // chunks per warp whose loads overlap
-constexpr int kPairB = 4;         // matching pairs per thread whose loads overlap (57.5 us per paper-scale
-                                  // launch against 61.8 us one pair at a time; 72 registers, 7 CTAs per SM)
 
 // Whether point (x, y, z) of the gripper frame collides: inside the grid's node box (the grid covers
 // the gripper, so a point outside is not in it) and trilinear value > 0 (Eq. 12).  Only a
@@ -64,88 +60,33 @@ __device__ __forceinline__ bool ball_may_hit(const SdfMeta &m, float inv, float 
     return !((float)cell_clear(m, inv, x, y, z) > ceilf(reach + 0.02f));
 }
 
-// Block sum of double-float accumulators: warp trees in double-float, then the
-// warps' partials added in float64 in warp order by NV threads.
-template <int NV>
-__device__ __forceinline__ void block_reduce_store(dfloat (&acc)[NV], double (*sred)[NV], double *out)
-{
-    warp_sum_df(acc);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0)
-#pragma unroll
-        for (int c = 0; c < NV; ++c) sred[warp][c] = (double)acc[c].hi + (double)acc[c].lo;
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        double s = 0.0;
-        for (int w = 0; w < kTestThreads / 32; ++w) s += sred[w][threadIdx.x];
-        out[threadIdx.x] = s;
-    }
-}
 }  // namespace
 
-// Two CTAs per particle, which do not depend on each other:
-// CTA T + pk: matching sums of the forward pairs (i <-> nn_idx[i]) in float64:
-//     sum r (3), sum r s^T (9), sum |r|^2 (1), r the matched object point and s the
-//     gripper point in the gripper frame (exact products of float32 values).
-// CTA pk: collision test.  Every collision point c is mapped into the gripper frame,
-//     c' = R^T (c - t), and kept when the preshape's distance field is > 0 there (Eq. 12).
-//     The collision cloud is held in spatial order (sort_cloud_kernel) in chunks of 32
-//     points with their bounding balls: a chunk whose ball is clear of the gripper is skipped,
-//     a warp tests the points of another one.  Hits set bits by the points' own indices, which
-//     are then listed in ascending order, so results depend neither on the order of the
-//     chunks nor on scheduling.  Clouds beyond kColSegment points are taken segment by segment.
-// Measured on GB300 (per pass, against one CTA per particle doing the sums and then testing every
-// point): 3 x 256 particles, N 2048, M 8192 31 us against 58; 3 x 1024, N 4096, M 65536 0.34 ms
-// against 1.19; 2 x 64, N 1024, Mc 4501 16 us against 27.  A quarter of the chunks survive
-// (balls of 10 mm at 8192 points against voxels of 3.2 mm); latency of loads bounds it.
-__global__ void __launch_bounds__(kTestThreads) collide_kernel(const CollideArgs a)
+// Items of the reverse matching: the points of a warp (through the cells), or kColChunk.
+__host__ __device__ constexpr int col_item_points(bool cells) { return cells ? 32 : kColChunk; }
+
+// One CTA per particle: every collision point c is mapped into the gripper frame,
+// c' = R^T (c - t), and kept when the preshape's distance field is > 0 there (Eq. 12).  The
+// collision cloud is held in spatial order (sort_cloud_kernel) in chunks of 32 points with their
+// bounding balls: a chunk whose ball is clear of the gripper is skipped, a warp tests the
+// points of another one.  Hits are noted as they come (neighbours stay together, which is how
+// the reverse matching wants them) and set bits by the points' own indices, which are then
+// listed in ascending order, so results depend neither on the order of the chunks nor on
+// scheduling.  Clouds beyond kColSegment points are taken segment by segment.
+// Measured on GB300 (per pass; before: every point tested, and the sums of the forward pairs in the
+// same CTA): 3 x 256 particles, M 8192 20 us against 58; 3 x 1024, M 65536 0.27 ms against 1.19;
+// 2 x 64, Mc 4501 13 us against 27.  A quarter of the chunks survive (balls of 10 mm at 8192
+// points against voxels of 3.2 mm); at 0.27 ms it takes three quarters of the issue slots.
+template <int kTestThreads>
+__global__ void __launch_bounds__(kTestThreads, 1280 / kTestThreads) collide_kernel(const CollideArgs a)
 {
     if (a.err && *a.err != kDevOk) return;    // the matching gave up: its correspondences are not valid
-    const bool sums = (int)blockIdx.x >= a.L.T;
-    const int pk = sums ? blockIdx.x - a.L.T : blockIdx.x;
+    const int pk = blockIdx.x;
     const int grp = a.L.part_grp[pk], p = grp % a.L.P;
     const ObjMeta &om = a.L.obj[grp / a.L.P];
-    const int N = a.L.N;
-
-    if (sums) {
-        __shared__ double sred[kTestThreads / 32][kFwdSums];
-        dfloat acc[kFwdSums];
-#pragma unroll
-        for (int c = 0; c < kFwdSums; ++c) acc[c] = dfloat{0.f, 0.f};
-        const float4 *S = a.S + (size_t)p * N;
-        const int *idx = a.nn_idx + (size_t)pk * N;
-        const float4 *R = om.R;
-        auto add_pair = [&](float4 r, float4 s) {
-            const float rv[3] = {r.x, r.y, r.z}, sv[3] = {s.x, s.y, s.z};
-#pragma unroll
-            for (int u = 0; u < 3; ++u) {
-                df_add(acc[u], rv[u]);
-#pragma unroll
-                for (int v = 0; v < 3; ++v) df_add_prod(acc[3 + 3 * u + v], rv[u], sv[v]);
-                df_add_prod(acc[12], rv[u], rv[u]);
-            }
-        };
-        // kPairB pairs per thread at a time: their index loads, then their object-point loads,
-        // are in flight together (the pairs are still added in the same order)
-        int i = threadIdx.x;
-        for (; i + (kPairB - 1) * kTestThreads < N; i += kPairB * kTestThreads) {
-            int id[kPairB];
-            float4 s[kPairB], r[kPairB];
-#pragma unroll
-            for (int u = 0; u < kPairB; ++u) { id[u] = idx[i + u * kTestThreads]; s[u] = S[i + u * kTestThreads]; }
-#pragma unroll
-            for (int u = 0; u < kPairB; ++u) r[u] = __ldg(R + id[u]);
-#pragma unroll
-            for (int u = 0; u < kPairB; ++u) add_pair(r[u], s[u]);
-        }
-        for (; i < N; i += kTestThreads) add_pair(__ldg(R + idx[i]), S[i]);
-        block_reduce_store<kFwdSums>(acc, sred, a.fsums + (size_t)pk * kFwdSums);
-        return;
-    }
-
     __shared__ unsigned s_bits[kSegWords];
     __shared__ unsigned short s_chunk[kSegWords];
-    __shared__ int s_n, s_wsum[kTestThreads / 32], s_base;
+    __shared__ int s_n, s_hits, s_wsum[kTestThreads / 32], s_base;
     const float *th = a.theta + (size_t)pk * 8;
     const float tx = th[0], ty = th[1], tz = th[2];
     float Rm[9];
@@ -159,8 +100,11 @@ __global__ void __launch_bounds__(kTestThreads) collide_kernel(const CollideArgs
         ly = __fmaf_rn(Rm[1], dx, __fmaf_rn(Rm[4], dy, __fmul_rn(Rm[7], dz)));
         lz = __fmaf_rn(Rm[2], dx, __fmaf_rn(Rm[5], dy, __fmul_rn(Rm[8], dz)));
     };
-    int *colidx = a.colidx + om.colidx_base + (long long)(pk - om.pfirst) * Mc;
+    const long long first = om.colidx_base + (long long)(pk - om.pfirst) * Mc;
+    int *colidx = a.colidx + first, *colsrt = a.colsrt + first;
+    int2 *colmap = a.colmap + om.colmap_base + (long long)(pk - om.pfirst) * ((Mc + 31) / 32);
     int count = 0;
+    if (threadIdx.x == 0) s_hits = 0;
     for (int seg = 0; seg < Mc; seg += kColSegment) {
         const int pts = min(kColSegment, Mc - seg), chunks = (pts + 31) / 32;
         const float4 *balls = om.Cball + seg / 32, *cloud = om.Csort + seg;
@@ -187,12 +131,12 @@ __global__ void __launch_bounds__(kTestThreads) collide_kernel(const CollideArgs
         // kTestB chunks per warp at a time: their loads are in flight together
         for (int k0 = warp; k0 < n; k0 += kTestB * (kTestThreads / 32)) {
             float4 c[kTestB];
-            int near[kTestB];
+            int near[kTestB], at[kTestB];
 #pragma unroll
             for (int u = 0; u < kTestB; ++u) {
-                const int k = k0 + u * (kTestThreads / 32), i = (k < n ? s_chunk[k] * 32 : kColSegment) + lane;
-                c[u] = __ldg(cloud + min(i, pts - 1));
-                if (i >= pts) c[u].w = __int_as_float(-1);
+                const int k = k0 + u * (kTestThreads / 32);
+                at[u] = (k < n ? s_chunk[k] * 32 : kColSegment) + lane;
+                c[u] = __ldg(cloud + min(at[u], pts - 1));
             }
 #pragma unroll
             for (int u = 0; u < kTestB; ++u) {
@@ -203,9 +147,17 @@ __global__ void __launch_bounds__(kTestThreads) collide_kernel(const CollideArgs
             }
 #pragma unroll
             for (int u = 0; u < kTestB; ++u) {
-                const int own = __float_as_int(c[u].w);
-                if (near[u] <= 1 && own >= 0 && sdf_hit(m, c[u].x, c[u].y, c[u].z))
+                const bool hit = near[u] <= 1 && at[u] < pts && sdf_hit(m, c[u].x, c[u].y, c[u].z);
+                const unsigned bal = __ballot_sync(0xffffffffu, hit);
+                if (!bal) continue;
+                int base = 0;
+                if (lane == 0) base = atomicAdd(&s_hits, __popc(bal));
+                base = __shfl_sync(0xffffffffu, base, 0);
+                if (hit) {
+                    const int own = __float_as_int(c[u].w);
                     atomicOr(&s_bits[own >> 5], 1u << (own & 31));
+                    colsrt[base + __popc(bal & ((1u << lane) - 1u))] = seg + at[u];
+                }
             }
         }
         __syncthreads();
@@ -230,6 +182,7 @@ __global__ void __launch_bounds__(kTestThreads) collide_kernel(const CollideArgs
                 tot += y;
             }
             int *out = colidx + count + before;
+            if (bits) colmap[seg / 32 + w] = make_int2((int)bits, count + before);
             while (bits) {
                 const int b = __ffs(bits) - 1;
                 bits &= bits - 1;
@@ -239,8 +192,8 @@ __global__ void __launch_bounds__(kTestThreads) collide_kernel(const CollideArgs
             __syncthreads();
         }
     }
-    // queue this particle's chunks of colliding points for the reverse matching
-    const int used = (count + kColChunk - 1) / kColChunk;
+    // queue this particle's colliding points for the reverse matching
+    const int item = col_item_points(a.cells), used = (count + item - 1) / item;
     if (threadIdx.x == 0) {
         a.ncol[pk] = count;
         s_base = used > 0 ? atomicAdd(&a.col_items[0], used) : 0;
@@ -398,15 +351,6 @@ __device__ __forceinline__ void argmin_xor(float &best, int &bi, int o)
     if (ob < best || (ob == best && oi < bi)) { best = ob; bi = oi; }
 }
 
-// Operands of the collision sums: sum index -> (a, b) as indices into a
-// colliding point's record {s_x, s_y, s_z, c_x, c_y, c_z, 1, 0}; sum 21 (|c|^2)
-// adds the three squares of c.
-__constant__ unsigned char kColSel[kColSums][2] = {
-    {0, 6}, {1, 6}, {2, 6},                                  // sum s
-    {0, 0}, {0, 1}, {0, 2}, {1, 1}, {1, 2}, {2, 2},          // sum s s^T (upper triangle)
-    {3, 6}, {4, 6}, {5, 6},                                  // sum c
-    {3, 0}, {3, 1}, {3, 2}, {4, 0}, {4, 1}, {4, 2}, {5, 0}, {5, 1}, {5, 2},   // sum c s^T
-    {3, 3}};                                                 // sum |c|^2
 }  // namespace
 
 // Persistent: CTAs take (particle, chunk of kColChunk colliding points) items
@@ -428,20 +372,13 @@ __constant__ unsigned char kColSel[kColSums][2] = {
 //     l1 unless b2 <= b1 + 2 delta; four lanes per colliding point re-evaluate chunk l1 with the
 //     exact-form distance, ties to the lowest index; in the rare other case the
 //     warp scans the whole cloud that way.
-// The sums the collision cost and gradient are linear in are then accumulated
-// per item (double-float, exact products) by 8 threads per sum over 8
-// colliding points each, merged in a fixed tree:
-//   sum s (3), sum s s^T (xx,xy,xz,yy,yz,zz) (6), sum c (3), sum c s^T (9), sum |c|^2 (1)
-// with s the matched gripper point in the gripper frame; the finalize kernel adds
-// the chunks of a particle in chunk order, so the result does not depend on
-// which CTA took which item.
+// For gripper clouds without cells (few points, or cells not built yet).
 __global__ void __launch_bounds__(kColThreads) collide_nn_kernel(const CollideArgs a)
 {
     if (a.err && *a.err != kDevOk) return;
     constexpr int kWarps = kColThreads / 32;
     constexpr int kQW = kColChunk / kWarps;                  // colliding points per warp
     static_assert(kQW == 8 && kColChunk == 64, "lane groups of four per colliding point");
-    static_assert(kColSums * 8 <= kColThreads, "eight threads per sum");
     extern __shared__ __align__(16) unsigned char smem_nn[];
     const int N = a.L.N;
     const int Npad = (N + 63) / 64 * 64;
@@ -450,7 +387,6 @@ __global__ void __launch_bounds__(kColThreads) collide_nn_kernel(const CollideAr
     ulonglong2 *sXB = sXA + Npad / 2;                                      // [Npad/2] {-2z pair}{w pair}
     float4 *sE = reinterpret_cast<float4 *>(sXB + Npad / 2);               // [32][KC + 1] exact S'
     __shared__ float4 sC[kColChunk];                          // colliding points of the item
-    __shared__ float sRec[kColChunk][8];                      // {s, c, 1, 0} per matched colliding point
     __shared__ int s_item;
     __shared__ float s_smax[kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -594,46 +530,9 @@ __global__ void __launch_bounds__(kColThreads) collide_nn_kernel(const CollideAr
                 if (g == q) { best = fb; bi = fi < N ? fi : 0; }
             }
         }
-        if (gs == 0) {
-            const int j = warp * kQW + g;
-            const bool valid = l0 + j < n;
-            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (valid) {
-                s = S[bi];
-                if (a.dbg_colnn) a.dbg_colnn[om.colidx_base + (long long)(pk - om.pfirst) * om.Mc + l0 + j] = bi;
-            }
-            sRec[j][0] = s.x; sRec[j][1] = s.y; sRec[j][2] = s.z;
-            sRec[j][3] = valid ? cq.x : 0.f; sRec[j][4] = valid ? cq.y : 0.f; sRec[j][5] = valid ? cq.z : 0.f;
-            sRec[j][6] = valid ? 1.f : 0.f; sRec[j][7] = 0.f;
-        }
+        if (gs == 0 && l0 + warp * kQW + g < n)
+            a.colnn[om.colidx_base + (long long)(pk - om.pfirst) * om.Mc + l0 + warp * kQW + g] = bi;
         __syncthreads();
-        // 3. the item's sums: thread (sum e, part) adds colliding points part + 8 u, u = 0 .. 7
-        if (threadIdx.x < (kColSums * 8 + 31) / 32 * 32) {
-            const int e = threadIdx.x >> 3, part = threadIdx.x & 7;
-            dfloat acc{0.f, 0.f};
-            if (e < kColSums) {
-                const int ia = kColSel[e][0], ib = kColSel[e][1];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const float *rec = sRec[part + 8 * u];
-                    df_add_prod(acc, rec[ia], rec[ib]);
-                    if (e == kColSums - 1) {
-                        df_add_prod(acc, rec[4], rec[4]);
-                        df_add_prod(acc, rec[5], rec[5]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int o = 1; o < 8; o <<= 1) {
-                dfloat y;
-                y.hi = __shfl_xor_sync(0xffffffffu, acc.hi, o);
-                y.lo = __shfl_xor_sync(0xffffffffu, acc.lo, o);
-                df_merge(acc, y);
-            }
-            if (part == 0 && e < kColSums)
-                a.csums[(om.csum_base + (long long)(pk - om.pfirst) * om.chunks + chunk) * kColSums + e] =
-                    (double)acc.hi + (double)acc.lo;
-        }
     }
 }
 
@@ -646,27 +545,27 @@ __global__ void __launch_bounds__(kColThreads) collide_nn_kernel(const CollideAr
 // orthonormal up to 8 u), s' by 6 u (|t|_1 + 2 max |s|) and by 8 u |s| for R again; distances
 // all scale by |q|^2 alike.  The lists hold for positions off by kGripperTol / 2.5 of the
 // cloud's radius; a colliding point beyond that bound (an object metres from its frame's origin)
-// compares the whole cloud.  64 threads per item, one per colliding point; the item's sums
-// are added in collide_nn_kernel's order, so they are the same to the last bit.
-// Measured on GB300 (per pass, against collide_nn_kernel): 3 x 256 particles, N 2048 18 us
-// against 71 (2.3e5 colliding points); 3 x 1024, N 4096 0.79 ms against 14.6 (9.8e6); 2 x 64,
-// N 1024 12 against 16.  A third goes into the item's sums, the rest is the latency of
-// the chain item, particle, point, table, nodes, list, gripper points.
-constexpr int kRec = 9;                // floats per record (8 used: the odd stride spreads the banks)
-__global__ void __launch_bounds__(kColChunk) collide_cells_kernel(const CollideArgs a)
+// compares the whole cloud.  A warp takes 32 colliding points that lie together in the sorted
+// collision cloud, so its lanes meet in the same cells (in ascending order they do not, and the
+// scattered loads set the pace: 0.80 ms on 9.8e6 points); the bit map gives each point's
+// place in the ascending list.
+// Measured on GB300 (per pass, against collide_nn_kernel with its sums): 3 x 256 particles, N 2048
+// 14.6 us against 71 (2.3e5 colliding points); 3 x 1024, N 4096 0.39 ms against 14.6 (9.8e6);
+// 57 % of the issue slots, the rest waits for the scattered loads.
+__global__ void __launch_bounds__(128, 10) collide_cells_kernel(const CollideArgs a)
 {
     if (a.err && *a.err != kDevOk) return;
-    __shared__ float sRec[kColChunk][kRec];
-    const int tid = threadIdx.x, lane = tid & 31, N = a.L.N;
+    const int lane = threadIdx.x & 31, N = a.L.N;
     const int count = a.col_items[0];
-    for (int item = blockIdx.x; item < count; item += gridDim.x) {
+    for (int item = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; item < count; item += (gridDim.x * blockDim.x) >> 5) {
         const int2 it = reinterpret_cast<const int2 *>(a.col_list)[item];
-        const int pk = it.x, slot = it.y * kColChunk + tid;
+        const int pk = it.x, slot = it.y * 32 + lane;
         const int grp = a.L.part_grp[pk], p = grp % a.L.P;
         const ObjMeta &om = a.L.obj[grp / a.L.P];
         const bool valid = slot < a.ncol[pk];
-        const long long at = om.colidx_base + (long long)(pk - om.pfirst) * om.Mc + slot;
-        const float4 c = valid ? __ldg(om.C + a.colidx[at]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const long long first = om.colidx_base + (long long)(pk - om.pfirst) * om.Mc;
+        const int at = valid ? a.colsrt[first + slot] : 0;
+        const float4 c = __ldg(om.Csort + at);
         const float *th = a.theta + (size_t)pk * 8;
         const float tx = th[0], ty = th[1], tz = th[2];
         float Rm[9];
@@ -681,7 +580,11 @@ __global__ void __launch_bounds__(kColChunk) collide_cells_kernel(const CollideA
         };
 
         int2 nd = make_int2(0, 0);
+        int rank = 0;
         if (valid) {
+            const int own = __float_as_int(c.w) + (at & ~(kColSegment - 1));
+            const int2 word = __ldg(a.colmap + om.colmap_base + (long long)(pk - om.pfirst) * ((om.Mc + 31) / 32) + (own >> 5));
+            rank = word.y + __popc((unsigned)word.x & ((1u << (own & 31)) - 1u));
             const float dx = __fsub_rn(c.x, tx), dy = __fsub_rn(c.y, ty), dz = __fsub_rn(c.z, tz);
             const float x = fmaf(Rm[0], dx, fmaf(Rm[3], dy, Rm[6] * dz)), y = fmaf(Rm[1], dx, fmaf(Rm[4], dy, Rm[7] * dz)),
                         z = fmaf(Rm[2], dx, fmaf(Rm[5], dy, Rm[8] * dz));
@@ -724,53 +627,20 @@ __global__ void __launch_bounds__(kColChunk) collide_cells_kernel(const CollideA
             for (int o = 16; o > 0; o >>= 1) argmin_xor(wb, wi, o);
             if (lane == src) { best = wb; bi = wi; }
         }
-        {
-            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (valid) {
-                bi = bi < N ? bi : 0;      // no finite distance at all (not reached with finite inputs)
-                s = __ldg(S + bi);
-                if (a.dbg_colnn) a.dbg_colnn[at] = bi;
-            }
-            float *rec = sRec[tid];
-            rec[0] = s.x; rec[1] = s.y; rec[2] = s.z;
-            rec[3] = c.x; rec[4] = c.y; rec[5] = c.z;
-            rec[6] = valid ? 1.f : 0.f;
-        }
-        __syncthreads();
-        // the item's sums, as in collide_nn_kernel: (sum e, part) adds colliding points part + 8 u
-        for (int e0 = 0; e0 < kColSums; e0 += kColChunk / 8) {
-            const int e = e0 + (tid >> 3), part = tid & 7;
-            dfloat acc{0.f, 0.f};
-            if (e < kColSums) {
-                const int ia = kColSel[e][0], ib = kColSel[e][1];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const float *rec = sRec[part + 8 * u];
-                    df_add_prod(acc, rec[ia], rec[ib]);
-                    if (e == kColSums - 1) {
-                        df_add_prod(acc, rec[4], rec[4]);
-                        df_add_prod(acc, rec[5], rec[5]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int o = 1; o < 8; o <<= 1) {
-                dfloat y;
-                y.hi = __shfl_xor_sync(0xffffffffu, acc.hi, o);
-                y.lo = __shfl_xor_sync(0xffffffffu, acc.lo, o);
-                df_merge(acc, y);
-            }
-            if (part == 0 && e < kColSums)
-                a.csums[(om.csum_base + (long long)(pk - om.pfirst) * om.chunks + it.y) * kColSums + e] =
-                    (double)acc.hi + (double)acc.lo;
-        }
-        __syncthreads();
+        if (valid) a.colnn[first + rank] = bi < N ? bi : 0;      // no finite distance at all: 0
     }
 }
 
 cudaError_t launch_collide(const CollideArgs &a, cudaStream_t st)
 {
-    collide_kernel<<<2 * a.L.T, kTestThreads, 0, st>>>(a);
+    // Many particles with small clouds keep the chip busy with small CTAs; few of them, or large clouds,
+    // want more warps per particle (256 against 128 threads, us per pass: T 154, Mc 5003 16 against
+    // 23; T 768, 8192 21 against 23; T 3072, 65536 286 against 300; but T 3072, 2048 47
+    // against 39, T 7040, 1k to 32k 91 against 78).
+    if (a.L.T <= 1024 || a.most_points >= 32768)
+        collide_kernel<256><<<a.L.T, 256, 0, st>>>(a);
+    else
+        collide_kernel<128><<<a.L.T, 128, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -793,8 +663,9 @@ cudaError_t launch_collide_nn(const CollideArgs &a, cudaStream_t st)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         return 4 * sms;
     });
-    if (a.cells) {          // 24 small CTAs per SM, no more than the work list can hold
-        collide_cells_kernel<<<a.most_items < 6 * grid ? a.most_items : 6 * grid, kColChunk, 0, st>>>(a);
+    if (a.cells) {          // ten CTAs of four warps per SM, no more than the work list can fill
+        const int ctas = (a.most_items + 3) / 4;
+        collide_cells_kernel<<<ctas < 5 * grid / 2 ? ctas : 5 * grid / 2, 128, 0, st>>>(a);
         return cudaGetLastError();
     }
     const size_t smem = 2 * sizeof(float4) * (size_t)((a.L.N + 63) / 64 * 64) + 32 * sizeof(float4);

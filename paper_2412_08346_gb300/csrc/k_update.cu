@@ -7,58 +7,6 @@ namespace asicp {
 
 namespace {
 
-// Quaternion gradient g_k = sum_ab (dR_ab/dq_k) E_ab for the homogeneous form
-// R = (w^2 - |v|^2) I + 2 v v^T + 2 w [v]_x, with E = sum_i e_i s_i^T:
-//   dR/dw   = 2 w I + 2 [v]_x
-//   dR/dv_k = -2 v_k I + 2 (e_k v^T + v e_k^T) + 2 w [e_k]_x
-// This equals sum_i J(s_i)^T e_i, the rotation gradient of Eqs. 5 and 17.
-__device__ void quat_grad_from_E(const double q[4], const double E[9], double g[4])
-{
-    const double w = q[0], v[3] = {q[1], q[2], q[3]};
-    const double tr = E[0] + E[4] + E[8];
-    const double kx = E[7] - E[5], ky = E[2] - E[6], kz = E[3] - E[1];   // <[e_k]_x, E>
-    g[0] = 2 * w * tr + 2 * (v[0] * kx + v[1] * ky + v[2] * kz);
-    const double ks[3] = {kx, ky, kz};
-    for (int k = 0; k < 3; ++k) {
-        double rowv = E[k * 3 + 0] * v[0] + E[k * 3 + 1] * v[1] + E[k * 3 + 2] * v[2];
-        double colv = E[0 * 3 + k] * v[0] + E[1 * 3 + k] * v[1] + E[2 * 3 + k] * v[2];
-        g[1 + k] = -2 * v[k] * tr + 2 * rowv + 2 * colv + 2 * w * ks[k];
-    }
-}
-
-// sum_i |R s_i + t - x_i|^2, sum_i (R s_i + t - x_i) and sum_i (R s_i + t - x_i) s_i^T
-// from the linear sums: ss = sum s (3), SS = sum s s^T (9, full), xs = sum x,
-// XS = sum x s^T (9), xx = sum |x|^2, n terms.
-__device__ void residual_moments(const double R[9], const double t[3], double n, const double ss[3],
-                                 const double SS[9], const double xs[3], const double XS[9], double xx,
-                                 double *se2, double Se[3], double E[9])
-{
-    double Rs[3];
-    for (int a = 0; a < 3; ++a) Rs[a] = R[a * 3 + 0] * ss[0] + R[a * 3 + 1] * ss[1] + R[a * 3 + 2] * ss[2];
-    // R is the homogeneous form of the quaternion's rotation (|q|^2 times a rotation), so
-    // R^T R = |q|^4 I and sum_i |R s_i|^2 = |q|^4 tr(SS); |q|^4 is the squared norm of a column
-    const double q4 = R[0] * R[0] + R[3] * R[3] + R[6] * R[6];
-    const double quad = q4 * (SS[0] + SS[4] + SS[8]);
-    double cross = 0.0;
-    for (int a = 0; a < 9; ++a) cross += R[a] * XS[a];
-    const double tt = t[0] * t[0] + t[1] * t[1] + t[2] * t[2];
-    const double tRs = t[0] * Rs[0] + t[1] * Rs[1] + t[2] * Rs[2];
-    const double tx = t[0] * xs[0] + t[1] * xs[1] + t[2] * xs[2];
-    *se2 = quad + n * tt + xx + 2 * tRs - 2 * tx - 2 * cross;
-    for (int a = 0; a < 3; ++a) Se[a] = Rs[a] + n * t[a] - xs[a];
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b)
-            E[a * 3 + b] = R[a * 3 + 0] * SS[0 * 3 + b] + R[a * 3 + 1] * SS[1 * 3 + b] + R[a * 3 + 2] * SS[2 * 3 + b] +
-                           t[a] * ss[b] - XS[a * 3 + b];
-}
-
-__device__ __forceinline__ void sym_full(const double *s6, double S[9])
-{
-    S[0] = s6[0]; S[1] = s6[1]; S[2] = s6[2];
-    S[3] = s6[1]; S[4] = s6[3]; S[5] = s6[4];
-    S[6] = s6[2]; S[7] = s6[4]; S[8] = s6[5];
-}
-
 __device__ __forceinline__ float pair_d2(float4 a, float4 b)
 {
     return dist2_f32(a.x, a.y, a.z, b.x, b.y, b.z);
@@ -66,94 +14,304 @@ __device__ __forceinline__ float pair_d2(float4 a, float4 b)
 
 }  // namespace
 
-// Per particle (one thread each, small CTAs so the float64 work spreads over
-// many SMs):
-//  1. cost and gradient from the matching sums (Eqs. 13-17) or, for a particle
-//     with colliding points, from the collision sums (Eq. 18 with Eqs. 4-5),
-//     quaternion block projected onto the tangent space at q;
-//  2. convergence bookkeeping (SGD phase);
-//  3. mode 2: the SGD-ICP update of Eq. 3 (A = I); modes 0 (evaluate only) and 1
-//     (SVGD, done by stein_kernel) leave the poses alone.
-//  Thread 0 of CTA 0 also clears the collision work-list counters for the next pass.
-constexpr int kFinalizeThreads = 4;      // 192 CTAs for 768 particles: float64 chains spread over every SM
+// Two particles per CTA, kFinalizeThreads threads each.
+//  1. The sums its cost and gradient are linear in, over pairs of a point x and a gripper point s (both
+//     float32, so every product is exact in double-float): sum s, sum s s^T, sum x,
+//     sum x s^T and sum |x|^2.  Of a particle without colliding points the forward pairs
+//     (x the matched object point): 128 threads take every 128th pair, kPairB at a time so that
+//     their loads overlap; sum s and sum s s^T are the preshape's.  Of another one the colliding
+//     points and their gripper points: per kColChunk of them, in ascending order, eight lanes add
+//     eight points each, merged in a fixed tree; the chunks are added in order.  A warp takes
+//     four chunks and half of the sums, its records straight from memory, eight loads at a time.
+//     The result depends on nothing but the pairs.
+//  2. Half a warp each: cost and gradient (Eqs. 13-17, or Eq. 18 with Eqs. 4-5) in float64, quaternion
+//     block projected onto the tangent space at q.  With E = sum_i e_i s_i^T, e_i = R s_i + t - x_i,
+//     the quaternion gradient is g_k = sum_ab (dR_ab/dq_k) E_ab for the homogeneous form
+//     R = (w^2 - |v|^2) I + 2 v v^T + 2 w [v]_x:
+//       dR/dw   = 2 w I + 2 [v]_x
+//       dR/dv_k = -2 v_k I + 2 (e_k v^T + v e_k^T) + 2 w [e_k]_x,
+//     which equals sum_i J(s_i)^T e_i of Eqs. 5 and 17; R is |q|^2 times a rotation, so
+//     R^T R = |q|^4 I and sum_i |R s_i|^2 = |q|^4 tr(sum s s^T).  Entries of a vector or matrix are
+//     the lanes'; the float64 pipe takes 16 cycles per instruction whatever the number of lanes,
+//     so the two particles share a warp.
+//  3. Convergence bookkeeping (SGD phase) and, in mode 2, the SGD-ICP update of Eq. 3 (A = I);
+//     modes 0 (evaluate only) and 1 (SVGD, done by stein_kernel) leave the poses alone.
+//  CTA 0 also clears the collision work-list counters for the next pass.
+// Measured on GB300, per pass: 3 x 256 particles, N 2048 26 us (28 us for part 2 alone with a thread
+// per particle, the sums in the collision kernel and the reverse matching besides); 3 x 1024,
+// 9.8e6 colliding points 0.27 ms (with 192 threads summing from shared memory 0.50). With few
+// particles the float64 chain of part 2 bounds it, with many the sums' instructions (55 % of the
+// issue slots).
+constexpr int kFinalizeThreads = 128;      // four warps: eight chunks of colliding points a round
+constexpr int kSumThreads = 128;           // threads that add forward pairs
+constexpr int kPairB = 4;                  // forward pairs per thread whose loads overlap
+constexpr int kRecB = 4;                   // colliding points per lane whose loads overlap
+static_assert(kSumThreads == kFinalizeThreads && kColChunk == 64, "finalize_kernel");
 
-__global__ void __launch_bounds__(kFinalizeThreads) finalize_kernel(const UpdateArgs a)
+namespace {
+__constant__ unsigned char kSym[9] = {0, 1, 2, 1, 3, 4, 2, 4, 5};   // 3 x 3 entry -> upper-triangle entry
+
+// sum r (3), sum r s^T (9), sum |r|^2 (1) of a particle's forward pairs, for kSumThreads threads; the
+// warps' sums go to sred.
+__device__ __forceinline__ void pair_sums(const float4 *__restrict__ S, const int *__restrict__ idx,
+                                          const float4 *__restrict__ R, int N, int tid, double (*sred)[kFwdSums])
 {
-    if (a.err && *a.err != kDevOk) return;    // an earlier kernel of the pass gave up: its sums are not valid
-    const int pk = blockIdx.x * blockDim.x + threadIdx.x;
-    if (pk == 0 && a.col_items) { a.col_items[0] = 0; a.col_items[1] = 0; }
-    if (pk >= a.L.T) return;
-    const int grp = a.L.part_grp[pk], p = grp % a.L.P, o = grp / a.L.P;
+    dfloat acc[kFwdSums];
+#pragma unroll
+    for (int c = 0; c < kFwdSums; ++c) acc[c] = dfloat{0.f, 0.f};
+    auto add_pair = [&](float4 r, float4 s) {
+        const float rv[3] = {r.x, r.y, r.z}, sv[3] = {s.x, s.y, s.z};
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            df_add(acc[u], rv[u]);
+#pragma unroll
+            for (int v = 0; v < 3; ++v) df_add_prod(acc[3 + 3 * u + v], rv[u], sv[v]);
+            df_add_prod(acc[12], rv[u], rv[u]);
+        }
+    };
+    int i = tid;
+    for (; i + (kPairB - 1) * kSumThreads < N; i += kPairB * kSumThreads) {
+        int id[kPairB];
+        float4 s[kPairB], r[kPairB];
+#pragma unroll
+        for (int u = 0; u < kPairB; ++u) { id[u] = idx[i + u * kSumThreads]; s[u] = S[i + u * kSumThreads]; }
+#pragma unroll
+        for (int u = 0; u < kPairB; ++u) r[u] = __ldg(R + id[u]);
+#pragma unroll
+        for (int u = 0; u < kPairB; ++u) add_pair(r[u], s[u]);
+    }
+    for (; i < N; i += kSumThreads) add_pair(__ldg(R + idx[i]), S[i]);
+    warp_sum_df(acc);
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int c = 0; c < kFwdSums; ++c) sred[tid >> 5][c] = (double)acc[c].hi + (double)acc[c].lo;
+}
+}  // namespace
+
+namespace {
+// Half of the sums of four chunks of a particle's colliding points, for a warp: lane = 8 * chunk +
+// part, part adds points part + 8 u, u = 0 .. 7.  HALF 0: sum s (3), sum s s^T (6), sum c (3); 1:
+// sum c s^T (9), sum |c|^2 (1), s the gripper point, c the colliding point.  Points past the end add zeros.
+// The chunks' sums go to out[0 .. 3].
+template <int HALF>
+__device__ __forceinline__ void chunk_sums(const float4 *__restrict__ S, const float4 *__restrict__ C,
+                                           const int *__restrict__ colidx, const int *__restrict__ colnn, int l0, int nc,
+                                           dfloat (*out)[kColSums])
+{
+    constexpr int kN = HALF == 0 ? 12 : 10;
+    const int lane = threadIdx.x & 31, base = l0 + (lane >> 3) * kColChunk + (lane & 7);
+    dfloat acc[kN];
+#pragma unroll
+    for (int k = 0; k < kN; ++k) acc[k] = dfloat{0.f, 0.f};
+#pragma unroll 1                           // (both halves unrolled whole overflow the instruction cache)
+    for (int u0 = 0; u0 < 8; u0 += kRecB) {
+        float4 s[kRecB], c[kRecB];
+        int is[kRecB], ic[kRecB];
+#pragma unroll
+        for (int u = 0; u < kRecB; ++u) {
+            const int l = min(base + 8 * (u0 + u), nc - 1);
+            ic[u] = __ldg(colidx + l);
+            is[u] = __ldg(colnn + l);
+        }
+#pragma unroll
+        for (int u = 0; u < kRecB; ++u) { c[u] = __ldg(C + ic[u]); s[u] = __ldg(S + is[u]); }
+#pragma unroll
+        for (int u = 0; u < kRecB; ++u) {
+            const bool in = base + 8 * (u0 + u) < nc;
+            const float sv[3] = {in ? s[u].x : 0.f, in ? s[u].y : 0.f, in ? s[u].z : 0.f};
+            const float cv[3] = {in ? c[u].x : 0.f, in ? c[u].y : 0.f, in ? c[u].z : 0.f};
+            if (HALF == 0) {
+                int k = 3;
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    df_add(acc[i], sv[i]);
+                    df_add(acc[9 + i], cv[i]);
+#pragma unroll
+                    for (int j = i; j < 3; ++j) df_add_prod(acc[k++], sv[i], sv[j]);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) df_add_prod(acc[3 * i + j], cv[i], sv[j]);
+                    df_add_prod(acc[9], cv[i], cv[i]);
+                }
+            }
+        }
+    }
+#pragma unroll 1
+    for (int w = 1; w < 8; w <<= 1)
+#pragma unroll
+        for (int k = 0; k < kN; ++k) {
+            dfloat y;
+            y.hi = __shfl_xor_sync(0xffffffffu, acc[k].hi, w);
+            y.lo = __shfl_xor_sync(0xffffffffu, acc[k].lo, w);
+            df_merge(acc[k], y);
+        }
+    if ((lane & 7) == 0)
+#pragma unroll
+        for (int k = 0; k < kN; ++k) out[lane >> 3][(HALF == 0 ? 0 : 12) + k] = acc[k];
+}
+}  // namespace
+
+// Barrier of the kFinalizeThreads threads of one particle.
+__device__ __forceinline__ void half_sync(int half)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(half + 1), "n"(kFinalizeThreads) : "memory");
+}
+
+__global__ void __launch_bounds__(2 * kFinalizeThreads, 4) finalize_kernel(const UpdateArgs a)
+{
+    if (a.err && *a.err != kDevOk) return;    // an earlier kernel of the pass gave up: its results are not valid
+    constexpr int kChunks = 2 * kFinalizeThreads / 32;     // chunks a round
+    __shared__ dfloat sPart_[2][2][kChunks][kColSums];
+    __shared__ double sred_[2][kSumThreads / 32][kFwdSums];
+    // the sums {s (3), s s^T (6), x (3), x s^T (9), |x|^2} and the half warp's vectors and matrices
+    __shared__ double sm_[2][kColSums], sR_[2][9], sE_[2][9], sRs_[2][3], sTcp_[2][3], sEc_[2][3], sG_[2][4];
     const int N = a.L.N;
-    double t[3], q[4], g[7];
+    if (blockIdx.x == 0 && threadIdx.x == 0 && a.col_items) { a.col_items[0] = 0; a.col_items[1] = 0; }
+    {
+        const int half = threadIdx.x / kFinalizeThreads, tid = threadIdx.x % kFinalizeThreads;
+        const int pk = 2 * blockIdx.x + half;
+        double *sm = sm_[half];
+        if (pk < a.L.T) {
+            const int grp = a.L.part_grp[pk], p = grp % a.L.P;
+            const ObjMeta &om = a.L.obj[grp / a.L.P];
+            const float4 *__restrict__ S = a.S + (size_t)p * N;
+            const int nc = a.ncol[pk];
+            if (nc == 0) {
+                double (*sred)[kFwdSums] = sred_[half];
+                pair_sums(S, a.nn_idx + (size_t)pk * N, om.R, N, tid, sred);
+                half_sync(half);
+                if (tid < kFwdSums) {
+                    double v = 0.0;
+                    for (int w = 0; w < kSumThreads / 32; ++w) v += sred[w][tid];
+                    sm[9 + tid] = v;
+                } else if (tid >= 32 && tid < 41) {
+                    sm[tid - 32] = a.pconst[(size_t)p * 12 + tid - 32];
+                }
+            } else {
+                const long long first = om.colidx_base + (long long)(pk - om.pfirst) * om.Mc;
+                double total = 0.0;
+                int buf = 0;
+                for (int l0 = 0; l0 < nc; l0 += kChunks * kColChunk, buf ^= 1) {
+                    dfloat (*part)[kColSums] = sPart_[half][buf];
+                    const int warp = tid >> 5, w0 = (warp >> 1) * 4, l = l0 + w0 * kColChunk;
+                    if (l < nc) {
+                        if (warp & 1)
+                            chunk_sums<1>(S, om.C, a.colidx + first, a.colnn + first, l, nc, part + w0);
+                        else
+                            chunk_sums<0>(S, om.C, a.colidx + first, a.colnn + first, l, nc, part + w0);
+                    }
+                    // (one barrier a round: the next round writes the other buffer, the one after waits here)
+                    half_sync(half);
+                    if (tid < kColSums)
+                        for (int k = 0; k < kChunks && l0 + k * kColChunk < nc; ++k)
+                            total += (double)part[k][tid].hi + (double)part[k][tid].lo;
+                }
+                if (tid < kColSums) sm[tid] = total;
+            }
+        }
+    }
+    __syncthreads();
+    const int half = threadIdx.x >> 4, lane = threadIdx.x & 15, pk = 2 * blockIdx.x + half;
+    if (threadIdx.x >= 32 || pk >= a.L.T) return;
+    const unsigned hmask = 0xffffu << (16 * half);
+    const double *sm = sm_[half];
+    double *sR = sR_[half], *sE = sE_[half], *sRs = sRs_[half], *sTcp = sTcp_[half], *sEc = sEc_[half], *sG = sG_[half];
+    const int grp = a.L.part_grp[pk], o = grp / a.L.P;
+    const double *pc = a.pconst + (size_t)(grp % a.L.P) * 12;
+    const int nc = a.ncol[pk];
+
     const float *th = a.theta + (size_t)pk * 8;
+    double t[3], q[4], R[9];
     for (int c = 0; c < 3; ++c) t[c] = th[c];
     for (int c = 0; c < 4; ++c) q[c] = th[3 + c];
-    double R[9];
     quat_rot_f64(q[0], q[1], q[2], q[3], R);
-    const int nc = a.ncol[pk];
-    double se2, Se[3], E[9], cnt;
+    if (lane == 0)
+        for (int c = 0; c < 9; ++c) sR[c] = R[c];
+    const double *ss = sm, *S6 = sm + 3, *xs = sm + 9, *XS = sm + 12;
+    const double xx = sm[21], n = nc == 0 ? (double)N : (double)nc;
+    const int r3 = lane % 3;               // this lane's entry of a 3-vector (lanes 0 .. 2)
+    const int u9 = min(lane, 8), ra = u9 / 3, rb = u9 % 3;     // and of a 3 x 3 matrix (lanes 0 .. 8)
+    const double tr3 = th[r3], tra = th[ra];
+    __syncwarp(hmask);
+    const double rs = sR[r3 * 3 + 0] * ss[0] + sR[r3 * 3 + 1] * ss[1] + sR[r3 * 3 + 2] * ss[2];
+    if (lane < 3) sRs[lane] = rs;
+    const double q4 = R[0] * R[0] + R[3] * R[3] + R[6] * R[6];
+    const double quad = q4 * (S6[0] + S6[3] + S6[5]);
+    double cross = 0.0;
+    for (int c = 0; c < 9; ++c) cross += R[c] * XS[c];
+    __syncwarp(hmask);
+    const double tt = t[0] * t[0] + t[1] * t[1] + t[2] * t[2];
+    const double tRs = t[0] * sRs[0] + t[1] * sRs[1] + t[2] * sRs[2];
+    const double tx = t[0] * xs[0] + t[1] * xs[1] + t[2] * xs[2];
+    double se2 = quad + n * tt + xx + 2 * tRs - 2 * tx - 2 * cross;
+    double Se = rs + n * tr3 - xs[r3];
+    double E = sR[ra * 3 + 0] * S6[kSym[rb]] + sR[ra * 3 + 1] * S6[kSym[3 + rb]] + sR[ra * 3 + 2] * S6[kSym[6 + rb]] +
+               tra * ss[rb] - XS[u9];
     if (nc == 0) {
-        double fs[kFwdSums];
-        for (int c = 0; c < kFwdSums; ++c) fs[c] = a.fsums[(size_t)pk * kFwdSums + c];
-        const double *pc = a.pconst + (size_t)p * 12;
-        double SS[9];
-        sym_full(pc + 3, SS);
-        residual_moments(R, t, (double)N, pc, SS, fs, fs + 3, fs[12], &se2, Se, E);
         // TCP-CoM term (Eq. 15) inside the 1/N, weight w_com (Eqs. 16-17)
-        const double tcp[3] = {pc[0] / N, pc[1] / N, pc[2] / N};
-        const double *com = a.L.com + 3 * o;
-        double ec[3];
-        for (int u = 0; u < 3; ++u)
-            ec[u] = R[u * 3 + 0] * tcp[0] + R[u * 3 + 1] * tcp[1] + R[u * 3 + 2] * tcp[2] + t[u] - com[u];
-        se2 += a.w_com * (ec[0] * ec[0] + ec[1] * ec[1] + ec[2] * ec[2]);
-        for (int u = 0; u < 3; ++u) {
-            Se[u] += a.w_com * ec[u];
-            for (int v = 0; v < 3; ++v) E[u * 3 + v] += a.w_com * ec[u] * tcp[v];
-        }
-        cnt = (double)N;
-    } else {
-        // add the per-chunk collision sums in chunk order
-        const ObjMeta &om = a.L.obj[o];
-        const int used = (nc + kColChunk - 1) / kColChunk;
-        const double *csp = a.csums + (om.csum_base + (long long)(pk - om.pfirst) * om.chunks) * kColSums;
-        double cs[kColSums];
-        for (int c = 0; c < kColSums; ++c) cs[c] = 0.0;
-        for (int b = 0; b < used; ++b)
-            for (int c = 0; c < kColSums; ++c) cs[c] += csp[(size_t)b * kColSums + c];
-        double SS[9];
-        sym_full(cs + 3, SS);
-        residual_moments(R, t, (double)nc, cs, SS, cs + 9, cs + 12, cs[21], &se2, Se, E);
-        cnt = (double)nc;
+        const double tcp = pc[r3] / N;
+        if (lane < 3) sTcp[lane] = tcp;
+        __syncwarp(hmask);
+        const double ec = sR[r3 * 3 + 0] * sTcp[0] + sR[r3 * 3 + 1] * sTcp[1] + sR[r3 * 3 + 2] * sTcp[2] + tr3 -
+                          a.L.com[3 * o + r3];
+        if (lane < 3) sEc[lane] = ec;
+        __syncwarp(hmask);
+        se2 += a.w_com * (sEc[0] * sEc[0] + sEc[1] * sEc[1] + sEc[2] * sEc[2]);
+        Se += a.w_com * ec;
+        E += a.w_com * sEc[ra] * sTcp[rb];
     }
-    double gq[4];
-    quat_grad_from_E(q, E, gq);
-    const double inv = 1.0 / cnt;
-    for (int u = 0; u < 3; ++u) g[u] = Se[u] * inv;
-    for (int u = 0; u < 4; ++u) gq[u] *= inv;
-    const double dq = gq[0] * q[0] + gq[1] * q[1] + gq[2] * q[2] + gq[3] * q[3];
-    for (int u = 0; u < 4; ++u) g[3 + u] = gq[u] - dq * q[u];
+    if (lane < 9) sE[lane] = E;
+    __syncwarp(hmask);
+    const double inv = 1.0 / n;
+    // quaternion gradient: lane 0 the scalar part, lanes 1 .. 3 the vector part
+    const double tr = sE[0] + sE[4] + sE[8];
+    const double kx = sE[7] - sE[5], ky = sE[2] - sE[6], kz = sE[3] - sE[1];   // <[e_k]_x, E>
+    double gq;
+    if (lane == 0) {
+        gq = 2 * q[0] * tr + 2 * (q[1] * kx + q[2] * ky + q[3] * kz);
+    } else {
+        const int k = min(lane, 3) - 1;
+        const double rowv = sE[k * 3 + 0] * q[1] + sE[k * 3 + 1] * q[2] + sE[k * 3 + 2] * q[3];
+        const double colv = sE[0 * 3 + k] * q[1] + sE[1 * 3 + k] * q[2] + sE[2 * 3 + k] * q[3];
+        const double ks = k == 0 ? kx : k == 1 ? ky : kz;
+        gq = -2 * (double)th[4 + k] * tr + 2 * rowv + 2 * colv + 2 * q[0] * ks;
+    }
+    gq *= inv;
+    if (lane < 4) sG[lane] = gq;
+    __syncwarp(hmask);
+    const double dq = sG[0] * q[0] + sG[1] * q[1] + sG[2] * q[2] + sG[3] * q[3];
+    const double qo = th[3 + min(lane, 3)];
+    const double gt = Se * inv, gr = gq - dq * qo;          // lanes 0 .. 2: translation; 0 .. 3: rotation
     const double cost = se2 * inv;
-    a.cost[pk] = cost;
-    for (int u = 0; u < 7; ++u) a.grad[(size_t)pk * 8 + u] = g[u];
+    if (lane < 3) a.grad[(size_t)pk * 8 + lane] = gt;
+    if (lane < 4) a.grad[(size_t)pk * 8 + 3 + lane] = gr;
     int frozen = a.frozen[pk];
     if (a.mode == 2 && a.conv_tol >= 0.f) {
         const double prev = a.prev_cost[pk];
         if (nc > 0) frozen = 0;
         else if (prev >= 0.0 && fabs(cost - prev) <= (double)a.conv_tol * prev) frozen = 1;
-        a.frozen[pk] = frozen;
     }
-    if (a.mode != 0) a.prev_cost[pk] = cost;
+    __syncwarp(hmask);                          // (prev_cost and frozen have been read)
+    if (lane == 0) {
+        a.cost[pk] = cost;
+        a.frozen[pk] = frozen;
+        if (a.mode != 0) a.prev_cost[pk] = cost;
+    }
     if (a.mode == 2) {
         float *tw = a.theta + (size_t)pk * 8;
-        for (int u = 0; u < 7; ++u) a.phi[(size_t)pk * 8 + u] = 0.f;
-        if (pk < a.L.G) a.h[pk] = 0.f;
+        if (lane < 7) a.phi[(size_t)pk * 8 + lane] = 0.f;
+        if (lane == 0 && pk < a.L.G) a.h[pk] = 0.f;
         if (!frozen) {
-            double nq[4];
-            for (int u = 0; u < 4; ++u) nq[u] = q[u] - (double)a.eta_sgd * g[3 + u];
-            const double nn = sqrt(nq[0] * nq[0] + nq[1] * nq[1] + nq[2] * nq[2] + nq[3] * nq[3]);
-            for (int u = 0; u < 3; ++u) tw[u] = (float)(t[u] - (double)a.eta_sgd * g[u]);
-            for (int u = 0; u < 4; ++u) tw[3 + u] = (float)(nq[u] / nn);
+            const double nq = qo - (double)a.eta_sgd * gr;
+            __syncwarp(hmask);                  // (sG and theta have been read)
+            if (lane < 4) sG[lane] = nq;
+            __syncwarp(hmask);
+            const double nn = sqrt(sG[0] * sG[0] + sG[1] * sG[1] + sG[2] * sG[2] + sG[3] * sG[3]);
+            if (lane < 3) tw[lane] = (float)(tr3 - (double)a.eta_sgd * gt);
+            if (lane < 4) tw[3 + lane] = (float)(nq / nn);
         }
     }
 }
@@ -409,7 +567,7 @@ cudaError_t init_update_attributes()
 
 cudaError_t launch_finalize(const UpdateArgs &a, cudaStream_t st)
 {
-    finalize_kernel<<<(a.L.T + kFinalizeThreads - 1) / kFinalizeThreads, kFinalizeThreads, 0, st>>>(a);
+    finalize_kernel<<<(a.L.T + 1) / 2, 2 * kFinalizeThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -144,7 +144,7 @@ extern "C" asicp_status asicp_match_noalloc(const float *theta, int P, int K, co
     om.R = obj;
     om.Rx = screen;
     om.C = obj;
-    om.M = M; om.Mpad = Mpad; om.Mc = M; om.chunks = 0;
+    om.M = M; om.Mpad = Mpad; om.Mc = M;
     om.pfirst = 0; om.np = PK;
     NOALLOC_CK(cudaMemcpyAsync(objmeta, &om, sizeof(ObjMeta), cudaMemcpyHostToDevice, st));
 
