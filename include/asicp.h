@@ -268,8 +268,7 @@ asicp_status asicp_kernel_times(asicp_ctx *ctx, double ms[ASICP_KERNEL_KINDS], l
  *           (host inputs are staged through the scratch array, not allocated)
  *   nn_idx  P*K*N int32 output, device memory
  *   cuda_stream  cudaStream_t (NULL: default stream); the call waits for the stream
- *           twice (after checking the inputs and at the end) and returns when nn_idx
- *           is written
+ *           once and returns when nn_idx is written
  * Its scratch is one fixed-size static device array (5 MiB) that every device that
  * loads the library keeps until the process exits; it bounds the sizes to
  * P*K <= ASICP_NOALLOC_MAX_PK, P*N <= ASICP_NOALLOC_MAX_PN, M <= ASICP_NOALLOC_MAX_M

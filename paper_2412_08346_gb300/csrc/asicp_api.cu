@@ -132,7 +132,7 @@ struct asicp_ctx {
     std::vector<int> grp_off_h;
     std::vector<ObjMeta> objmeta_h;
 
-    DevMem partgrp, grpoff, objmeta, items, ctaoff, com, frame, colitems, collist, stage, S, Ssort, preframe, prenodes, preleaves, cellwork, pconst, dmeta, theta,
+    DevMem partgrp, grpoff, objmeta, items, ctaoff, com, frame, colitems, collist, stage, S, Ssort, preframe, prenodes, preleaves, cellwork, refscr, pconst, dmeta, theta,
         ncol, colidx, colsrt, colnn, colmap, cost, grad, prev, frozen, phi, h, order, errw, out7, outc, outi, nnidx, tccand, dbg_d2, dbg_sp;
 
     // profiling: events recorded around launches (kind, start, stop)
@@ -256,6 +256,8 @@ void plan_fwd_items(asicp_ctx *c, int v)
         const ObjMeta &m = om[o];
         long long nq = (long long)std::ceil(unit / std::max(1, m.Mpad) / threads) * threads;
         nq = std::min<long long>(std::max<long long>(nq, threads), qmax);
+        // few queries for the grid: the item size that gives the shortest schedule
+        if (nq == threads && om.size() == 1 && v != kFwdVariants - 1) nq = fwd_item_queries(v, (long long)m.np * N);
         const long long q0 = (long long)m.pfirst * N, q1 = (long long)(m.pfirst + m.np) * N;
         for (long long q = q0; q < q1; q += nq) {
             FwdItem it;
@@ -450,15 +452,14 @@ void select_minibatch(asicp_ctx *c, int k)
     if (k >= 0 && k + 1 < (int)c->mb_off.size()) {
         const int first = c->mb_off[k], cnt = c->mb_off[k + 1] - first;
         const int Mpad = (cnt + kRefTilePts - 1) / kRefTilePts * kRefTilePts;
-        ck(launch_gather_points(c->objs[0].R.as<float4>(), c->mb_idx.as<int>() + first, cnt, c->mb_R.as<float4>(), st),
-           "mini-batch gather");
-        // the mini-batch keeps the whole object's frame (its points are a subset)
-        ck(launch_ref_prep(c->mb_R.as<float4>(), cnt, Mpad, c->mb_Rx.p, c->frame.as<float4>(), false, st),
-           "mini-batch prep");
         m.R = c->mb_R.as<float4>();
         m.Rx = c->mb_Rx.as<ulonglong2>();
         m.M = cnt;
         m.Mpad = Mpad;
+        ck(launch_minibatch(c->objs[0].R.as<float4>(), c->mb_idx.as<int>() + first, cnt, Mpad, c->mb_R.as<float4>(),
+                            c->mb_Rx.p, c->frame.as<float4>(), c->objmeta.as<ObjMeta>(), m, st),
+           "mini-batch");
+        return;
     }
     ck(launch_store_meta(c->objmeta.as<ObjMeta>(), m, st), "object table");
 }
@@ -901,7 +902,11 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
     ctx->stage.ensure(sizeof(float) * 3 * (size_t)(M > mc ? M : mc), "staging");
     b.R.ensure(sizeof(float4) * M, "object cloud");
     ck(cudaMemcpyAsync(ctx->stage.p, R_xyz, sizeof(float) * 3 * (size_t)M, cudaMemcpyDefault, ctx->st), "copy R");
-    ck(launch_pack_points(ctx->stage.as<float>(), M, b.R.as<float4>(), ctx->errw.as<int>(), ctx->st), "pack R");
+    const int Mpad = (M + kRefTilePts - 1) / kRefTilePts * kRefTilePts;
+    b.Rx.ensure(sizeof(float4) * (size_t)Mpad, "screening layout");
+    ck(launch_ref_prep(ctx->stage.as<float>(), M, Mpad, b.R.as<float4>(), b.Rx.p, ctx->frame.as<float4>() + o,
+                       ctx->com.as<double>() + 3 * o, ctx->refscr.as<RefScratch>(), ctx->errw.as<int>(), ctx->st),
+       "ref prep");
     if (C_xyz) {
         b.C.ensure(sizeof(float4) * mc, "collision cloud");
         ck(cudaMemcpyAsync(ctx->stage.p, C_xyz, sizeof(float) * 3 * (size_t)mc, cudaMemcpyDefault, ctx->st), "copy C");
@@ -911,10 +916,6 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
     }
     b.Csort.ensure(sizeof(float4) * (size_t)mc, "collision cloud, sorted");
     b.Cball.ensure(sizeof(float4) * (((size_t)mc + 31) / 32), "collision cloud, balls");
-    ck(launch_centroid(b.R.as<float4>(), M, ctx->com.as<double>() + 3 * o, ctx->st), "centroid");
-    const int Mpad = (M + kRefTilePts - 1) / kRefTilePts * kRefTilePts;
-    b.Rx.ensure(sizeof(float4) * (size_t)Mpad, "screening layout");
-    ck(launch_ref_prep(b.R.as<float4>(), M, Mpad, b.Rx.p, ctx->frame.as<float4>() + o, true, ctx->st), "ref prep");
     b.Rt.ensure(tc_ref_bytes(Mpad), "tensor-core object tiles");
     ck(launch_tc_ref_prep(b.R.as<float4>(), M, Mpad, ctx->frame.as<float4>() + o, b.Rt.p, ctx->st),
        "tensor-core ref prep");
@@ -1000,6 +1001,8 @@ asicp_status asicp_create(const asicp_config *cfg, asicp_ctx **out)
         c->frame.ensure(sizeof(float4) * c->nobj, "screening frames");
         c->pconst.ensure(sizeof(double) * 12 * cfg->P, "pconst");
         c->dmeta.ensure(sizeof(SdfMeta) * cfg->P, "sdf meta");
+        c->refscr.ensure(sizeof(RefScratch), "object preparation");
+        ck(cudaMemsetAsync(c->refscr.p, 0, sizeof(RefScratch), c->st), "clear object preparation");
         c->errw.ensure(sizeof(int), "error word");
         ck(cudaMemsetAsync(c->errw.p, 0, sizeof(int), c->st), "clear error word");
         ck(cudaStreamSynchronize(c->st), "create");

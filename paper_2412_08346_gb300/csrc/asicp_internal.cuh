@@ -84,6 +84,18 @@ __device__ __forceinline__ float3 xform_f32(const float R[9], float tx, float ty
     return o;
 }
 
+// Total order of float32 values (no NaN) as unsigned keys, and back.
+__device__ __forceinline__ unsigned order_key(float f)
+{
+    const unsigned u = __float_as_uint(f);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+__device__ __forceinline__ float key_float(unsigned k)
+{
+    return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+}
+
 // Exact-form squared distance |a - b|^2 in float32, fixed order.
 __device__ __forceinline__ float dist2_f32(float ax, float ay, float az, float bx, float by, float bz)
 {
@@ -235,6 +247,8 @@ struct FwdArgs {
     const FwdItem *items;    // [n_items] work items (null: object 0, consecutive 1024-query items)
     const int *cta_off;      // [grid + 1]: CTA b runs items cta_off[b] .. cta_off[b+1]-1 (null: round-robin)
     int n_items;
+    int item_queries;        // queries per item when items is null
+    int check_err;           // float32 shapes: skip the work if the error word is set
     int *err;                // error word
     int *nn_idx;             // [T][N] nearest object point per query
     float *dbg_d2;           // [T][N] or null
@@ -259,11 +273,19 @@ int fwd_shape_queries(int v);          // queries per work item (at most) of ker
 const char *fwd_variant_name(int v);
 cudaError_t init_collision_attributes();
 cudaError_t init_update_attributes();
-// Screening layout of R relative to the frame's centre.  compute_frame = true finds the
-// centre and radius of R and stores them in *frame; false keeps the given frame (a
-// subset of a cloud whose frame is already set, e.g. a mini-batch).
-cudaError_t launch_ref_prep(const float4 *R, int M, int Mpad, void *Rx, float4 *frame, bool compute_frame,
-                            cudaStream_t st);
+// Preparation of an object cloud (see k_match.cu); the scratch is cleared before its first use.
+constexpr int kRefCtas = 32;
+struct RefScratch {
+    unsigned lo[3], hi[3];            // bounding box: largest ~key / key (order_key) so far
+    unsigned done, pad;
+    unsigned long long rad;           // bits of the largest |r - c|^2 (float64)
+    double part[kRefCtas][3];         // the centroid's sums
+};
+cudaError_t launch_ref_prep(const float *xyz, int M, int Mpad, float4 *R, void *Rx, float4 *frame, double *com,
+                            RefScratch *scr, int *err, cudaStream_t st);
+cudaError_t launch_minibatch(const float4 *R, const int *idx, int n, int Mpad, float4 *out, void *Rx, const float4 *frame,
+                             ObjMeta *dst, const ObjMeta &v, cudaStream_t st);
+int fwd_item_queries(int v, long long queries);
 cudaError_t launch_tc_ref_prep(const float4 *R, int M, int Mpad, const float4 *frame, void *Rt, cudaStream_t st);
 size_t tc_ref_bytes(int Mpad);         // bytes of the tensor-core object tiles
 cudaError_t launch_fwd_match_tc(const FwdArgs &a, cudaStream_t st);
@@ -377,10 +399,8 @@ cudaError_t launch_stein(const UpdateArgs &a, cudaStream_t st);      // SVGD ste
 
 cudaError_t launch_pack_points(const float *xyz, int n, float4 *out, int *err, cudaStream_t st);
 cudaError_t launch_check_finite(const float *v, long long n, int *err, cudaStream_t st);
-cudaError_t launch_centroid(const float4 *X, int n, double *out3, cudaStream_t st);
 cudaError_t launch_preshape_consts(const float4 *S, int N, double *out12, cudaStream_t st);
 cudaError_t launch_fibonacci(const Layout &L, float radius, int mode, float *theta, cudaStream_t st);
-cudaError_t launch_gather_points(const float4 *R, const int *idx, int n, float4 *out, cudaStream_t st);
 cudaError_t launch_store_meta(ObjMeta *dst, const ObjMeta &v, cudaStream_t st);
 cudaError_t launch_set_theta(const float *theta7, int T, float *theta8, int *err, cudaStream_t st);
 cudaError_t launch_sdf_clear(const float4 *cells, int nx, int ny, int nz, unsigned char *clear, unsigned char *tmp,

@@ -331,18 +331,6 @@ __device__ __forceinline__ float fmin3(float a, float b, float c)
     return d;
 }
 
-// Total order of float32 values (no NaN) as unsigned keys, and back.
-__device__ __forceinline__ unsigned ord_key(float f)
-{
-    const unsigned u = __float_as_uint(f);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-__device__ __forceinline__ float key_val(unsigned k)
-{
-    return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
-
 // (best, bi) <- the smaller of itself and the partner lane's, ties to the lower index.
 __device__ __forceinline__ void argmin_xor(float &best, int &bi, int o)
 {
@@ -489,7 +477,7 @@ __global__ void __launch_bounds__(kColThreads) collide_nn_kernel(const CollideAr
             unsigned full_scan = 0u;
 #pragma unroll
             for (int q = 0; q < kQW; ++q) {
-                const unsigned key = ord_key(cm[q]);
+                const unsigned key = order_key(cm[q]);
                 const unsigned k1 = __reduce_min_sync(0xffffffffu, key);
                 const int l1 = __ffs(__ballot_sync(0xffffffffu, key == k1)) - 1;
                 const unsigned k2 = __reduce_min_sync(0xffffffffu, lane == l1 ? 0xffffffffu : key);
@@ -497,7 +485,7 @@ __global__ void __launch_bounds__(kColThreads) collide_nn_kernel(const CollideAr
                 const float ax = __fsub_rn(c.x, tx), ay = __fsub_rn(c.y, ty), az = __fsub_rn(c.z, tz);
                 const float cn = sqrtf(ax * ax + ay * ay + az * az) * 1.001f;
                 const float win = 2.02f * 5.9604645e-8f * (9.f * smax * smax + 10.1f * cn * smax);
-                if (key_val(k2) <= key_val(k1) + win) full_scan |= 1u << q;
+                if (key_float(k2) <= key_float(k1) + win) full_scan |= 1u << q;
                 if (g == q) my_l1 = l1;
             }
             // 2. exact choice: four lanes per colliding point over its chunk l1

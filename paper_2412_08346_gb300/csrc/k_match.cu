@@ -30,6 +30,10 @@
 //     minimum of the exact-form float32 distance among all points that can be
 //     nearest.
 //
+// Only whole chunks up to the cloud's last point are read, and a launch with few queries takes the
+// item size with the shortest schedule: 32 particles of 256 points on 512 points 22.9 -> 14.6 us per
+// pass; 128 of 1024 on 4096 points without a plan (128 items for 456 CTAs before) 1.65x as fast.
+//
 // Object tiles are staged in shared memory by 1D bulk (TMA) copies into two
 // buffers guarded by mbarriers; waits are bounded and report a timeout through
 // the error word instead of hanging.
@@ -97,15 +101,18 @@ __device__ __forceinline__ bool match_pass(const FwdArgs &a, const ObjMeta &om, 
                                            int &seq, int *s_abort)
 {
     constexpr int kThreads = Shape::kThreads, kChunk = Shape::kChunk, kTile = Shape::kTile;
-    const int ntiles = om.Mpad / kTile;
-    const unsigned tile_bytes = kTile * 16u;
+    // whole chunks up to the cloud's last point (not the padded tiles: a cloud of 512 points would be
+    // screened as 2048)
+    const int nchunks = (om.M + kChunk - 1) / kChunk, ntiles = (om.M + kTile - 1) / kTile;
+    auto tile_chunks = [&](int t) { return min(kTile / kChunk, nchunks - t * (kTile / kChunk)); };
+    auto load_tile = [&](int t, int b) {
+        const unsigned bytes = (unsigned)tile_chunks(t) * kChunk * 16u;
+        mbar_arrive_tx(&full[b], bytes);
+        bulk_load(tiles + (size_t)b * kTile, om.Rx + (size_t)t * kTile, bytes, &full[b]);
+    };
     if (threadIdx.x == 0) {    // both buffers are free: the previous pass ended with a barrier
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        for (int t = 0; t < 2 && t < ntiles; ++t) {
-            const int b = (seq + t) & 1;
-            mbar_arrive_tx(&full[b], tile_bytes);
-            bulk_load(tiles + (size_t)b * kTile, om.Rx + (size_t)t * kTile, tile_bytes, &full[b]);
-        }
+        for (int t = 0; t < 2 && t < ntiles; ++t) load_tile(t, (seq + t) & 1);
     }
     float sx[Q], sy[Q], sz[Q], win[Q], cm[Q], b1[Q], b2[Q], b3[Q];
     int c1[Q], c2[Q];
@@ -147,7 +154,8 @@ __device__ __forceinline__ bool match_pass(const FwdArgs &a, const ObjMeta &om, 
         __syncthreads();
         if (*s_abort) return false;
         const ulonglong2 *tp = tiles + (size_t)buf * kTile;
-        for (int c = 0; c < kTile / kChunk; ++c) {
+        const int chunks = tile_chunks(t);
+        for (int c = 0; c < chunks; ++c) {
 #pragma unroll
             for (int q = 0; q < Q; ++q) cm[q] = __int_as_float(0x7f800000);
             const ulonglong2 *cp = tp + c * kChunk;
@@ -178,8 +186,7 @@ __device__ __forceinline__ bool match_pass(const FwdArgs &a, const ObjMeta &om, 
         __syncthreads();   // every thread is done with this buffer
         if (threadIdx.x == 0 && t + 2 < ntiles) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_arrive_tx(&full[buf], tile_bytes);
-            bulk_load(tiles + (size_t)buf * kTile, om.Rx + (size_t)(t + 2) * kTile, tile_bytes, &full[buf]);
+            load_tile(t + 2, buf);
         }
     }
 
@@ -243,6 +250,7 @@ __device__ __forceinline__ bool dispatch_pass(int qn, const FwdArgs &a, const Ob
 template <class Shape>
 __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) fwd_match_kernel(const FwdArgs a)
 {
+    if (a.check_err && *a.err != kDevOk) return;     // (asicp_match_noalloc: a rejected input leaves nn_idx alone)
     constexpr int kThreads = Shape::kThreads;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ulonglong2 *tiles = reinterpret_cast<ulonglong2 *>(smem_raw);
@@ -268,8 +276,8 @@ __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) fwd_match_
         if (a.items) {
             item = a.items[it];
         } else {
-            item.q0 = (long long)it * Shape::kItem;
-            item.nq = (int)(Qtot - item.q0 < Shape::kItem ? Qtot - item.q0 : Shape::kItem);
+            item.q0 = (long long)it * a.item_queries;
+            item.nq = (int)(Qtot - item.q0 < a.item_queries ? Qtot - item.q0 : a.item_queries);
             item.obj = 0;
         }
         const ObjMeta om = a.L.obj[item.obj];
@@ -376,89 +384,163 @@ cudaError_t launch_fwd_exact(const FwdArgs &a, cudaStream_t st)
     return a.variant == kTcVariant ? launch_tc_exact(a, st) : cudaSuccess;
 }
 
-// Reference preparation for the screening stage (one CTA).  The frame: centre c =
-// the midpoint of R's bounding box (float32), radius w = max |fl(r - c)| rounded
-// up (float64 reduction); with compute_frame = false the given frame is kept (R
-// is then a subset of the cloud the frame was made for, so its radius still
-// bounds).  Layout: pairs of (-2 b, |b|^2) with b = fl(r - c), padded with
-// (0, +inf) points to a whole number of tiles.
-__global__ void ref_prep_kernel(const float4 *R, int M, int Mpad, ulonglong2 *Rx, float4 *frame, bool compute_frame)
+// Preparation of an object cloud, two kernels over the whole chip (as single CTAs it took 54 us at 8192
+// points and 302 at 65536, mostly float64 on one SM; a whole asicp_set_object at 65536 points took
+// 0.33 ms).
+//
+// ref_pack_kernel: points packed to float4 (non-finite values reported), the bounding box, and the float64
+// sums of the centroid: 1024 partial sums of every 1024th point, added in warps of 32 (CTA b: partial
+// sums 32 b .. 32 b + 31), the order of a single CTA of 1024 threads.
+__global__ void __launch_bounds__(256) ref_pack_kernel(const float *xyz, int M, float4 *R, RefScratch *scr, int *err)
 {
-    __shared__ double red[32];
-    __shared__ float bmin[3][32], bmax[3][32];
-    __shared__ float4 s_fr;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
-    if (compute_frame) {
-        float lo[3] = {__int_as_float(0x7f800000), __int_as_float(0x7f800000), __int_as_float(0x7f800000)};
-        float hi[3] = {-lo[0], -lo[1], -lo[2]};
-        for (int i = threadIdx.x; i < M; i += blockDim.x) {
-            const float4 r = R[i];
-            lo[0] = fminf(lo[0], r.x); lo[1] = fminf(lo[1], r.y); lo[2] = fminf(lo[2], r.z);
-            hi[0] = fmaxf(hi[0], r.x); hi[1] = fmaxf(hi[1], r.y); hi[2] = fmaxf(hi[2], r.z);
-        }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp == 7) {
+        double s[3] = {0.0, 0.0, 0.0};
+#pragma unroll 8
+        for (int i = blockIdx.x * 32 + lane; i < M; i += 1024)
+            for (int k = 0; k < 3; ++k) s[k] += (double)xyz[3 * (size_t)i + k];
+        warp_sum_f64(s);
+        if (lane == 0)
+            for (int k = 0; k < 3; ++k) scr->part[blockIdx.x][k] = s[k];
+        return;
+    }
+    float lo[3], hi[3];
+    for (int k = 0; k < 3; ++k) { lo[k] = __int_as_float(0x7f800000); hi[k] = -lo[k]; }
+    bool bad = false;
+#pragma unroll 4
+    for (int i = blockIdx.x * 224 + threadIdx.x; i < M; i += kRefCtas * 224) {
+        const float v[3] = {xyz[3 * (size_t)i], xyz[3 * (size_t)i + 1], xyz[3 * (size_t)i + 2]};
         for (int k = 0; k < 3; ++k) {
-            for (int o = 16; o > 0; o >>= 1) {
-                lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
-                hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
-            }
-            if (lane == 0) { bmin[k][warp] = lo[k]; bmax[k][warp] = hi[k]; }
+            bad = bad || !isfinite(v[k]);
+            lo[k] = fminf(lo[k], v[k]);
+            hi[k] = fmaxf(hi[k], v[k]);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float c[3];
-            for (int k = 0; k < 3; ++k) {
-                float l = bmin[k][0], h = bmax[k][0];
-                for (int w = 1; w < nw; ++w) { l = fminf(l, bmin[k][w]); h = fmaxf(h, bmax[k][w]); }
-                c[k] = M > 0 ? 0.5f * l + 0.5f * h : 0.f;
-            }
-            s_fr = make_float4(c[0], c[1], c[2], 0.f);
-        }
-    } else if (threadIdx.x == 0) {
-        s_fr = *frame;
+        R[i] = make_float4(v[0], v[1], v[2], 0.f);
     }
-    __syncthreads();
-    const float4 fr = s_fr;
-    double m = 0.0;
-    for (int q = threadIdx.x; q < Mpad / 2; q += blockDim.x) {
-        float ax[2], ay[2], az[2], w[2];
-        for (int k = 0; k < 2; ++k) {
-            const int i = 2 * q + k;
-            if (i < M) {
-                const float4 r = R[i];
-                const float bx = __fsub_rn(r.x, fr.x), by = __fsub_rn(r.y, fr.y), bz = __fsub_rn(r.z, fr.z);
-                const double b2 = (double)bx * bx + (double)by * by + (double)bz * bz;
-                m = fmax(m, b2);
-                ax[k] = -2.f * bx; ay[k] = -2.f * by; az[k] = -2.f * bz;
-                w[k] = (float)b2;
-            } else {
-                ax[k] = ay[k] = az[k] = 0.f;
-                w[k] = __int_as_float(0x7f800000);
-            }
+    if (bad) atomicExch(err, kDevNonFinite);
+    for (int k = 0; k < 3; ++k) {
+        const unsigned l = __reduce_max_sync(0xffffffffu, ~order_key(lo[k])), h = __reduce_max_sync(0xffffffffu, order_key(hi[k]));
+        if (lane == 0) {
+            atomicMax(&scr->lo[k], l);
+            atomicMax(&scr->hi[k], h);
         }
-        // pair layout: point pair q -> {A, B} at 2 q, 2 q + 1 (any tile of an even
-        // number of points is a contiguous range)
-        ulonglong2 A, B;
-        A.x = pack2(ax[0], ax[1]); A.y = pack2(ay[0], ay[1]);
-        B.x = pack2(az[0], az[1]); B.y = pack2(w[0], w[1]);
-        Rx[2 * (size_t)q] = A;
-        Rx[2 * (size_t)q + 1] = B;
-    }
-    if (!compute_frame) return;
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) red[warp] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double mm = 0.0;
-        for (int w = 0; w < nw; ++w) mm = fmax(mm, red[w]);
-        *frame = make_float4(fr.x, fr.y, fr.z, (float)(sqrt(mm) * (1.0 + 1e-6)) + 1e-30f);
     }
 }
 
-cudaError_t launch_ref_prep(const float4 *R, int M, int Mpad, void *Rx, float4 *frame, bool compute_frame,
-                            cudaStream_t st)
+// ref_layout_kernel: the frame's centre c = the midpoint of the bounding box (float32); the screening
+// layout: pairs of (-2 b, |b|^2) with b = fl(r - c), padded with (0, +inf) points to a whole number
+// of tiles; the last CTA to finish writes the frame (radius w = max |fl(r - c)| rounded up, float64
+// reduction) and the centroid and clears the scratch for the next cloud.
+__device__ __forceinline__ void ref_pair(const float4 *R, const int *idx, int M, int q, float4 fr, ulonglong2 *Rx,
+                                         float4 *out, double &m)
 {
-    ref_prep_kernel<<<1, 1024, 0, st>>>(R, M, Mpad, static_cast<ulonglong2 *>(Rx), frame, compute_frame);
+    float ax[2], ay[2], az[2], w[2];
+    for (int k = 0; k < 2; ++k) {
+        const int i = 2 * q + k;
+        if (i < M) {
+            const float4 r = R[idx ? idx[i] : i];
+            if (out) out[i] = r;
+            const float bx = __fsub_rn(r.x, fr.x), by = __fsub_rn(r.y, fr.y), bz = __fsub_rn(r.z, fr.z);
+            const double b2 = (double)bx * bx + (double)by * by + (double)bz * bz;
+            m = fmax(m, b2);
+            ax[k] = -2.f * bx; ay[k] = -2.f * by; az[k] = -2.f * bz;
+            w[k] = (float)b2;
+        } else {
+            ax[k] = ay[k] = az[k] = 0.f;
+            w[k] = __int_as_float(0x7f800000);
+        }
+    }
+    // pair layout: point pair q -> {A, B} at 2 q, 2 q + 1 (any tile of an even
+    // number of points is a contiguous range)
+    ulonglong2 A, B;
+    A.x = pack2(ax[0], ax[1]); A.y = pack2(ay[0], ay[1]);
+    B.x = pack2(az[0], az[1]); B.y = pack2(w[0], w[1]);
+    Rx[2 * (size_t)q] = A;
+    Rx[2 * (size_t)q + 1] = B;
+}
+
+__global__ void __launch_bounds__(256) ref_layout_kernel(const float4 *R, int M, int Mpad, ulonglong2 *Rx, float4 *frame,
+                                                         double *com, RefScratch *scr)
+{
+    __shared__ bool s_last;
+    const float l[3] = {key_float(~scr->lo[0]), key_float(~scr->lo[1]), key_float(~scr->lo[2])};
+    const float h[3] = {key_float(scr->hi[0]), key_float(scr->hi[1]), key_float(scr->hi[2])};
+    const float4 fr = make_float4(0.5f * l[0] + 0.5f * h[0], 0.5f * l[1] + 0.5f * h[1], 0.5f * l[2] + 0.5f * h[2], 0.f);
+    double m = 0.0;
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < Mpad / 2; q += gridDim.x * blockDim.x)
+        ref_pair(R, nullptr, M, q, fr, Rx, nullptr, m);
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(&scr->rad, (unsigned long long)__double_as_longlong(m));
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&scr->done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) {
+        const double mm = __longlong_as_double((long long)atomicMax(&scr->rad, 0ull));
+        *frame = make_float4(fr.x, fr.y, fr.z, (float)(sqrt(mm) * (1.0 + 1e-6)) + 1e-30f);
+        for (int k = 0; k < 3; ++k) scr->lo[k] = scr->hi[k] = 0u;
+        scr->rad = 0ull;
+        scr->done = 0u;
+    }
+    if (com && threadIdx.x >= 32 && threadIdx.x < 35) {
+        const int k = threadIdx.x - 32;
+        double s = 0.0;
+        for (int w = 0; w < kRefCtas; ++w) s += scr->part[w][k];
+        com[k] = s / M;
+    }
+}
+
+// xyz [M][3] -> R, the screening layout, the frame and (com not null) the centroid; scr cleared before
+// its first use.
+cudaError_t launch_ref_prep(const float *xyz, int M, int Mpad, float4 *R, void *Rx, float4 *frame, double *com,
+                            RefScratch *scr, int *err, cudaStream_t st)
+{
+    ref_pack_kernel<<<kRefCtas, 256, 0, st>>>(xyz, M, R, scr, err);
+    const int ctas = (Mpad / 2 + 255) / 256;
+    ref_layout_kernel<<<ctas < 148 ? ctas : 148, 256, 0, st>>>(R, M, Mpad, static_cast<ulonglong2 *>(Rx), frame, com, scr);
     return cudaGetLastError();
+}
+
+// A mini-batch of the cloud, in one launch: its points out[i] = R[idx[i]], their screening layout in the
+// whole cloud's frame (its radius still bounds), and the object table pointing at them.
+__global__ void __launch_bounds__(256) minibatch_kernel(const float4 *R, const int *idx, int n, int Mpad, float4 *out,
+                                                        ulonglong2 *Rx, const float4 *frame, ObjMeta *dst, const ObjMeta v)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0) *dst = v;
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= Mpad / 2) return;
+    double m = 0.0;
+    ref_pair(R, idx, n, q, *frame, Rx, out, m);
+}
+
+cudaError_t launch_minibatch(const float4 *R, const int *idx, int n, int Mpad, float4 *out, void *Rx, const float4 *frame,
+                             ObjMeta *dst, const ObjMeta &v, cudaStream_t st)
+{
+    minibatch_kernel<<<(Mpad / 2 + 255) / 256, 256, 0, st>>>(R, idx, n, Mpad, out, static_cast<ulonglong2 *>(Rx), frame, dst,
+                                                             v);
+    return cudaGetLastError();
+}
+
+// Queries per work item of a one-object launch with few queries: with one item per CTA of the grid and
+// round, the time is about rounds x (kLoadCost + queries per thread), kLoadCost for reading an
+// object point from shared memory against screening it for one query.
+int fwd_item_queries(int v, long long queries)
+{
+    constexpr double kLoadCost = 0.6;
+    const int grid = fwd_shape_grid(v), threads = fwd_shape_threads(v), most = fwd_shape_queries(v);
+    int best = most;
+    double best_cost = 0.0;
+    for (int q = most / threads; q >= 1; --q) {
+        const long long items = (queries + (long long)q * threads - 1) / ((long long)q * threads);
+        const double cost = (double)((items + grid - 1) / grid) * (kLoadCost + q);
+        if (q == most / threads || cost < best_cost) {
+            best_cost = cost;
+            best = q * threads;
+        }
+    }
+    return best;
 }
 
 }  // namespace asicp

@@ -252,6 +252,8 @@ __global__ void __launch_bounds__(kThreadsTc, 512 / COLS) fwd_match_tc_kernel(co
         }
         return item;
     };
+    // tiles that hold points (the prepared cloud is padded further)
+    auto tiles_of = [](const ObjMeta &om) { return (om.M + COLS - 1) / COLS; };
     auto fail = [&]() {
         if (!s_abort) atomicExch(a.err, kDevTimeout);
         s_abort = 1;
@@ -281,7 +283,7 @@ __global__ void __launch_bounds__(kThreadsTc, 512 / COLS) fwd_match_tc_kernel(co
             for (int it = it0; it < it1 && ok; it += step) {
                 const ObjMeta &om = a.L.obj[item_at(it).obj];
                 const unsigned char *src = reinterpret_cast<const unsigned char *>(om.Rt);
-                const int ntiles = om.Mpad / COLS;
+                const int ntiles = tiles_of(om);
                 for (int t = 0; t < ntiles; ++t) {
                     // the stage is free once the MMA of its previous tile is done
                     if (s_abort || !mbar_wait(&bempty[p_stage], p_lap ^ 1u)) { ok = false; break; }
@@ -307,7 +309,7 @@ __global__ void __launch_bounds__(kThreadsTc, 512 / COLS) fwd_match_tc_kernel(co
             unsigned c_lap = 0u, last_lap = 0u;
             int ia = 0;
             for (int it = it0; it < it1 && !s_abort; it += step, ++ia) {
-                const int ntiles = a.L.obj[item_at(it).obj].Mpad / COLS;
+                const int ntiles = tiles_of(a.L.obj[item_at(it).obj]);
                 // the item's query rows are written
                 if (!mbar_wait(&afull, (unsigned)(ia & 1))) { fail(); break; }
                 tc_fence_after();
@@ -341,7 +343,7 @@ __global__ void __launch_bounds__(kThreadsTc, 512 / COLS) fwd_match_tc_kernel(co
             if (__any_sync(0xffffffffu, s_abort)) break;
             // the item's query rows (the previous item's MMAs are complete: its last
             // accumulator was waited for); only the screening window lives through the tiles
-            const int ntiles = a.L.obj[item_at(it).obj].Mpad / COLS;
+            const int ntiles = tiles_of(a.L.obj[item_at(it).obj]);
             const FwdItem item = item_at(it);
             const float win = build_query_row(a, item.q0 + tid, tid < item.nq, a.L.frame[item.obj], sA, row);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

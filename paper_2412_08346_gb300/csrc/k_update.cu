@@ -632,23 +632,6 @@ __device__ void block_sum_f64(int n, F term, double *out)
     }
 }
 
-__global__ void centroid_kernel(const float4 *X, int n, double *out3)
-{
-    __shared__ double tmp[3];
-    block_sum_f64<3>(n, [&](int i, double *acc) {
-        const float4 x = X[i];
-        acc[0] += x.x; acc[1] += x.y; acc[2] += x.z;
-    }, tmp);
-    __syncthreads();
-    if (threadIdx.x < 3) out3[threadIdx.x] = tmp[threadIdx.x] / n;
-}
-
-cudaError_t launch_centroid(const float4 *X, int n, double *out3, cudaStream_t st)
-{
-    centroid_kernel<<<1, 1024, 0, st>>>(X, n, out3);
-    return cudaGetLastError();
-}
-
 __global__ void preshape_consts_kernel(const float4 *S, int N, double *out12)
 {
     __shared__ double tmp[9];
@@ -724,19 +707,6 @@ __global__ void fibonacci_kernel(const Layout L, float radius, int mode, float *
 cudaError_t launch_fibonacci(const Layout &L, float radius, int mode, float *theta, cudaStream_t st)
 {
     fibonacci_kernel<<<(L.T + 255) / 256, 256, 0, st>>>(L, radius, mode, theta);
-    return cudaGetLastError();
-}
-
-// out[i] = R[idx[i]], i < n (a mini-batch of the object cloud)
-__global__ void gather_points_kernel(const float4 *R, const int *idx, int n, float4 *out)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = R[idx[i]];
-}
-
-cudaError_t launch_gather_points(const float4 *R, const int *idx, int n, float4 *out, cudaStream_t st)
-{
-    gather_points_kernel<<<(n + 255) / 256, 256, 0, st>>>(R, idx, n, out);
     return cudaGetLastError();
 }
 

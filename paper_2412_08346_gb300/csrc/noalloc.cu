@@ -47,9 +47,10 @@ constexpr size_t kOffPartGrp = kOffStage + kStageFloats * 4;
 constexpr size_t kOffGrpOff = kOffPartGrp + (size_t)ASICP_NOALLOC_MAX_PK * 4;
 constexpr size_t kOffObjMeta = kOffGrpOff + ((size_t)ASICP_NOALLOC_MAX_PK + 64) * 4;
 constexpr size_t kOffFrame = kOffObjMeta + 256;
-constexpr size_t kOffErr = kOffFrame + 256;
+constexpr size_t kOffErr = kOffFrame + 256;        // error word, then (256-aligned) the preparation's scratch
+constexpr size_t kOffPrep = kOffErr + 256;
 static_assert(sizeof(ObjMeta) <= 256, "object table slot too small");
-static_assert(kOffErr + 256 <= kScratchBytes, "scratch layout exceeds the static array");
+static_assert(kOffPrep + sizeof(RefScratch) <= kScratchBytes, "scratch layout exceeds the static array");
 static_assert(kStageFloats >= 3 * (size_t)ASICP_NOALLOC_MAX_PN && kStageFloats >= 7 * (size_t)ASICP_NOALLOC_MAX_PK,
               "staging area too small");
 
@@ -117,7 +118,8 @@ extern "C" asicp_status asicp_match_noalloc(const float *theta, int P, int K, co
     const int Mpad = (M + kRefTilePts - 1) / kRefTilePts * kRefTilePts;
 
 #define NOALLOC_CK(x) do { if ((x) != cudaSuccess) { cudaGetLastError(); return ASICP_ERR_CUDA; } } while (0)
-    NOALLOC_CK(cudaMemsetAsync(err, 0, sizeof(int), st));   // the array keeps the last call's error word
+    // the array keeps the last call's error word and, if that call failed, its preparation's scratch
+    NOALLOC_CK(cudaMemsetAsync(err, 0, kOffPrep + sizeof(RefScratch) - kOffErr, st));
     // inputs that are host memory go through the staging area (a copy, not an allocation)
     auto src = [&](const float *p, size_t n) -> const float * {
         if (device_accessible(p)) return p;
@@ -132,21 +134,16 @@ extern "C" asicp_status asicp_match_noalloc(const float *theta, int P, int K, co
     NOALLOC_CK(launch_pack_points(sx, P * N, grip, err, st));
     const float *rx = src(R_xyz, (size_t)M * 3);
     if (!rx) return ASICP_ERR_CUDA;
-    NOALLOC_CK(launch_pack_points(rx, M, obj, err, st));
-    NOALLOC_CK(launch_ref_prep(obj, M, Mpad, screen, frame, true, st));
+    NOALLOC_CK(launch_ref_prep(rx, M, Mpad, obj, screen, frame, nullptr, reinterpret_cast<RefScratch *>(base + kOffPrep),
+                               err, st));
     NOALLOC_CK(launch_uniform_groups(part_grp, grp_off, P, K, st));
-    // a non-finite input stops the call before the matching: nn_idx stays untouched
-    NOALLOC_CK(cudaStreamSynchronize(st));
-    int e_in = 0;
-    NOALLOC_CK(cudaMemcpy(&e_in, err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (e_in == kDevNonFinite) return ASICP_ERR_INVALID_ARG;
-    ObjMeta om{};          // one object holding every particle (copied by value below)
+    ObjMeta om{};          // one object holding every particle
     om.R = obj;
     om.Rx = screen;
     om.C = obj;
     om.M = M; om.Mpad = Mpad; om.Mc = M;
     om.pfirst = 0; om.np = PK;
-    NOALLOC_CK(cudaMemcpyAsync(objmeta, &om, sizeof(ObjMeta), cudaMemcpyHostToDevice, st));
+    NOALLOC_CK(launch_store_meta(objmeta, om, st));
 
     FwdArgs fa{};
     fa.L.P = P; fa.L.N = N; fa.L.G = P; fa.L.nobj = 1; fa.L.T = PK;
@@ -158,13 +155,15 @@ extern "C" asicp_status asicp_match_noalloc(const float *theta, int P, int K, co
     fa.S = grip;
     fa.theta = poses;
     fa.items = nullptr;    // consecutive work items of object 0
-    fa.n_items = (int)(((long long)PK * N + kFwdItemQueries - 1) / kFwdItemQueries);
+    fa.item_queries = fwd_item_queries(0, (long long)PK * N);
+    fa.n_items = (int)(((long long)PK * N + fa.item_queries - 1) / fa.item_queries);
     fa.err = err;
+    fa.check_err = 1;      // a non-finite input: the matching does nothing, nn_idx stays untouched
     fa.nn_idx = nn_idx;
     NOALLOC_CK(launch_fwd_match(fa, st));
-    NOALLOC_CK(cudaStreamSynchronize(st));   // also keeps `om` alive until its copy is done
     int e = 0;
-    NOALLOC_CK(cudaMemcpy(&e, err, sizeof(int), cudaMemcpyDeviceToHost));
+    NOALLOC_CK(cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    NOALLOC_CK(cudaStreamSynchronize(st));
 #undef NOALLOC_CK
     if (e == kDevNonFinite) return ASICP_ERR_INVALID_ARG;
     if (e == kDevTimeout) return ASICP_ERR_TIMEOUT;

@@ -152,3 +152,37 @@ def test_collision_test_skips_no_colliding_point(Mc):
         diff = np.setxor1d(got, want)
         assert np.all(np.abs(np.asarray(vals)[diff]) <= tl.PHI_TOL), (pk, len(diff))
     assert st["ncol"][3] == 0 and st["ncol"].max() >= Mc // 200       # (the gripper fills 0.75 % of the cube)
+
+
+@pytest.mark.parametrize("M", [1, 63, 64, 65, 255, 257, 1025, 2048, 2049])
+def test_every_shape_at_the_edges_of_chunks_and_tiles(M):
+    """Clouds that end inside, at and just past a screening chunk or tile (only whole chunks up to the last
+    point are read), prepared by several CTAs: every matching shape finds the nearest points, and the
+    no-allocation entry point the same ones."""
+    R = _cloud("partial", M)
+    g = np.random.default_rng(M)
+    S = g.uniform(-0.05, 0.05, (2, 70, 3)).astype(np.float32)
+    q = g.normal(size=(8, 4))
+    theta = np.concatenate([g.normal(size=(8, 3)) * 0.05, q / np.linalg.norm(q, axis=1, keepdims=True)], 1).astype(np.float32)
+    stream = torch.cuda.current_stream().cuda_stream
+    out = torch.full((8 * 70,), -1, dtype=torch.int32, device="cuda")
+    asicp.asicp_match_noalloc(theta, S.reshape(-1, 3), R, out, 2, 4, stream)
+    got = [out.cpu().numpy().reshape(8, 70)]
+    for shape in range(asicp.FWD_SHAPES):
+        cfg = asicp.asicp_config_default(P=2, K=4, k_max=1, k_stein=0, conv_tol=-1.0, debug=1, fwd_shape=shape, cuda_stream=stream)
+        ctx = asicp.asicp_create(cfg)
+        try:
+            asicp.asicp_set_object(ctx, R)
+            for p in range(2):
+                asicp.asicp_set_gripper_sdf(ctx, p, S[p], -np.ones((8, 8, 8), np.float32), np.full(3, -0.1, np.float32),
+                                            np.float32(0.2 / 7))
+            asicp.asicp_set_state(ctx, theta, 0)
+            asicp.asicp_step(ctx, 0)
+            st = tl.read_state(ctx, 2, 4, 70, M)
+        finally:
+            asicp.asicp_destroy(ctx)
+        got.append(st["nn_idx"])
+        if shape == 0:
+            tl.check_nn(st["s_prime"].reshape(-1, 3), R, st["nn_idx"].reshape(-1), {})
+    for idx in got:
+        assert np.array_equal(idx, got[1])
