@@ -69,6 +69,47 @@ struct DevMem {
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
 
+// Page-locked host memory that inputs and results of at most kPinPiece bytes pass through; grows on
+// demand up to kPinMost.  Larger pieces (or without memory) are copied straight between the caller's
+// arrays and the device.
+constexpr size_t kPinPiece = (size_t)256 << 10, kPinMost = (size_t)2 << 20;
+struct PinMem {
+    unsigned char *p = nullptr;
+    size_t bytes = 0;
+    PinMem() = default;
+    PinMem(const PinMem &) = delete;
+    PinMem &operator=(const PinMem &) = delete;
+    ~PinMem() { if (p) cudaFreeHost(p); }
+    bool ensure(size_t want)       // (contents are not kept; no copy may be in flight)
+    {
+        if (want <= bytes) return true;
+        if (want > kPinMost) return false;
+        if (p) cudaFreeHost(p);
+        p = nullptr;
+        bytes = 0;
+        want = std::max(want, (size_t)64 << 10);
+        void *q = nullptr;
+        if (cudaHostAlloc(&q, want, cudaHostAllocDefault) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        p = static_cast<unsigned char *>(q);
+        bytes = want;
+        return true;
+    }
+};
+
+// Ordinary host memory, which an asynchronous copy would have to stage.
+bool pageable(const void *p)
+{
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeUnregistered;
+}
+
 struct ObjBufs {
     DevMem R, Rx, Rt, C;      // C stays empty when the collision cloud is R itself
     DevMem nodes, leaves;     // matching cells of R
@@ -112,7 +153,6 @@ struct asicp_ctx {
 
     // mini-batches of the object cloud per iteration (Table I), one object only
     std::vector<int> mb_off;          // [iters + 1] on the host (sizes are fixed at capture)
-    long long mb_version = 0;         // bumped by every asicp_set_minibatch
     DevMem mb_idx, mb_R, mb_Rx;
 
     int fwd_variant = 0;              // forward-matching kernel shape (autotuner's choice)
@@ -142,7 +182,18 @@ struct asicp_ctx {
     double acc_ms[kTimeKinds] = {};
     long long acc_n[kTimeKinds] = {};
 
+    // results on their way to the caller (flushed by finish()) and the page-locked memory they and the
+    // inputs pass through; pin_busy: a copy from it has been enqueued and not waited for
+    struct Out { void *dst; const void *src; size_t bytes; };
+    std::vector<Out> outs;
+    PinMem pin, pin_in;
+    bool pin_busy = false;
+    size_t pin_used = 0;              // bytes of pin_in taken by copies in flight
+    DevMem outp, outg;                // phi and gradient as they are returned
+
     // CUDA graph of asicp_run's iteration loop (captured once per buffer layout)
+    std::vector<int> loop_mb;         // mini-batch offsets it was captured with, and the object's entry
+    ObjMeta loop_meta{};
     cudaStream_t cap_st = nullptr;
     cudaGraphExec_t loop_exec = nullptr;
     std::vector<const void *> loop_key;
@@ -211,19 +262,102 @@ asicp_status guarded(asicp_ctx *ctx, F &&f)
     }
 }
 
-void sync_and_check_err(asicp_ctx *c, const char *what)
+// Results of a call, copied as 32-bit words into page-locked memory by one kernel: word 0 is the error
+// word, the pieces follow.
+constexpr int kPieces = 8;
+struct OutPieces {
+    const unsigned *src[kPieces];
+    unsigned words[kPieces];
+    int n;
+};
+__global__ void collect_kernel(const OutPieces o, const int *err, unsigned *dst)
 {
-    ck(cudaStreamSynchronize(c->st), what);
-    int e = 0;
-    ck(cudaMemcpy(&e, c->errw.p, sizeof(int), cudaMemcpyDeviceToHost), "read error word");
-    if (e == kDevNonFinite) {
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    if (i == 0) dst[0] = (unsigned)*err;
+    unsigned base = 4;                     // (16 bytes: the pieces stay aligned for any type)
+    for (int k = 0; k < o.n; ++k) {
+        for (unsigned w = i; w < o.words[k]; w += step) dst[base + w] = o.src[k][w];
+        base += (o.words[k] + 3u) & ~3u;
+    }
+}
+
+// Enqueue a result: it is in the caller's array when finish() returns.
+void copy_out(asicp_ctx *c, void *dst, const void *src, size_t bytes)
+{
+    if (dst && bytes) c->outs.push_back({dst, src, bytes});
+}
+
+// Wait for the stream, once: with the results asked for and the error word in page-locked memory; then
+// hand the results over, or report the error.
+void finish(asicp_ctx *c, const char *what)
+{
+    OutPieces o{};
+    std::vector<asicp_ctx::Out> staged;
+    size_t total = 16;
+    for (const auto &x : c->outs) {
+        const size_t room = (x.bytes + 15) / 16 * 16;
+        if (o.n < kPieces && x.bytes % 4 == 0 && x.bytes <= kPinPiece && total + room <= kPinMost && pageable(x.dst)) {
+            o.src[o.n] = static_cast<const unsigned *>(x.src);
+            o.words[o.n++] = (unsigned)(x.bytes / 4);
+            total += room;
+            staged.push_back(x);
+        } else {
+            const cudaError_t e = cudaMemcpyAsync(x.dst, x.src, x.bytes, cudaMemcpyDefault, c->st);
+            if (e != cudaSuccess) c->outs.clear();
+            ck(e, what);
+        }
+    }
+    int err = 0;
+    if (c->pin.ensure(total)) {
+        const int blocks = (int)std::min<size_t>((total / 4 + 255) / 256, 128);
+        collect_kernel<<<blocks, 256, 0, c->st>>>(o, c->errw.as<int>(), reinterpret_cast<unsigned *>(c->pin.p));
+        c->outs.clear();
+        ck(cudaGetLastError(), what);
+        ck(cudaStreamSynchronize(c->st), what);
+        err = *reinterpret_cast<const int *>(c->pin.p);
+        size_t at = 16;
+        for (const auto &x : staged) {
+            if (err == kDevOk) std::memcpy(x.dst, c->pin.p + at, x.bytes);
+            at += (x.bytes + 15) / 16 * 16;
+        }
+    } else {
+        c->outs.clear();
+        for (const auto &x : staged) ck(cudaMemcpyAsync(x.dst, x.src, x.bytes, cudaMemcpyDefault, c->st), what);
+        ck(cudaMemcpyAsync(&err, c->errw.p, sizeof(int), cudaMemcpyDeviceToHost, c->st), what);
+        ck(cudaStreamSynchronize(c->st), what);
+    }
+    c->pin_busy = false;
+    if (err == kDevNonFinite) {
         ck(cudaMemsetAsync(c->errw.p, 0, sizeof(int), c->st), "clear error word");
         fail(ASICP_ERR_INVALID_ARG, std::string(what) + ": non-finite value in the input");
     }
-    if (e == kDevTimeout) {
+    if (err == kDevTimeout) {
         ck(cudaMemsetAsync(c->errw.p, 0, sizeof(int), c->st), "clear error word");
         fail(ASICP_ERR_TIMEOUT, std::string(what) + ": a bounded device wait expired");
     }
+}
+
+// Enqueue the copy of an input; the source may be reused once the call has returned (pageable memory is
+// copied here and now, other memory by the time of finish()).
+void upload(asicp_ctx *c, void *dst, const void *src, size_t bytes, const char *what)
+{
+    if (bytes > 0 && bytes <= kPinPiece && pageable(src)) {
+        if (!c->pin_busy) c->pin_used = 0;
+        if (c->pin_busy && c->pin_used + bytes > c->pin_in.bytes) {
+            ck(cudaStreamSynchronize(c->st), what);
+            c->pin_busy = false;
+            c->pin_used = 0;
+        }
+        if (c->pin_busy || c->pin_in.ensure(bytes)) {
+            unsigned char *at = c->pin_in.p + c->pin_used;
+            std::memcpy(at, src, bytes);
+            c->pin_busy = true;
+            c->pin_used += (bytes + 255) / 256 * 256;
+            ck(cudaMemcpyAsync(dst, at, bytes, cudaMemcpyHostToDevice, c->st), what);
+            return;
+        }
+    }
+    ck(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, c->st), what);
 }
 
 double gamma_of(const asicp_config &c, int k)
@@ -752,7 +886,7 @@ std::vector<const void *> loop_key(const asicp_ctx *c)
             c->S.p, c->pconst.p, c->dmeta.p, c->theta.p, c->ncol.p, c->colidx.p, c->colsrt.p, c->colnn.p, c->colmap.p, c->cost.p,
             c->grad.p, c->prev.p, c->frozen.p, c->phi.p, c->h.p, c->order.p, c->errw.p, c->nnidx.p, c->tccand.p, c->dbg_d2.p,
             c->dbg_sp.p, c->mb_idx.p, c->mb_R.p, c->mb_Rx.p,
-            reinterpret_cast<const void *>((size_t)c->mb_version), reinterpret_cast<const void *>((size_t)c->T),
+            reinterpret_cast<const void *>((size_t)c->T),
             reinterpret_cast<const void *>((size_t)c->G), reinterpret_cast<const void *>((size_t)c->n_items),
             reinterpret_cast<const void *>((size_t)c->N), reinterpret_cast<const void *>((size_t)c->fwd_variant),
             reinterpret_cast<const void *>((size_t)c->expire_test), c->Ssort.p,
@@ -766,7 +900,10 @@ std::vector<const void *> loop_key(const asicp_ctx *c)
 void run_loop_graph(asicp_ctx *c)
 {
     std::vector<const void *> key = loop_key(c);
-    if (!c->loop_exec || key != c->loop_key) {
+    // (mini-batches: their sizes and the object's entry are in the graph, the indices are read at replay)
+    const bool same_mb = c->mb_off == c->loop_mb &&
+                         (c->mb_off.empty() || std::memcmp(&c->loop_meta, &c->objmeta_h[0], sizeof(ObjMeta)) == 0);
+    if (!c->loop_exec || key != c->loop_key || !same_mb) {
         if (c->loop_exec) {
             cudaGraphExecDestroy(c->loop_exec);
             c->loop_exec = nullptr;
@@ -792,16 +929,12 @@ void run_loop_graph(asicp_ctx *c)
         cudaGraphDestroy(g);
         ck(e, "instantiate graph");
         c->loop_key = key;
+        c->loop_mb = c->mb_off;
+        c->loop_meta = c->objmeta_h[0];
     }
     accumulate_graph_events(c);
     ck(cudaGraphLaunch(c->loop_exec, c->st), "graph launch");
     c->graph_pending = c->cfg.profile != 0;
-}
-
-void copy_out(void *dst, const void *src, size_t bytes, cudaStream_t st, const char *what)
-{
-    if (!dst || bytes == 0) return;
-    ck(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, st), what);
 }
 
 __global__ void repack_kernel(const float *src8, int n, float *dst7)
@@ -874,7 +1007,7 @@ void autotune_impl(asicp_ctx *c, float *ms_out)
     }
     c->pool.push_back(e0);
     c->pool.push_back(e1);
-    sync_and_check_err(c, "autotune");
+    finish(c, "autotune");
     c->fwd_variant = best_v;
     plan_fwd_items(c, best_v);
     c->tuned = true;
@@ -889,7 +1022,6 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
     const int mc = C_xyz ? Mc : M;
     if (!ctx->mb_off.empty()) {   // mini-batches index the previous cloud
         ctx->mb_off.clear();
-        ++ctx->mb_version;
     }
     // what the layout (object table, work plan) and the captured loop depend on
     const bool was_set = b.set;
@@ -901,7 +1033,7 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
     ctx->run_done = false;
     ctx->stage.ensure(sizeof(float) * 3 * (size_t)(M > mc ? M : mc), "staging");
     b.R.ensure(sizeof(float4) * M, "object cloud");
-    ck(cudaMemcpyAsync(ctx->stage.p, R_xyz, sizeof(float) * 3 * (size_t)M, cudaMemcpyDefault, ctx->st), "copy R");
+    upload(ctx, ctx->stage.p, R_xyz, sizeof(float) * 3 * (size_t)M, "copy R");
     const int Mpad = (M + kRefTilePts - 1) / kRefTilePts * kRefTilePts;
     b.Rx.ensure(sizeof(float4) * (size_t)Mpad, "screening layout");
     ck(launch_ref_prep(ctx->stage.as<float>(), M, Mpad, b.R.as<float4>(), b.Rx.p, ctx->frame.as<float4>() + o,
@@ -909,7 +1041,7 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
        "ref prep");
     if (C_xyz) {
         b.C.ensure(sizeof(float4) * mc, "collision cloud");
-        ck(cudaMemcpyAsync(ctx->stage.p, C_xyz, sizeof(float) * 3 * (size_t)mc, cudaMemcpyDefault, ctx->st), "copy C");
+        upload(ctx, ctx->stage.p, C_xyz, sizeof(float) * 3 * (size_t)mc, "copy C");
         ck(launch_pack_points(ctx->stage.as<float>(), mc, b.C.as<float4>(), ctx->errw.as<int>(), ctx->st), "pack C");
     } else {
         b.C.release();
@@ -919,7 +1051,7 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
     b.Rt.ensure(tc_ref_bytes(Mpad), "tensor-core object tiles");
     ck(launch_tc_ref_prep(b.R.as<float4>(), M, Mpad, ctx->frame.as<float4>() + o, b.Rt.p, ctx->st),
        "tensor-core ref prep");
-    sync_and_check_err(ctx, "set_object");
+    finish(ctx, "set_object");
     b.M = M;
     b.Mpad = Mpad;
     b.Mc = mc;
@@ -1052,7 +1184,6 @@ asicp_status asicp_set_particle_counts(asicp_ctx *ctx, const int *K, int n)
 asicp_status asicp_set_minibatch(asicp_ctx *ctx, const int *offsets, const int *indices, int iters)
 {
     return guarded(ctx, [&] {
-        ++ctx->mb_version;
         if (!offsets) {
             ctx->mb_off.clear();
             return;
@@ -1078,7 +1209,9 @@ asicp_status asicp_set_minibatch(asicp_ctx *ctx, const int *offsets, const int *
         ctx->mb_idx.ensure(sizeof(int) * idx.size(), "mini-batch indices");
         ctx->mb_R.ensure(sizeof(float4) * M, "mini-batch points");
         ctx->mb_Rx.ensure(sizeof(float4) * Mpad, "mini-batch screening layout");
-        ck(cudaMemcpy(ctx->mb_idx.p, idx.data(), sizeof(int) * idx.size(), cudaMemcpyHostToDevice), "upload indices");
+        upload(ctx, ctx->mb_idx.p, idx.data(), sizeof(int) * idx.size(), "upload indices");
+        ck(cudaStreamSynchronize(ctx->st), "upload indices");
+        ctx->pin_busy = false;
         ctx->mb_off = off;
         ctx->run_done = false;
     });
@@ -1130,7 +1263,7 @@ asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_
         ctx->stage.ensure(nc, "staging");
         ck(launch_sdf_clear(ctx->cells[preshape].as<float4>(), nx, ny, nz, ctx->clear[preshape].as<unsigned char>(),
                             ctx->stage.as<unsigned char>(), ctx->st), "sdf clearances");
-        sync_and_check_err(ctx, "set_gripper_sdf");
+        finish(ctx, "set_gripper_sdf");
         SdfMeta m{};
         m.grid = ctx->grids[preshape].as<float>();
         m.cells = ctx->cells[preshape].as<float4>();
@@ -1154,11 +1287,11 @@ asicp_status asicp_set_state(asicp_ctx *ctx, const float *theta, int k)
         build_layout(ctx);
         const size_t T = ctx->T;
         ctx->stage.ensure(sizeof(float) * 7 * T, "staging");
-        ck(cudaMemcpyAsync(ctx->stage.p, theta, sizeof(float) * 7 * T, cudaMemcpyDefault, ctx->st), "copy theta");
+        upload(ctx, ctx->stage.p, theta, sizeof(float) * 7 * T, "copy theta");
         ck(launch_set_theta(ctx->stage.as<float>(), (int)T, ctx->theta.as<float>(), ctx->errw.as<int>(), ctx->st),
            "set theta");
         reset_convergence(ctx);
-        sync_and_check_err(ctx, "set_state");
+        finish(ctx, "set_state");
         ctx->k_next = k;
         ctx->theta_set = true;
         ctx->stepped = false;
@@ -1202,11 +1335,10 @@ asicp_status asicp_run(asicp_ctx *ctx, const float *theta0)
         const int T = ctx->T;
         if (theta0) {
             ctx->stage.ensure(sizeof(float) * 7 * T, "staging");
-            ck(cudaMemcpyAsync(ctx->stage.p, theta0, sizeof(float) * 7 * (size_t)T, cudaMemcpyDefault, ctx->st),
-               "copy theta0");
+            upload(ctx, ctx->stage.p, theta0, sizeof(float) * 7 * (size_t)T, "copy theta0");
             ck(launch_set_theta(ctx->stage.as<float>(), T, ctx->theta.as<float>(), ctx->errw.as<int>(), ctx->st),
                "set theta0");
-            sync_and_check_err(ctx, "run");
+            finish(ctx, "run");
         } else {
             ck(launch_fibonacci(ctx->layout(), ctx->cfg.init_radius, ctx->cfg.init_mode, ctx->theta.as<float>(),
                                 ctx->st),
@@ -1240,11 +1372,11 @@ asicp_status asicp_best_grasps_at(asicp_ctx *ctx, int object, int topk, float *t
                                                                      ctx->out7.as<float>(), ctx->outc.as<float>(),
                                                                      ctx->outi.as<int>());
             ck(cudaGetLastError(), "gather best");
-            copy_out(theta, ctx->out7.p, sizeof(float) * 7 * n, ctx->st, "copy best theta");
-            copy_out(cost, ctx->outc.p, sizeof(float) * n, ctx->st, "copy best cost");
-            copy_out(preshape, ctx->outi.p, sizeof(int) * n, ctx->st, "copy best preshape");
+            copy_out(ctx, theta, ctx->out7.p, sizeof(float) * 7 * n);
+            copy_out(ctx, cost, ctx->outc.p, sizeof(float) * n);
+            copy_out(ctx, preshape, ctx->outi.p, sizeof(int) * n);
         }
-        sync_and_check_err(ctx, "best_grasps");
+        finish(ctx, "best_grasps");
         if (n_out) *n_out = n;
     });
 }
@@ -1262,41 +1394,35 @@ asicp_status asicp_get_state(asicp_ctx *ctx, const asicp_state_view *v)
         const bool dbg = v->nn_idx || v->nn_d2 || v->s_prime || v->col_list || v->col_nn;
         if (dbg && !ctx->cfg.debug) fail(ASICP_ERR_STATE, "get_state: debug arrays need config.debug = 1");
         const int T = ctx->T;
+        if (!(ctx->stepped || ctx->run_done) && (v->cost || v->ncol || v->h || dbg))
+            fail(ASICP_ERR_STATE, "get_state: no step has run since the poses were set");
         if (v->theta) {
             repack_kernel<<<(T + 127) / 128, 128, 0, ctx->st>>>(ctx->theta.as<float>(), T, ctx->out7.as<float>());
             ck(cudaGetLastError(), "repack theta");
-            copy_out(v->theta, ctx->out7.p, sizeof(float) * 7 * T, ctx->st, "copy theta");
-            ck(cudaStreamSynchronize(ctx->st), "get_state");
         }
         if (v->phi) {
-            repack_kernel<<<(T + 127) / 128, 128, 0, ctx->st>>>(ctx->phi.as<float>(), T, ctx->out7.as<float>());
+            ctx->outp.ensure(sizeof(float) * 7 * T, "phi");
+            repack_kernel<<<(T + 127) / 128, 128, 0, ctx->st>>>(ctx->phi.as<float>(), T, ctx->outp.as<float>());
             ck(cudaGetLastError(), "repack phi");
-            copy_out(v->phi, ctx->out7.p, sizeof(float) * 7 * T, ctx->st, "copy phi");
-            ck(cudaStreamSynchronize(ctx->st), "get_state");
         }
         if (v->grad) {
-            ctx->stage.ensure(sizeof(double) * 7 * T, "staging");
-            repack_f64_kernel<<<(T + 127) / 128, 128, 0, ctx->st>>>(ctx->grad.as<double>(), T, ctx->stage.as<double>());
+            ctx->outg.ensure(sizeof(double) * 7 * T, "gradient");
+            repack_f64_kernel<<<(T + 127) / 128, 128, 0, ctx->st>>>(ctx->grad.as<double>(), T, ctx->outg.as<double>());
             ck(cudaGetLastError(), "repack grad");
-            copy_out(v->grad, ctx->stage.p, sizeof(double) * 7 * T, ctx->st, "copy grad");
-            ck(cudaStreamSynchronize(ctx->st), "get_state");
         }
-        if (ctx->stepped || ctx->run_done) {
-            copy_out(v->cost, ctx->cost.p, sizeof(double) * T, ctx->st, "copy cost");
-            copy_out(v->ncol, ctx->ncol.p, sizeof(int) * T, ctx->st, "copy ncol");
-            copy_out(v->h, ctx->h.p, sizeof(float) * ctx->G, ctx->st, "copy h");
-            if (ctx->cfg.debug) {
-                copy_out(v->nn_idx, ctx->nnidx.p, sizeof(int) * (size_t)T * ctx->N, ctx->st, "copy nn_idx");
-                copy_out(v->nn_d2, ctx->dbg_d2.p, sizeof(float) * (size_t)T * ctx->N, ctx->st, "copy nn_d2");
-                copy_out(v->s_prime, ctx->dbg_sp.p, sizeof(float) * 3 * (size_t)T * ctx->N, ctx->st, "copy s_prime");
-                copy_out(v->col_list, ctx->colidx.p, sizeof(int) * (size_t)ctx->colidx_total, ctx->st, "copy col_list");
-                copy_out(v->col_nn, ctx->colnn.p, sizeof(int) * (size_t)ctx->colidx_total, ctx->st, "copy col_nn");
-            }
-        } else if (v->cost || v->ncol || v->h || dbg) {
-            fail(ASICP_ERR_STATE, "get_state: no step has run since the poses were set");
-        }
-        copy_out(v->frozen, ctx->frozen.p, sizeof(int) * T, ctx->st, "copy frozen");
-        sync_and_check_err(ctx, "get_state");
+        copy_out(ctx, v->theta, ctx->out7.p, sizeof(float) * 7 * T);
+        copy_out(ctx, v->phi, ctx->outp.p, sizeof(float) * 7 * T);
+        copy_out(ctx, v->grad, ctx->outg.p, sizeof(double) * 7 * T);
+        copy_out(ctx, v->cost, ctx->cost.p, sizeof(double) * T);
+        copy_out(ctx, v->ncol, ctx->ncol.p, sizeof(int) * T);
+        copy_out(ctx, v->h, ctx->h.p, sizeof(float) * ctx->G);
+        copy_out(ctx, v->frozen, ctx->frozen.p, sizeof(int) * T);
+        copy_out(ctx, v->nn_idx, ctx->nnidx.p, sizeof(int) * (size_t)T * ctx->N);
+        copy_out(ctx, v->nn_d2, ctx->dbg_d2.p, sizeof(float) * (size_t)T * ctx->N);
+        copy_out(ctx, v->s_prime, ctx->dbg_sp.p, sizeof(float) * 3 * (size_t)T * ctx->N);
+        copy_out(ctx, v->col_list, ctx->colidx.p, sizeof(int) * (size_t)ctx->colidx_total);
+        copy_out(ctx, v->col_nn, ctx->colnn.p, sizeof(int) * (size_t)ctx->colidx_total);
+        finish(ctx, "get_state");
     });
 }
 

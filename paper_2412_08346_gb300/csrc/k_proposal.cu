@@ -748,6 +748,7 @@ __global__ void sample_kernel(const float *out, const float *cen, const float *d
 // ---------------------------------------------------------------- handle
 struct Buf {
     void *p = nullptr;
+    size_t bytes = 0;
     ~Buf() { if (p) cudaFree(p); }
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
@@ -764,7 +765,20 @@ void pck(cudaError_t e)
     }
 }
 
-void alloc(Buf &b, size_t bytes) { pck(cudaMalloc(&b.p, bytes < 16 ? 16 : bytes)); }
+void alloc(Buf &b, size_t bytes)
+{
+    b.bytes = bytes < 16 ? 16 : bytes;
+    pck(cudaMalloc(&b.p, b.bytes));
+}
+
+void grow(Buf &b, size_t bytes)
+{
+    if (bytes <= b.bytes) return;
+    if (b.p) cudaFree(b.p);
+    b.p = nullptr;
+    b.bytes = 0;
+    alloc(b, bytes);
+}
 
 }  // namespace
 }  // namespace asicp
@@ -778,8 +792,10 @@ struct asicp_prop {
     cudaStream_t st = nullptr;
     long long step = 0;
     int lastB = 0;
+    unsigned char *pin = nullptr;      // page-locked memory: inputs, then results; or null
+    ~asicp_prop() { if (pin) cudaFreeHost(pin); }
     Buf w, m, v, grad, slices, wbf, wt4, wt5, wl, clouds, tg, cen, mean, h1, h2, pool, z, o, dO, lossp, dz, dg, live,
-        rows, dh2, dh1, outb, errw;
+        rows, dh2, dh1, outb, sdraws, stheta, scen, errw;
 };
 
 namespace {
@@ -797,24 +813,69 @@ asicp_status prop_guard(F &&f)
     }
 }
 
-// After a synchronisation: a bounded device wait that expired (the tensor-core
-// layers) is reported as TIMEOUT, once.
-void check_device_error(asicp_prop *pr)
+// Small inputs and results in ordinary host memory pass through the handle's page-locked memory, with one
+// wait per call.  Larger ones are copied straight: through page-locked memory a training step's 0.9 MB
+// of gradients and parameters each took 60 us longer.
+constexpr size_t kPinPiece = (size_t)64 << 10, kPinBytes = (size_t)256 << 10;
+
+bool pageable(const void *p)
 {
-    int e = 0;
-    pck(cudaMemcpy(&e, pr->errw.p, sizeof(int), cudaMemcpyDeviceToHost));
-    if (e != kDevOk) {
-        pck(cudaMemset(pr->errw.p, 0, sizeof(int)));
-        throw PropErr{ASICP_ERR_TIMEOUT};
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
     }
+    return at.type == cudaMemoryTypeUnregistered;
 }
 
-// device copy of an input that may be host memory
-const float *staged(asicp_prop *pr, const float *src, size_t n, Buf &buf)
-{
-    pck(cudaMemcpyAsync(buf.p, src, n * sizeof(float), cudaMemcpyDefault, pr->st));
-    return buf.as<float>();
-}
+// One call's copies.  Inputs may be reused when the call returns, results are there.
+struct Transfer {
+    asicp_prop *pr;
+    size_t in = 0, out = 0;
+    struct Out { void *dst; size_t at, bytes; };
+    std::vector<Out> outs;
+
+    explicit Transfer(asicp_prop *p) : pr(p) {}
+    ~Transfer() { if (in || out) cudaStreamSynchronize(pr->st); }      // (left by an error: nothing stays in flight)
+    // device copy of an input that may be host memory
+    const float *load(const float *src, size_t n, Buf &buf)
+    {
+        const size_t bytes = n * sizeof(float);
+        if (pr->pin && bytes <= kPinPiece && in + bytes <= kPinBytes && pageable(src)) {
+            unsigned char *at = pr->pin + in;
+            std::memcpy(at, src, bytes);
+            in += (bytes + 255) / 256 * 256;
+            pck(cudaMemcpyAsync(buf.p, at, bytes, cudaMemcpyHostToDevice, pr->st));
+        } else {
+            pck(cudaMemcpyAsync(buf.p, src, bytes, cudaMemcpyDefault, pr->st));
+        }
+        return buf.as<float>();
+    }
+    void store(void *dst, const void *src, size_t bytes)
+    {
+        if (!dst || !bytes) return;
+        if (pr->pin && bytes <= kPinPiece && out + bytes <= kPinBytes && pageable(dst)) {
+            outs.push_back({dst, out, bytes});
+            pck(cudaMemcpyAsync(pr->pin + kPinBytes + out, src, bytes, cudaMemcpyDeviceToHost, pr->st));
+            out += (bytes + 255) / 256 * 256;
+        } else {
+            pck(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, pr->st));
+        }
+    }
+    // A bounded device wait that expired (the tensor-core layers) is reported as TIMEOUT, once.
+    void finish()
+    {
+        int e = 0;
+        store(&e, pr->errw.p, sizeof(int));
+        pck(cudaStreamSynchronize(pr->st));
+        for (const Out &x : outs) std::memcpy(x.dst, pr->pin + kPinBytes + x.at, x.bytes);
+        in = out = 0;
+        if (e != kDevOk) {
+            pck(cudaMemset(pr->errw.p, 0, sizeof(int)));
+            throw PropErr{ASICP_ERR_TIMEOUT};
+        }
+    }
+};
 
 // The clouds' mixture outputs in pr->o, centroids in pr->cen; store: keep h1 and h2 for a backward pass.
 void forward_impl(asicp_prop *pr, const float *clouds_dev, int B, bool store)
@@ -904,6 +965,9 @@ asicp_status asicp_prop_create(int P, int n_points, int max_batch, void *cuda_st
         alloc(pr->dh2, B * kH3 * kH2 * 4); alloc(pr->dh1, B * kH3 * kH1 * 4);
         alloc(pr->outb, B * pr->nout * 4);
         alloc(pr->errw, sizeof(int));
+        void *pin = nullptr;
+        if (cudaHostAlloc(&pin, 2 * kPinBytes, cudaHostAllocDefault) == cudaSuccess) pr->pin = static_cast<unsigned char *>(pin);
+        else cudaGetLastError();
         pck(cudaMemsetAsync(pr->errw.p, 0, sizeof(int), pr->st));
         pck(cudaMemsetAsync(pr->w.p, 0, np * 4, pr->st));
         pck(cudaMemsetAsync(pr->m.p, 0, np * 4, pr->st));
@@ -945,8 +1009,9 @@ asicp_status asicp_prop_get_params(asicp_prop *pr, float *params)
 {
     if (!pr || !params) return ASICP_ERR_INVALID_ARG;
     return prop_guard([&] {
-        pck(cudaMemcpyAsync(params, pr->w.p, pr->np * 4, cudaMemcpyDefault, pr->st));
-        pck(cudaStreamSynchronize(pr->st));
+        Transfer t(pr);
+        t.store(params, pr->w.p, pr->np * 4);
+        t.finish();
     });
 }
 
@@ -954,12 +1019,12 @@ asicp_status asicp_prop_forward(asicp_prop *pr, const float *clouds, int B, floa
 {
     if (!pr || !clouds || !out || B < 1 || B > pr->maxB) return ASICP_ERR_INVALID_ARG;
     return prop_guard([&] {
-        const float *c = staged(pr, clouds, (size_t)B * pr->npts * 3, pr->clouds);
+        Transfer t(pr);
+        const float *c = t.load(clouds, (size_t)B * pr->npts * 3, pr->clouds);
         forward_impl(pr, c, B, false);
-        pck(cudaMemcpyAsync(out, pr->o.p, (size_t)B * pr->nout * 4, cudaMemcpyDefault, pr->st));
-        if (centroids) pck(cudaMemcpyAsync(centroids, pr->cen.p, (size_t)B * 3 * 4, cudaMemcpyDefault, pr->st));
-        pck(cudaStreamSynchronize(pr->st));
-        check_device_error(pr);
+        t.store(out, pr->o.p, (size_t)B * pr->nout * 4);
+        t.store(centroids, pr->cen.p, (size_t)B * 3 * 4);
+        t.finish();
     });
 }
 
@@ -969,18 +1034,18 @@ asicp_status asicp_prop_loss_grad(asicp_prop *pr, const float *clouds, const flo
     if (!pr || !clouds || !targets || !loss || B < 1 || B > pr->maxB || T < 1 || T > ASICP_PROP_MAX_TARGETS)
         return ASICP_ERR_INVALID_ARG;
     return prop_guard([&] {
-        const float *c = staged(pr, clouds, (size_t)B * pr->npts * 3, pr->clouds);
-        const float *t = staged(pr, targets, (size_t)B * pr->P * T * 7, pr->tg);
+        Transfer io(pr);
+        const float *c = io.load(clouds, (size_t)B * pr->npts * 3, pr->clouds);
+        const float *t = io.load(targets, (size_t)B * pr->P * T * 7, pr->tg);
         forward_impl(pr, c, B, true);
         loss_kernel<<<dim3(pr->P, B), kLossThreads, 0, pr->st>>>(pr->o.as<float>(), pr->cen.as<float>(), t, pr->P, T,
                                                                  pr->dO.as<float>(), pr->lossp.as<float>());
         pck(cudaGetLastError());
         backward_impl(pr, c, B);
         std::vector<float> lp((size_t)B * pr->P);
-        pck(cudaMemcpyAsync(lp.data(), pr->lossp.p, lp.size() * 4, cudaMemcpyDeviceToHost, pr->st));
-        if (grad) pck(cudaMemcpyAsync(grad, pr->grad.p, pr->np * 4, cudaMemcpyDefault, pr->st));
-        pck(cudaStreamSynchronize(pr->st));
-        check_device_error(pr);
+        io.store(lp.data(), pr->lossp.p, lp.size() * 4);
+        io.store(grad, pr->grad.p, pr->np * 4);
+        io.finish();
         double s = 0.0;     // mean over objects of (1 / (P T)) sum over preshapes and targets
         for (float x : lp) s += x;
         *loss = (float)(s / ((double)pr->P * T * B));
@@ -1010,18 +1075,20 @@ asicp_status asicp_prop_sample(asicp_prop *pr, const float *out, const float *ce
         return ASICP_ERR_INVALID_ARG;
     return prop_guard([&] {
         const size_t n = (size_t)B * pr->P * K;
-        Buf dr, th, cn;
-        alloc(dr, n * 8 * 4);
-        alloc(th, n * 7 * 4);
-        alloc(cn, (size_t)B * 3 * 4);
-        pck(cudaMemcpyAsync(pr->outb.p, out, (size_t)B * pr->nout * 4, cudaMemcpyDefault, pr->st));
-        pck(cudaMemcpyAsync(dr.p, draws, n * 8 * 4, cudaMemcpyDefault, pr->st));
-        pck(cudaMemcpyAsync(cn.p, centroids, (size_t)B * 3 * 4, cudaMemcpyDefault, pr->st));
-        sample_kernel<<<(unsigned)((n + 255) / 256), 256, 0, pr->st>>>(pr->outb.as<float>(), cn.as<float>(),
-                                                                      dr.as<float>(), B, pr->P, K, th.as<float>());
+        // room for the draws and the poses, kept (K is at most 4096)
+        grow(pr->sdraws, n * 8 * 4);
+        grow(pr->stheta, n * 7 * 4);
+        grow(pr->scen, (size_t)B * 3 * 4);
+        Transfer t(pr);
+        t.load(out, (size_t)B * pr->nout, pr->outb);
+        t.load(draws, n * 8, pr->sdraws);
+        t.load(centroids, (size_t)B * 3, pr->scen);
+        sample_kernel<<<(unsigned)((n + 255) / 256), 256, 0, pr->st>>>(pr->outb.as<float>(), pr->scen.as<float>(),
+                                                                      pr->sdraws.as<float>(), B, pr->P, K,
+                                                                      pr->stheta.as<float>());
         pck(cudaGetLastError());
-        pck(cudaMemcpyAsync(theta, th.p, n * 7 * 4, cudaMemcpyDefault, pr->st));
-        pck(cudaStreamSynchronize(pr->st));
+        t.store(theta, pr->stheta.p, n * 7 * 4);
+        t.finish();
     });
 }
 
