@@ -103,17 +103,6 @@ __device__ __forceinline__ float dist2_f32(float ax, float ay, float az, float b
     return __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
 }
 
-// Exact-form nearest point among object points [lo, hi) (index order, strict <).
-__device__ __forceinline__ void exact_scan(const float4 *__restrict__ R, int lo, int hi, float sx, float sy, float sz,
-                                           float &best, int &bi)
-{
-    for (int r = lo; r < hi; ++r) {
-        const float4 v = __ldg(R + r);
-        const float d = dist2_f32(sx, sy, sz, v.x, v.y, v.z);
-        if (d < best) { best = d; bi = r; }
-    }
-}
-
 // Exact-form nearest point of query (qx, qy, qz) among all M object points, found by
 // the whole warp together (lane l takes points l, l + 32, ...; ties to the lower
 // index); every lane receives the result.  Call with all 32 lanes.
