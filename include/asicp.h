@@ -74,7 +74,10 @@ typedef enum {
  *                  workload and keeps the fastest (see asicp_autotune); 0: use fwd_shape
  *   fwd_shape     forward-matching kernel shape, 0 .. ASICP_FWD_SHAPES-1 (0 = default):
  *                  0 .. ASICP_FWD_SHAPES-2 are float32 kernels, ASICP_FWD_SHAPES-1 the
- *                  tensor-core screening with its exact-choice kernel (not with mini-batches).
+ *                  tensor-core screening with its exact-choice kernel (not with mini-batches),
+ *                  which clouds of 1024 to 2^18 points replace, once the passes so far would
+ *                  have paid for the build, by cells around the object that keep the points
+ *                  which can be nearest in them (same results).
  *                  Every shape returns the lowest-index minimum of the exact-form float32
  *                  distance over the points that can be nearest; they can differ only where
  *                  several points' float32 distances tie within rounding (near-ties)
@@ -187,8 +190,10 @@ asicp_status asicp_set_particle_counts(asicp_ctx *ctx, const int *K, int n);
  * sampled on a node-centred grid of nx*ny*nz float32 values, x fastest, positive
  * inside the gripper (Eq. 12), node (0,0,0) at origin, spacing voxel.  Computes
  * TCP = centroid of S (Section IV-B).  Every preshape must have the same N
- * (1 <= N <= 6144).  The context keeps a copy of the grid and a corner-packed
- * copy for the lookups (32 bytes per cell: 8 (nx-1)(ny-1)(nz-1) floats).
+ * (1 <= N <= 6144).  The context keeps a copy of the grid, a corner-packed
+ * copy for the lookups (32 bytes per cell: 8 (nx-1)(ny-1)(nz-1) floats) and a byte
+ * per cell for its distance to the gripper; for N >= 512 also cells around S for
+ * the reverse matching.
  * Errors: INVALID_ARG (index, N out of range, a grid dimension < 2, voxel <= 0, N differing
  * from an earlier preshape, non-finite value). */
 asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_xyz, int N,
@@ -245,12 +250,13 @@ asicp_status asicp_get_state(asicp_ctx *ctx, const asicp_state_view *view);
 /* With config.profile = 1: accumulated device time (ms) and launch count of the
  * path's kernels since the last reset (profile = 2: the forward-matching entry
  * only, the others stay 0).  ms[ASICP_KERNEL_KINDS] / launches[...]
- * order: forward matching (screening; with the float32 shapes also the exact
- * choice), collision test (with the matching sums), reverse matching, finalize
- * (cost, gradient, convergence, SGD step), Stein (SVGD step: the Stein direction
- * and the update kernel, timed and counted together as one launch per pass), and
- * the exact choice of the tensor-core shape (no launches with the float32
- * shapes).  reset = 1 clears the counters after reading.  Errors: STATE (profile
+ * order: forward matching (screening; with the float32 shapes and through the
+ * cells also the exact choice), collision test, reverse matching, finalize
+ * (the sums over the pairs, cost, gradient, convergence, SGD step), Stein (SVGD
+ * step: the Stein direction and the update kernel, timed and counted together as
+ * one launch per pass), and the exact choice of the tensor-core shape (no launches
+ * with the float32 shapes and through the cells).  With profile = 0 the collision
+ * test and the reverse matching may run beside the forward matching.  reset = 1 clears the counters after reading.  Errors: STATE (profile
  * off). */
 #define ASICP_KERNEL_KINDS 6
 asicp_status asicp_kernel_times(asicp_ctx *ctx, double ms[ASICP_KERNEL_KINDS], long long launches[ASICP_KERNEL_KINDS],
@@ -313,7 +319,7 @@ asicp_status asicp_autotune(asicp_ctx *ctx, int *chosen, float *ms);
 /* Testing aid for the bounded-wait path.  Every device-side wait of the library
  * is bounded (2^32 SM clock cycles, about 2 s); when one expires, the kernel sets
  * the context's error word, drains its copies in flight with the full budget and
- * returns, the later kernels of the pass see the error word and skip their work,
+ * returns, the finalize and Stein kernels see the error word and skip their work,
  * and the next call that reads results (asicp_get_state, asicp_best_grasps)
  * returns TIMEOUT and clears the word; the context stays usable.  With on != 0 the
  * float32 matching shapes' kernels of later asicp_step / asicp_run calls make each

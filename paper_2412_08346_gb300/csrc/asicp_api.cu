@@ -195,6 +195,9 @@ struct asicp_ctx {
     std::vector<int> loop_mb;         // mini-batch offsets it was captured with, and the object's entry
     ObjMeta loop_meta{};
     cudaStream_t cap_st = nullptr;
+    // the collision test's branch of a pass and the events that part and join the two
+    cudaStream_t side_st = nullptr;
+    cudaEvent_t parted = nullptr, joined = nullptr;
     cudaGraphExec_t loop_exec = nullptr;
     std::vector<const void *> loop_key;
     std::vector<Ev> graph_events;     // event pairs inside the graph (profile = 1)
@@ -237,6 +240,9 @@ struct asicp_ctx {
         for (auto e : pool) cudaEventDestroy(e);
         if (loop_exec) cudaGraphExecDestroy(loop_exec);
         if (cap_st) cudaStreamDestroy(cap_st);
+        if (parted) cudaEventDestroy(parted);
+        if (joined) cudaEventDestroy(joined);
+        if (side_st) cudaStreamDestroy(side_st);
     }
 };
 
@@ -538,10 +544,10 @@ void reset_convergence(asicp_ctx *c)
 }
 
 template <class L>
-void timed(asicp_ctx *c, int kind, L &&launch, const char *what)
+void timed(asicp_ctx *c, int kind, L &&launch, const char *what, cudaStream_t side = nullptr)
 {
     cudaEvent_t a = nullptr, b = nullptr;
-    cudaStream_t st = work_stream(c);
+    cudaStream_t st = side ? side : work_stream(c);
     // inside a capture, an external record makes the event a graph node that every
     // replay records (a plain record would only express a capture dependency)
     const unsigned flags = c->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
@@ -575,7 +581,6 @@ void accumulate_graph_events(asicp_ctx *c)
     c->graph_pending = false;
 }
 
-// One pass of cost/gradient evaluation (+ update for mode 1/2).
 // Object 0's table points at the mini-batch of iteration k (k < the number of
 // mini-batches) or back at the whole cloud (otherwise), on the work stream.
 void select_minibatch(asicp_ctx *c, int k)
@@ -768,6 +773,54 @@ void ensure_pre_cells(asicp_ctx *c, int passes)
     c->pre_built = true;
 }
 
+// The collision test and the reverse matching of a pass read the poses only, as the forward matching
+// does, and write buffers of their own: they run on a second stream beside it, and both are joined
+// before the finalize kernel.  With kernel timers the pass is one stream, so that each time is the
+// kernel's own.  What is on the second stream is joined also when a launch of the first one fails.
+//
+// Parting and joining cost about 3 us of a captured pass and 5 us of a direct one.  A captured loop gains
+// more where the matching leaves room beside it: the float32 kernels with few queries (32 particles of 256
+// points on 512 points, whole search: 2033 -> 1788 us; mini-batch ramp of 32 particles 2594 -> 2150 us) and
+// the cells with many (6.3 M queries 4845 -> 4613 us; 1.6 M: 9637 -> 9590 us; but 0.13 M: 1857 -> 1900 us).
+// A direct pass gains with many queries only (12.6 M: 1328 -> 1277 us; 0.16 M: 106 -> 111 us).
+constexpr long long kPartQueries = 1 << 20;
+
+bool parts(const asicp_ctx *c)
+{
+    return c->cfg.profile == 0 && ((c->capturing && !c->cells_on) || (long long)c->T * c->N >= kPartQueries);
+}
+
+class Branch {
+public:
+    Branch(asicp_ctx *c, bool on) : c_(c), on_(on)
+    {
+        if (!on_) return;
+        ck(cudaEventRecord(c->parted, work_stream(c)), "part the pass");
+        ck(cudaStreamWaitEvent(c->side_st, c->parted, 0), "part the pass");
+        open_ = true;
+    }
+    ~Branch()
+    {
+        if (open_) (void)close();
+    }
+    cudaStream_t stream() const { return on_ ? c_->side_st : nullptr; }
+    void join()
+    {
+        if (on_) ck(close(), "join the pass");
+    }
+
+private:
+    cudaError_t close()
+    {
+        open_ = false;
+        const cudaError_t e = cudaEventRecord(c_->joined, c_->side_st);
+        return e == cudaSuccess ? cudaStreamWaitEvent(work_stream(c_), c_->joined, 0) : e;
+    }
+    asicp_ctx *c_;
+    bool on_, open_ = false;
+};
+
+// One pass of cost/gradient evaluation (+ update for mode 1/2).
 void iterate(asicp_ctx *c, int mode, float gamma, int k)
 {
     select_minibatch(c, k);
@@ -790,6 +843,7 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
         fa.dbg_d2 = c->dbg_d2.as<float>();
         fa.dbg_sp = c->dbg_sp.as<float>();
     }
+    Branch side(c, parts(c));
     timed(c, kTimeMatch, [&](cudaStream_t st) { return launch_fwd_match(fa, st); }, "forward matching kernel");
     if (fwd_has_exact_kernel(fa))
         timed(c, kTimeExact, [&](cudaStream_t st) { return launch_fwd_exact(fa, st); }, "exact choice kernel");
@@ -806,7 +860,6 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
     ca.colmap = c->colmap.as<int2>();
     ca.col_items = c->colitems.as<int>();
     ca.col_list = c->collist.as<int>();
-    ca.err = c->errw.as<int>();
     for (const ObjMeta &m : c->objmeta_h) ca.most_points = std::max(ca.most_points, m.Mc);
     ca.cells = c->pre_built;
     if (ca.cells) {
@@ -818,8 +871,10 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
         ca.pre_leaf_cap = s.leaf_cap;
         ca.most_items = (int)std::min<long long>(std::max<long long>(1, c->colmap_total), INT_MAX);
     }
-    timed(c, kTimeCollide, [&](cudaStream_t st) { return launch_collide(ca, st); }, "collision kernel");
-    timed(c, kTimeCollideNN, [&](cudaStream_t st) { return launch_collide_nn(ca, st); }, "collision matching kernel");
+    timed(c, kTimeCollide, [&](cudaStream_t st) { return launch_collide(ca, st); }, "collision kernel", side.stream());
+    timed(c, kTimeCollideNN, [&](cudaStream_t st) { return launch_collide_nn(ca, st); }, "collision matching kernel",
+          side.stream());
+    side.join();
 
     UpdateArgs ua{};
     ua.L = L;
@@ -1126,6 +1181,9 @@ asicp_status asicp_create(const asicp_config *cfg, asicp_ctx **out)
     asicp_status s = guarded(c, [&] {
         // one-time kernel attributes, set outside any graph capture
         fwd_grid_size();
+        ck(cudaStreamCreateWithFlags(&c->side_st, cudaStreamNonBlocking), "side stream");
+        ck(cudaEventCreateWithFlags(&c->parted, cudaEventDisableTiming), "side stream event");
+        ck(cudaEventCreateWithFlags(&c->joined, cudaEventDisableTiming), "side stream event");
         ck(init_collision_attributes(), "collision kernel attributes");
         ck(init_update_attributes(), "update kernel attributes");
         ck(init_cells_attributes(), "cell kernel attributes");

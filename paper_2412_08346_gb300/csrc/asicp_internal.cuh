@@ -345,7 +345,6 @@ struct CollideArgs {
                               // only those with bits written (see ObjMeta::colmap_base)
     int *col_items;           // (count, next) of the reverse-matching work list
     int *col_list;            // [2 * items] (particle, item) pairs
-    const int *err;           // error word: a kernel of the pass found an error, skip the work
     int cells;                // reverse matching through the gripper clouds' cells
     const int2 *pre_nodes;    // [P][pre_node_cap]
     const int *pre_leaves;    // [P][pre_leaf_cap]

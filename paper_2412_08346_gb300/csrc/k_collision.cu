@@ -80,7 +80,6 @@ __host__ __device__ constexpr int col_item_points(bool cells) { return cells ? 3
 template <int kTestThreads>
 __global__ void __launch_bounds__(kTestThreads, 1280 / kTestThreads) collide_kernel(const CollideArgs a)
 {
-    if (a.err && *a.err != kDevOk) return;    // the matching gave up: its correspondences are not valid
     const int pk = blockIdx.x;
     const int grp = a.L.part_grp[pk], p = grp % a.L.P;
     const ObjMeta &om = a.L.obj[grp / a.L.P];
@@ -363,7 +362,6 @@ __device__ __forceinline__ void argmin_xor(float &best, int &bi, int o)
 // For gripper clouds without cells (few points, or cells not built yet).
 __global__ void __launch_bounds__(kColThreads) collide_nn_kernel(const CollideArgs a)
 {
-    if (a.err && *a.err != kDevOk) return;
     constexpr int kWarps = kColThreads / 32;
     constexpr int kQW = kColChunk / kWarps;                  // colliding points per warp
     static_assert(kQW == 8 && kColChunk == 64, "lane groups of four per colliding point");
@@ -542,7 +540,6 @@ __global__ void __launch_bounds__(kColThreads) collide_nn_kernel(const CollideAr
 // 57 % of the issue slots, the rest waits for the scattered loads.
 __global__ void __launch_bounds__(128, 10) collide_cells_kernel(const CollideArgs a)
 {
-    if (a.err && *a.err != kDevOk) return;
     const int lane = threadIdx.x & 31, N = a.L.N;
     const int count = a.col_items[0];
     for (int item = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; item < count; item += (gridDim.x * blockDim.x) >> 5) {

@@ -162,6 +162,8 @@ __device__ __forceinline__ void half_sync(int half)
 
 __global__ void __launch_bounds__(2 * kFinalizeThreads, 4) finalize_kernel(const UpdateArgs a)
 {
+    // (cleared also when the matching gave up: the collision test beside it may have run)
+    if (blockIdx.x == 0 && threadIdx.x == 0 && a.col_items) { a.col_items[0] = 0; a.col_items[1] = 0; }
     if (a.err && *a.err != kDevOk) return;    // an earlier kernel of the pass gave up: its results are not valid
     constexpr int kChunks = 2 * kFinalizeThreads / 32;     // chunks a round
     __shared__ dfloat sPart_[2][2][kChunks][kColSums];
@@ -169,7 +171,6 @@ __global__ void __launch_bounds__(2 * kFinalizeThreads, 4) finalize_kernel(const
     // the sums {s (3), s s^T (6), x (3), x s^T (9), |x|^2} and the half warp's vectors and matrices
     __shared__ double sm_[2][kColSums], sR_[2][9], sE_[2][9], sRs_[2][3], sTcp_[2][3], sEc_[2][3], sG_[2][4];
     const int N = a.L.N;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && a.col_items) { a.col_items[0] = 0; a.col_items[1] = 0; }
     {
         const int half = threadIdx.x / kFinalizeThreads, tid = threadIdx.x % kFinalizeThreads;
         const int pk = 2 * blockIdx.x + half;

@@ -186,3 +186,37 @@ def test_every_shape_at_the_edges_of_chunks_and_tiles(M):
             tl.check_nn(st["s_prime"].reshape(-1, 3), R, st["nn_idx"].reshape(-1), {})
     for idx in got:
         assert np.array_equal(idx, got[1])
+
+
+@pytest.mark.parametrize("K,N,shape", [(7, 33, 0), (256, 4095, 7), (256, 4096, 7), (257, 4096, 0)])
+def test_collision_test_beside_the_matching_gives_the_same_pass(K, N, shape):
+    """A pass with kernel timers runs its kernels one after the other, one without runs the collision test beside
+    the matching (in a captured loop, and directly from 2^20 gripper points on): the same poses and costs, also
+    after a matching whose waits expired while the collision test beside it ran."""
+    w = synth.custom_case(P=1, K=K, N=N, M=1500, grid=24, k_max=3, seed=5, k_stein=1)
+    out = []
+    for profile in (1, 0):
+        cfg = asicp.asicp_config_default(P=1, K=K, k_max=3, k_stein=1, conv_tol=-1.0, init_radius=0.05, profile=profile,
+                                         fwd_shape=shape, cuda_stream=torch.cuda.current_stream().cuda_stream)
+        ctx = asicp.asicp_create(cfg)
+        try:
+            keep = tl.upload(ctx, w)
+            if shape == 0 and profile == 0:
+                asicp.asicp_test_expire_waits(ctx, True)
+                asicp.asicp_run(ctx)
+                with pytest.raises(asicp.AsicpError):
+                    asicp.asicp_get_state(ctx, theta=np.zeros((K, 7), np.float32))
+                asicp.asicp_test_expire_waits(ctx, False)
+            asicp.asicp_run(ctx)
+            state = [np.zeros((K, 7), np.float32), np.zeros(K), np.zeros(K, np.int32)]
+            asicp.asicp_get_state(ctx, theta=state[0], cost=state[1], ncol=state[2])
+            asicp.asicp_step(ctx, 2)
+            more = [np.zeros((K, 7), np.float32), np.zeros(K), np.zeros(K, np.int32)]
+            asicp.asicp_get_state(ctx, theta=more[0], cost=more[1], ncol=more[2])
+            out.append(state + more)
+            del keep
+        finally:
+            asicp.asicp_destroy(ctx)
+    assert out[0][2].any()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
