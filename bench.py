@@ -10,7 +10,9 @@ points, 8192-point single-view partial object clouds of seeded procedural
 shapes, 64^3 SDF grids, 100 iterations (38 SVGD + 62 SGD).  The metric is
 forward matching throughput in particle*point pairs per second
 (P * K * N * M pairs per iteration, k_max + 1 evaluations per step) plus the
-milliseconds per grasp set.
+milliseconds per grasp set.  The pairs are those the nearest-neighbour search
+decides: the library's cells evaluate only the points that can be nearest and
+return the brute-force result, so the rate counts the brute-force pairs.
 
 N > 1 GPUs (torchrun): every rank optimises its own object (weak scaling, no
 data-path collective); the step time is the maximum over ranks.
@@ -49,6 +51,11 @@ FMA_PER_PAIR = 3          # of which FMA-pipe work (the compare runs as half a 3
 TC_ALG_FLOP_PER_PAIR = 8  # tensor-core shape, algorithmic: |r|^2 - 2 s'.r as an augmented K = 4 contraction
 TC_EXEC_FLOP_PER_PAIR = 32  # executed: one M=128 x N=256 x K=16 f16 MMA per 128 x 256 pairs (split operands)
 EPILOGUE_OPS_PER_PAIR = 1   # the tensor-core shape's epilogue: one compare per pair
+# cells_match_kernel, of the committed ncu capture of a paper-scale launch
+# (profiles/pass_kernels_paper-scale-P3-K256-N2048-M8192.md): executed lane instructions per gripper point
+# (transform, cell look-up, about 12 exact distances; 19.97 M warp instructions for 1.573 M points) and DRAM bytes
+CELLS_LANE_INST_PER_QUERY = 406
+CELLS_DRAM_BYTES_PER_LAUNCH = 3054848
 TC_SHAPE = "tc-f16x3-m128-n256"
 TOPK = 16
 METRIC = "AS-ICP particle*point pairs/s (forward matching) and ms per grasp set"
@@ -313,10 +320,10 @@ def run_gpu(args, rank, world, local_rank):
     stream = torch.cuda.current_stream()
     w = workload(rank, args.small)
     P, K, N, M = len(w.preshapes), w.K, w.preshapes[0].S.shape[0], len(w.objects[0].points)
-    # profile 2: CUDA events around the forward-matching kernel only (the roofline's kernel); every
-    # event is a node of the captured loop, and timing all kernels (profile 1) costs ~5 % of a grasp set
+    # no kernel timers in the timed region: every event is a node of the captured loop (the matching's
+    # alone, 202 of them, cost 1.2 of 9.6 ms); the kernels are timed in a second pass
     cfg = asicp.asicp_config_default(P=P, K=K, k_max=w.k_max, k_stein=w.k_stein, schedule=w.schedule,
-                                     profile=2, cuda_stream=stream.cuda_stream, fwd_shape=max(0, args.fwd_shape))
+                                     cuda_stream=stream.cuda_stream, fwd_shape=max(0, args.fwd_shape))
     ctx = asicp.asicp_create(cfg)
     obj = w.objects[0].points
     R_dev = torch.from_numpy(obj).to(dev)
@@ -351,7 +358,6 @@ def run_gpu(args, rank, world, local_rank):
         one_step()
         one_step(ctx_all)
     torch.cuda.synchronize()
-    asicp.asicp_kernel_times(ctx, reset=True)
 
     clocks = ClockSampler(local_rank)
     if world > 1:
@@ -371,7 +377,6 @@ def run_gpu(args, rank, world, local_rank):
     if world > 1:
         dist.barrier()
     clk = clocks.stop()
-    ms_t, launches_t = asicp.asicp_kernel_times(ctx, reset=True)
     # per-kernel breakdown (every kernel timed), the same number of steps after the timed region
     asicp.asicp_kernel_times(ctx_all, reset=True)
     all_ms = []
@@ -395,14 +400,18 @@ def run_gpu(args, rank, world, local_rank):
 
     # dominant kernel: forward matching; algorithmic work per launch = P*K*N*M pairs
     tc = asicp.FWD_VARIANTS[shape] == TC_SHAPE
-    match_avg_s = ms_t[0] / max(1, launches_t[0]) / 1e3          # timed region
+    match_avg_s = ms[0] / max(1, launches[0]) / 1e3              # breakdown pass
     exact_avg_s = ms[5] / max(1, launches[5]) / 1e3 if tc else 0.0   # breakdown pass
     pairs_per_launch = P * K * N * M
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    roofline = roofline_entry(tc, pairs_per_launch, match_avg_s, exact_avg_s, ms, sms, clk)
-    # match, collide, collide_nn, finalize per pass (+ the exact choice with the tensor-core shape),
+    cells = tc and launches[5] == 0       # no exact choice after the matching: it went through the cells
+    if cells:
+        roofline = cells_roofline_entry(P * K * N, M, match_avg_s, ms, sms, clk)
+    else:
+        roofline = roofline_entry(tc, pairs_per_launch, match_avg_s, exact_avg_s, ms, sms, clk)
+    # match, collide, collide_nn, finalize per pass (+ the exact choice after the tensor-core screening),
     # Stein direction and Stein update per SVGD pass, + init, reset, select, gather
-    launches_per_step = (5 if tc else 4) * (w.k_max + 1) + 2 * w.k_stein + 4
+    launches_per_step = (5 if tc and not cells else 4) * (w.k_max + 1) + 2 * w.k_stein + 4
 
     e2e = None
     if not args.no_e2e:
@@ -437,10 +446,10 @@ def run_gpu(args, rank, world, local_rank):
             "ms_per_grasp_set": max_ms / args.steps,
             "roofline": roofline,
             "kernel_ms_per_step": {k: v / args.steps for k, v in zip(asicp.KERNEL_KINDS, ms)},
-            "kernel_breakdown": ("kernel_ms_per_step, exact_kernel_ms and the shares come from a second pass of "
+            "kernel_breakdown": ("kernel_ms_per_step and the roofline's kernel times come from a second pass of "
                                  f"{args.steps} steps after the timed region with every kernel timed (CUDA events "
                                  f"in the captured loop: {statistics.median(all_ms):.1f} ms per grasp set there); "
-                                 "the timed region times the forward-matching kernel only"),
+                                 "the timed region has no kernel timers"),
             "gpu_launches": launches_per_step * args.steps,
             "clocks": clk,
         }
@@ -505,6 +514,25 @@ def roofline_entry(tc, pairs_per_launch, match_avg_s, exact_avg_s, ms, sms, clk)
                 f"{OPS_PER_PAIR} lane operations per pair (3 FMA + 1 compare)",
             "frac_fma_pipe": achieved / (lane_ops / FMA_PER_PAIR), "peak_fma_pipe": lane_ops / FMA_PER_PAIR / 1e9,
             "launch_ms": match_avg_s * 1e3, "pairs_per_launch": pairs_per_launch, "kernel_share": share,
+            "sms": sms, "sm_mhz": mhz}
+
+
+def cells_roofline_entry(queries, M, match_avg_s, ms, sms, clk):
+    """Roofline of cells_match_kernel in gripper points (queries) per second: the issue rate, SMs x 128
+    lane instructions per clock over the instructions a query executes (counted once by ncu).  The
+    rate of brute-force pairs that the search stands for is reported beside it."""
+    mhz = clk.get("sm_mhz") or SM_MAX_MHZ_NOMINAL
+    peak = sms * FP32_LANES_PER_SM * mhz * 1e6 / CELLS_LANE_INST_PER_QUERY
+    achieved = queries / match_avg_s
+    return {"bound": "alu", "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Gqueries/s",
+            "frac": achieved / peak, "kernel": "cells_match_kernel",
+            "peak_basis": f"{sms} SMs x {FP32_LANES_PER_SM} lane instructions per clock x {mhz:.0f} MHz / "
+                          f"{CELLS_LANE_INST_PER_QUERY} executed lane instructions per query (ncu)",
+            "traffic": CELLS_DRAM_BYTES_PER_LAUNCH,
+            "traffic_basis": "dram__bytes_read+write of one paper-scale launch from cold caches (ncu); cells, points "
+                             "and poses are L2-resident between the passes",
+            "launch_ms": match_avg_s * 1e3, "queries_per_launch": queries, "pairs_per_launch": queries * M,
+            "matching_pairs_per_s": queries * M / match_avg_s, "kernel_share": ms[0] / max(1e-9, sum(ms)),
             "sms": sms, "sm_mhz": mhz}
 
 
@@ -819,9 +847,9 @@ def run_k_sweep(args):
 def run_large(args):
     """The mixed-precision configuration (3 preshapes x 1024 particles, N=4096, M=65536 superquadric
     partial view, SDF 128^3): the float32 matching kernel (the autotuner's best float32 shape) and the
-    tensor-core screening + exact choice, each timed over a 4-iteration run (per-launch device time
-    from the library's event timers), and the fraction of correspondences on which the two agree in
-    one step from the same poses."""
+    tensor-core shape (which matches through the cells once they have paid for their build, as they have
+    by the timed run), each timed over a 4-iteration run (per-launch device time from the library's event
+    timers), and the fraction of correspondences on which the two agree in one step from the same poses."""
     import torch
     from paper_2412_08346_gb300 import asicp, synth
     import oracle

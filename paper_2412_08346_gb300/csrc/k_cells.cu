@@ -37,8 +37,9 @@
 // Measured on GB300 (per pass, against screening and exact choice on the tensor cores): 3 x 256
 // particles, N 2048, M 8192 34 us against 783; 3 x 1024, N 4096, M 65536 0.28 ms against 41.4;
 // lists of at most 12 points (with one flat grid of queries, which divided each by N: 12 38 us,
-// 16 44, 24 46, 32 52, 48 60; at 8 they stop shrinking and the budgets run out).  What bounds the matching is the latency of its dependent loads
-// (table, two or three nodes, list, points), all from L2 and L1; queries in the gripper
+// 16 44, 24 46, 32 52, 48 60; at 8 they stop shrinking and the budgets run out).  What bounds the
+// matching is the latency of its dependent loads (table, two or three nodes, list, points), all from
+// L2 and L1, at half of the issue slots; queries in the gripper
 // cloud's own order take 68 us.  The build (ten rounds of few and uneven cells, latency again)
 // takes 0.10 ms at 1024 points, 0.27 at 8192, 1.4 at 65536.
 #include "cells.cuh"

@@ -24,8 +24,8 @@
 //     therefore has d~(r*) <= b1 + 2 delta, so every chunk whose minimum exceeds
 //     that bound is excluded.  If only chunk c1 (and c2 when b2 <= b1 + 2 delta)
 //     can hold r*, their points are re-evaluated with the exact-form distance
-//     (dx^2 + dy^2 + dz^2 of s' - r in float32, original coordinates) in index
-//     order; if a third chunk could (b3 <= b1 + 2 delta, rare), the warp scans
+//     (dx^2 + dy^2 + dz^2 of s' - r in float32, original coordinates), ties to the
+//     lower index; if a third chunk could (b3 <= b1 + 2 delta, rare), the warp scans
 //     the whole cloud for that query together.  The result is the lowest-index
 //     minimum of the exact-form float32 distance among all points that can be
 //     nearest.
@@ -40,11 +40,6 @@
 // Object tiles are staged in shared memory by 1D bulk (TMA) copies into two
 // buffers guarded by mbarriers; waits are bounded and report a timeout through
 // the error word instead of hanging.
-//
-// The epilogue accumulates, in float64, the sums that the cost and gradient of
-// Eqs. 13-17 are linear in: sum r_i (3), sum r_i s_i^T (9), sum |r_i|^2 (1),
-// with r_i the matched object point and s_i the untransformed gripper point;
-// both are float32, so every product is exact in float64.
 #include "asicp_internal.cuh"
 #include "async_copy.cuh"
 
