@@ -1298,7 +1298,9 @@ asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_
         ctx->pre_set[preshape] = 0;
         ctx->run_done = false;
         ctx->S.ensure(sizeof(float4) * (size_t)ctx->cfg.P * N, "gripper clouds");
-        ctx->stage.ensure(sizeof(float) * 3 * (size_t)N, "staging");
+        // (room for the clearances' intermediate grids too: growing the buffer between them waits for the device)
+        const size_t nc = sdf_cells_bytes(nx, ny, nz) / (2 * sizeof(float4));
+        ctx->stage.ensure(std::max(sizeof(float) * 3 * (size_t)N, nc), "staging");
         ck(cudaMemcpyAsync(ctx->stage.p, S_xyz, sizeof(float) * 3 * (size_t)N, cudaMemcpyDefault, ctx->st), "copy S");
         float4 *Sp = ctx->S.as<float4>() + (size_t)preshape * N;
         ck(launch_pack_points(ctx->stage.as<float>(), N, Sp, ctx->errw.as<int>(), ctx->st), "pack S");
@@ -1316,9 +1318,7 @@ asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_
         ctx->cells[preshape].ensure(sdf_cells_bytes(nx, ny, nz), "corner-packed sdf grid");
         ck(launch_sdf_pack_cells(ctx->grids[preshape].as<float>(), nx, ny, nz, ctx->cells[preshape].as<float4>(), ctx->st),
            "pack sdf cells");
-        const size_t nc = sdf_cells_bytes(nx, ny, nz) / (2 * sizeof(float4));
         ctx->clear[preshape].ensure(nc, "sdf clearances");
-        ctx->stage.ensure(nc, "staging");
         ck(launch_sdf_clear(ctx->cells[preshape].as<float4>(), nx, ny, nz, ctx->clear[preshape].as<unsigned char>(),
                             ctx->stage.as<unsigned char>(), ctx->st), "sdf clearances");
         finish(ctx, "set_gripper_sdf");
