@@ -286,7 +286,9 @@ __device__ __forceinline__ bool dispatch_pass(int qn, const FwdArgs &a, const Ob
 template <class Shape>
 __global__ void __launch_bounds__(Shape::kThreads, Shape::kMinBlocks) fwd_match_kernel(const FwdArgs a)
 {
-    if (a.check_err && *a.err != kDevOk) return;     // (asicp_match_noalloc: a rejected input leaves nn_idx alone)
+    // asicp_match_noalloc: a rejected input leaves nn_idx alone (one thread looks, so that a CTA leaves whole
+    // also when another CTA's wait expires meanwhile)
+    if (a.check_err && __syncthreads_or(threadIdx.x == 0 && *a.err != kDevOk)) return;
     constexpr int kThreads = Shape::kThreads;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ulonglong2 *tiles = reinterpret_cast<ulonglong2 *>(smem_raw);
