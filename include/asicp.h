@@ -329,6 +329,13 @@ asicp_status asicp_autotune(asicp_ctx *ctx, int *chosen, float *ms);
  * context. */
 asicp_status asicp_test_expire_waits(asicp_ctx *ctx, int on);
 
+/* The same for a proposal network (asicp_proposal.h): with on != 0 the encoder of
+ * later forward and loss_grad calls gives up after 1000 cycles, the call returns
+ * TIMEOUT (its outputs and the kept gradient are then undefined) and the handle
+ * stays usable.  Errors: none beyond a NULL handle. */
+struct asicp_prop;
+asicp_status asicp_test_expire_proposal_waits(struct asicp_prop *prop, int on);
+
 /* Message of the last failing call on ctx (owned by ctx, valid until its next call). */
 const char *asicp_last_error(const asicp_ctx *ctx);
 

@@ -28,7 +28,8 @@ EXPORTED = ("asicp_config_default", "asicp_create", "asicp_destroy", "asicp_set_
             "asicp_set_gripper_sdf", "asicp_set_state", "asicp_step", "asicp_run", "asicp_best_grasps",
             "asicp_get_state", "asicp_kernel_times", "asicp_last_error", "asicp_match_noalloc",
             "asicp_set_object_at", "asicp_set_particle_counts", "asicp_best_grasps_at", "asicp_autotune",
-            "asicp_set_minibatch", "asicp_set_convergence", "asicp_test_expire_waits")
+            "asicp_set_minibatch", "asicp_set_convergence", "asicp_test_expire_waits",
+            "asicp_test_expire_proposal_waits")
 
 
 class AsicpError(RuntimeError):
@@ -81,6 +82,7 @@ def load(build_if_missing: bool = True):
     lib.asicp_set_state.argtypes = [vp, vp, ip]
     lib.asicp_set_convergence.argtypes = [vp, vp, vp]
     lib.asicp_test_expire_waits.argtypes = [vp, ip]
+    lib.asicp_test_expire_proposal_waits.argtypes = [vp, ip]
     lib.asicp_step.argtypes = [vp, ip]
     lib.asicp_run.argtypes = [vp, vp]
     lib.asicp_best_grasps.argtypes = [vp, ip, vp, vp, vp, C.POINTER(C.c_int)]

@@ -146,7 +146,7 @@ static_assert(kTile * kH1 * 2 + kW2Bytes == kTile * kH2 * 2, "h2 takes the place
 __global__ void __launch_bounds__(kTile) encode_kernel(const float *clouds, int npts, const double *mean, const bf16 *W1,
                                                        const float *b1, const float *b2, const float *b3,
                                                        const unsigned char *wl, int store, bf16 *h1, bf16 *h2,
-                                                       unsigned long long *pool, int *err)
+                                                       unsigned long long *pool, int *err, int expire)
 {
     extern __shared__ __align__(1024) unsigned char sm_enc[];
     unsigned char *sA = sm_enc, *sW2 = sm_enc + kTile * kH1 * 2, *sW3 = sm_enc + kTile * kH2 * 2;
@@ -202,6 +202,7 @@ __global__ void __launch_bounds__(kTile) encode_kernel(const float *clouds, int 
     const uint32_t tmem = s_tmem, mine = tmem + ((uint32_t)(warp * 32) << 16);
     // all threads learn whether the weights landed, so that they leave together
     bool ok = mbar_wait_warp(&landed, 0);
+    if (expire) ok = mbar_wait(&done, 0, kTestWaitCycles);     // (nothing has been committed to it yet)
     ok = __syncthreads_and(ok);
     const bool first = ok;
     if (tid == 0 && ok) {
@@ -286,12 +287,13 @@ __global__ void __launch_bounds__(kTile) encode_kernel(const float *clouds, int 
     }
 }
 
-// Pooled value of a channel and the point it came from.
+// Pooled value of a channel and the point it came from.  A channel that no tile contributed to (its waits
+// expired) keeps key 0: value 0 at point 0, a valid row.
 __device__ __forceinline__ float pool_value(unsigned long long key)
 {
     return __uint_as_float((unsigned)(key >> 32) << 16);
 }
-__device__ __forceinline__ int pool_point(unsigned long long key) { return (int)(0xffffffffu - (unsigned)key); }
+__device__ __forceinline__ int pool_point(unsigned long long key) { return key ? (int)(0xffffffffu - (unsigned)key) : 0; }
 
 // ---------------------------------------------------------------- head
 // out[m][n] = sum_k A[m][k] W[k][n], k ascending, one thread per output of a tile of kHeadRows x
@@ -507,7 +509,8 @@ __global__ void __launch_bounds__(kLossThreads) loss_kernel(const float *out, co
 // (at most kH3; live[b] of them).  A CTA takes kBackRows of them:
 //   dh2[r][j] = h2 > 0 ? sum over the channels pooled from r, ascending, of dg[ch] W3[ch][j] : 0,
 //   dh1[r][k] = h1 > 0 ? sum_j dh2[r][j] W2[j][k] : 0
-// into compact rows.  dg is already 0 where the pooled value is not positive.
+// into compact rows.  dg is already 0 where the pooled value is not positive.  After an expired wait of the encoder
+// (*err) this kernel and the two after it leave everything alone; the call returns TIMEOUT.
 // Measured on GB300 (32 clouds of 2048 points): this kernel, back_slices_kernel and grad_kernel 36 + 13
 // + 12 us, against 1.4 ms for dense float32 products over all points, their bias sums and the
 // slices of every parameter.
@@ -515,8 +518,9 @@ constexpr int kBackRows = 32;
 
 __global__ void __launch_bounds__(256) back_rows_kernel(const unsigned long long *pool, const float *dg, const bf16 *W3,
                                                         const bf16 *W2, const bf16 *h2, const bf16 *h1, int npts, int *live,
-                                                        int *rows, float *dh2, float *dh1)
+                                                        int *rows, float *dh2, float *dh1, const int *err)
 {
+    if (*err != kDevOk) return;
     __shared__ unsigned s_key[kH3];        // (point, channel), sorted
     __shared__ int s_first[kH3 + 1], s_wsum[8];
     __shared__ float s_d2[kBackRows][kH2];
@@ -597,8 +601,9 @@ constexpr int kSlice = kH2 * kH1 + kH2 + kH1 * 3 + kH1;
 
 __global__ void __launch_bounds__(256) back_slices_kernel(const float *clouds, const double *mean, const int *live,
                                                           const int *rows, const float *dh2, const float *dh1,
-                                                          const bf16 *h1, int npts, float *slices)
+                                                          const bf16 *h1, int npts, float *slices, const int *err)
 {
+    if (*err != kDevOk) return;
     constexpr int kRowsTile = 128, kCols = kH2 / 8;     // rows staged together; rows of dW2 per CTA
     __shared__ __align__(16) unsigned char sm[kRowsTile * kH1 * 4];
     __shared__ float s_d2[kRowsTile][kCols];
@@ -661,8 +666,9 @@ __global__ void __launch_bounds__(256) back_slices_kernel(const float *clouds, c
 __global__ void __launch_bounds__(256) grad_kernel(const float *dO, const bf16 *z, const float *dz,
                                                    const unsigned long long *pool, const float *dg, const bf16 *h2,
                                                    const float *slices, int npts, int B, int no, size_t w2, size_t w3,
-                                                   size_t w4, size_t w5, size_t np, float *grad)
+                                                   size_t w4, size_t w5, size_t np, float *grad, const int *err)
 {
+    if (*err != kDevOk) return;
     const size_t j = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (j >= np) return;
     float s = 0.f;
@@ -792,6 +798,7 @@ struct asicp_prop {
     cudaStream_t st = nullptr;
     long long step = 0;
     int lastB = 0;
+    int expire_test = 0;               // the encoder's first wait expires (testing)
     unsigned char *pin = nullptr;      // page-locked memory: inputs, then results; or null
     ~asicp_prop() { if (pin) cudaFreeHost(pin); }
     Buf w, m, v, grad, slices, wbf, wt4, wt5, wl, clouds, tg, cen, mean, h1, h2, pool, z, o, dO, lossp, dz, dg, live,
@@ -888,7 +895,8 @@ void forward_impl(asicp_prop *pr, const float *clouds_dev, int B, bool store)
     pck(cudaGetLastError());
     encode_kernel<<<dim3((pr->npts + kTile - 1) / kTile, B), kTile, kEncSmem, st>>>(
         clouds_dev, pr->npts, pr->mean.as<double>(), pr->wbf.as<bf16>() + pr->L[0].w, wf + pr->L[0].b, wf + pr->L[1].b,
-        wf + pr->L[2].b, pr->wl.as<unsigned char>(), store, pr->h1.as<bf16>(), pr->h2.as<bf16>(), pool, pr->errw.as<int>());
+        wf + pr->L[2].b, pr->wl.as<unsigned char>(), store, pr->h1.as<bf16>(), pr->h2.as<bf16>(), pool, pr->errw.as<int>(),
+        pr->expire_test);
     pck(cudaGetLastError());
     pck(launch_head<kZ>(pool, pr->wt4.as<bf16>(), wf + pr->L[3].b, nullptr, nullptr, pr->z.p, B, kHead, kH3, st));
     pck(launch_head<kO>(pr->z.p, pr->wt5.as<bf16>(), wf + pr->L[4].b, nullptr, nullptr, pr->o.p, B, pr->nout, kHead, st));
@@ -900,18 +908,19 @@ void backward_impl(asicp_prop *pr, const float *clouds_dev, int B)
     const int n = pr->npts, no = pr->nout;
     const bf16 *W = pr->wbf.as<bf16>(), *z = pr->z.as<bf16>(), *h1 = pr->h1.as<bf16>(), *h2 = pr->h2.as<bf16>();
     const unsigned long long *pool = pr->pool.as<unsigned long long>();
+    const int *err = pr->errw.as<int>();
     float *dz = pr->dz.as<float>(), *dg = pr->dg.as<float>(), *dh2 = pr->dh2.as<float>(), *dh1 = pr->dh1.as<float>();
     pck(launch_head<kDz>(pr->dO.p, W + pr->L[4].w, nullptr, z, nullptr, dz, B, kHead, no, st));
     pck(launch_head<kDg>(dz, W + pr->L[3].w, nullptr, nullptr, pool, dg, B, kH3, kHead, st));
     back_rows_kernel<<<dim3(kH3 / kBackRows, B), 256, 0, st>>>(pool, dg, W + pr->L[2].w, W + pr->L[1].w, h2, h1, n,
-                                                              pr->live.as<int>(), pr->rows.as<int>(), dh2, dh1);
+                                                              pr->live.as<int>(), pr->rows.as<int>(), dh2, dh1, err);
     pck(cudaGetLastError());
     back_slices_kernel<<<dim3(9, B), 256, 0, st>>>(clouds_dev, pr->mean.as<double>(), pr->live.as<int>(), pr->rows.as<int>(),
-                                                   dh2, dh1, h1, n, pr->slices.as<float>());
+                                                   dh2, dh1, h1, n, pr->slices.as<float>(), err);
     pck(cudaGetLastError());
     grad_kernel<<<(unsigned)((pr->np + 255) / 256), 256, 0, st>>>(pr->dO.as<float>(), z, dz, pool, dg, h2,
                                                                   pr->slices.as<float>(), n, B, no, pr->L[1].w, pr->L[2].w,
-                                                                  pr->L[3].w, pr->L[4].w, pr->np, pr->grad.as<float>());
+                                                                  pr->L[3].w, pr->L[4].w, pr->np, pr->grad.as<float>(), err);
     pck(cudaGetLastError());
 }
 
@@ -1090,6 +1099,13 @@ asicp_status asicp_prop_sample(asicp_prop *pr, const float *out, const float *ce
         t.store(theta, pr->stheta.p, n * 7 * 4);
         t.finish();
     });
+}
+
+asicp_status asicp_test_expire_proposal_waits(asicp_prop *pr, int on)
+{
+    if (!pr) return ASICP_ERR_INVALID_ARG;
+    pr->expire_test = on != 0;
+    return ASICP_OK;
 }
 
 }  // extern "C"

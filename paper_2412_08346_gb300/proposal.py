@@ -96,6 +96,9 @@ class Proposal:
                                         asicp._ptr(grad)), "asicp_prop_loss_grad")
         return float(loss.value), grad
 
+    def test_expire_waits(self, on: bool):
+        _ok(_lib().asicp_test_expire_proposal_waits(self.h, int(bool(on))), "asicp_test_expire_proposal_waits")
+
     def adam_step(self, lr: float):
         _ok(_lib().asicp_prop_adam_step(self.h, float(lr)), "asicp_prop_adam_step")
 
