@@ -154,6 +154,7 @@ struct asicp_ctx {
     // mini-batches of the object cloud per iteration (Table I), one object only
     std::vector<int> mb_off;          // [iters + 1] on the host (sizes are fixed at capture)
     DevMem mb_idx, mb_R, mb_Rx;
+    bool table_mb = false;            // the object table on the device points at a mini-batch
 
     int fwd_variant = 0;              // forward-matching kernel shape (autotuner's choice)
     bool tuned = false;
@@ -519,6 +520,7 @@ void build_layout(asicp_ctx *c)
        "object table");
     ck(cudaStreamSynchronize(c->st), "layout");
     c->layout_dirty = false;
+    c->table_mb = false;
     plan_fwd_items(c, c->fwd_variant);
 }
 
@@ -588,7 +590,8 @@ void select_minibatch(asicp_ctx *c, int k)
     if (c->mb_off.empty()) return;
     cudaStream_t st = work_stream(c);
     ObjMeta m = c->objmeta_h[0];
-    if (k >= 0 && k + 1 < (int)c->mb_off.size()) {
+    c->table_mb = k >= 0 && k + 1 < (int)c->mb_off.size();
+    if (c->table_mb) {
         const int first = c->mb_off[k], cnt = c->mb_off[k + 1] - first;
         const int Mpad = (cnt + kRefTilePts - 1) / kRefTilePts * kRefTilePts;
         m.R = c->mb_R.as<float4>();
@@ -601,6 +604,15 @@ void select_minibatch(asicp_ctx *c, int k)
         return;
     }
     ck(launch_store_meta(c->objmeta.as<ObjMeta>(), m, st), "object table");
+}
+
+// No mini-batches from here on: a table that a step has left at one points at the whole cloud again.
+void drop_minibatches(asicp_ctx *c)
+{
+    c->mb_off.clear();
+    if (!c->table_mb) return;
+    c->table_mb = false;                  // (a layout to be rebuilt writes the whole table)
+    if (!c->layout_dirty) ck(launch_store_meta(c->objmeta.as<ObjMeta>(), c->objmeta_h[0], c->st), "object table");
 }
 
 // Build the cells of the given clouds (at most kCellBatch of them, or as many as the scratch
@@ -989,6 +1001,7 @@ void run_loop_graph(asicp_ctx *c)
     }
     accumulate_graph_events(c);
     ck(cudaGraphLaunch(c->loop_exec, c->st), "graph launch");
+    if (!c->mb_off.empty()) c->table_mb = false;     // (the loop ends on the whole cloud)
     c->graph_pending = c->cfg.profile != 0;
 }
 
@@ -1075,9 +1088,7 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
     if (C_xyz && Mc < 1) fail(ASICP_ERR_INVALID_ARG, "set_object: Mc must be >= 1 when C is given");
     ObjBufs &b = ctx->objs[o];
     const int mc = C_xyz ? Mc : M;
-    if (!ctx->mb_off.empty()) {   // mini-batches index the previous cloud
-        ctx->mb_off.clear();
-    }
+    drop_minibatches(ctx);        // they index the previous cloud
     // what the layout (object table, work plan) and the captured loop depend on
     const bool was_set = b.set;
     const void *was[6] = {b.R.p, b.Rx.p, b.Rt.p, b.C.p, b.Csort.p, b.Cball.p};
@@ -1243,7 +1254,7 @@ asicp_status asicp_set_minibatch(asicp_ctx *ctx, const int *offsets, const int *
 {
     return guarded(ctx, [&] {
         if (!offsets) {
-            ctx->mb_off.clear();
+            drop_minibatches(ctx);
             return;
         }
         if (ctx->nobj != 1) fail(ASICP_ERR_INVALID_ARG, "set_minibatch: one object per context");
@@ -1264,6 +1275,7 @@ asicp_status asicp_set_minibatch(asicp_ctx *ctx, const int *offsets, const int *
                 if (idx[i] < 0 || idx[i] >= M || (i > off[k] && idx[i] <= idx[i - 1]))
                     fail(ASICP_ERR_INVALID_ARG, "set_minibatch: indices must be ascending within [0, M)");
         const int Mpad = (M + kRefTilePts - 1) / kRefTilePts * kRefTilePts;
+        drop_minibatches(ctx);    // (growing the buffers may fail: the old ramp must not outlive them)
         ctx->mb_idx.ensure(sizeof(int) * idx.size(), "mini-batch indices");
         ctx->mb_R.ensure(sizeof(float4) * M, "mini-batch points");
         ctx->mb_Rx.ensure(sizeof(float4) * Mpad, "mini-batch screening layout");
