@@ -220,8 +220,13 @@ asicp_status asicp_set_convergence(asicp_ctx *ctx, const double *prev_cost, cons
 /* One iteration k (0 <= k < k_max) of Algorithm 1 for all preshapes and
  * particles: transform, match, cost/gradient, collision test and collision
  * gradient, then the SVGD update (k < k_stein, Eqs. 7-11) or the SGD-ICP update
- * (Eq. 3).  Errors: STATE (inputs or poses not set, or sizes changed since the
- * poses were set), INVALID_ARG (k), CUDA. */
+ * (Eq. 3).  The call enqueues its kernels and returns, but for the call in which
+ * cells become due (see config.fwd_shape and asicp_set_gripper_sdf): that one
+ * allocates and may wait.  While cuda_stream is being captured by the caller, a step
+ * is launches only, matches without cells and sorts the collision clouds itself, so
+ * that a replay follows new objects and grippers of the same sizes.
+ * Errors: STATE (inputs or poses not set, or sizes changed since the poses were
+ * set), INVALID_ARG (k), CUDA. */
 asicp_status asicp_step(asicp_ctx *ctx, int k);
 
 /* Full optimisation of every object's grasp set: initial poses theta0 (T*7,

@@ -164,6 +164,7 @@ struct asicp_ctx {
     bool pre_oom = false;             // no room for the gripper clouds' cells
     bool pre_built = false;           // the gripper clouds' cells are built (all preshapes together)
     double pre_owed = 0.0;            // microseconds of reverse matching without them so far
+    bool recording = false;           // the caller's stream is being captured (see note_capture)
     bool expire_test = false;         // the float32 matching kernels' first copy waits expire (testing)
 
     // layout (rebuilt when objects, particle counts or N change)
@@ -661,7 +662,7 @@ void build_cells(asicp_ctx *c, const std::vector<CellBuild> &todo)
 void ensure_cells(asicp_ctx *c, int v, int passes)
 {
     c->cells_on = false;
-    if (v != kFwdVariants - 1 || c->cells_oom) return;
+    if (v != kFwdVariants - 1 || c->cells_oom || c->recording) return;
     std::vector<int> todo;
     int most = 0;
     double pairs = 0.0, points = 0.0;
@@ -719,14 +720,27 @@ void ensure_cells(asicp_ctx *c, int v, int passes)
     for (int o : todo) c->objs[o].cells_built = true;
 }
 
-// Sort the collision clouds that are new into their spatial order (before the kernels run, and
-// outside any capture), those of all objects together.
+// Whether the caller's own stream is being captured: the launches of this call run when its graph is replayed,
+// each time on the clouds the context then holds.  Nothing they prepare may count as done, and nothing that was
+// prepared from the present clouds may be recorded.
+void note_capture(asicp_ctx *c)
+{
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->st, &s) != cudaSuccess) {
+        cudaGetLastError();
+        s = cudaStreamCaptureStatusNone;
+    }
+    c->recording = s != cudaStreamCaptureStatusNone;
+}
+
+// Sort the collision clouds that are new (in a capture: all of them, at every replay) into their spatial
+// order before the kernels run, those of all objects together.
 void ensure_sorted(asicp_ctx *c)
 {
     CloudBatch batch{};
     int n = 0;
-    for (ObjBufs &o : c->objs) {
-        if (o.sorted) continue;
+    for (const ObjBufs &o : c->objs) {
+        if (o.sorted && !c->recording) continue;
         const float4 *src = o.C.p ? o.C.as<float4>() : o.R.as<float4>();
         for (int seg = 0; seg < o.Mc; seg += kColSegment) {
             batch.b[n++] = {src + seg, o.Csort.as<float4>() + seg, o.Cball.as<float4>() + seg / 32,
@@ -736,9 +750,10 @@ void ensure_sorted(asicp_ctx *c)
                 n = 0;
             }
         }
-        o.sorted = true;
     }
     if (n > 0) ck(launch_sort_clouds(batch, n, c->st), "collision cloud order");
+    if (!c->recording)
+        for (ObjBufs &o : c->objs) o.sorted = true;
 }
 
 // Decide whether the reverse matching of the next `passes` passes goes through the cells of the
@@ -750,7 +765,7 @@ constexpr double kPreRate = 5.7e6;
 
 void ensure_pre_cells(asicp_ctx *c, int passes)
 {
-    if (c->pre_built || c->pre_oom || c->N < kPreMinN) return;
+    if (c->pre_built || c->pre_oom || c->N < kPreMinN || c->recording) return;
     double tests = 0.0;
     for (const ObjMeta &m : c->objmeta_h) tests += (double)m.np * m.Mc;
     c->pre_owed += passes * (5.0 + tests / 32.0 * c->N / kPreRate);
@@ -873,7 +888,7 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
     ca.col_items = c->colitems.as<int>();
     ca.col_list = c->collist.as<int>();
     for (const ObjMeta &m : c->objmeta_h) ca.most_points = std::max(ca.most_points, m.Mc);
-    ca.cells = c->pre_built;
+    ca.cells = c->pre_built && !c->recording;
     if (ca.cells) {
         const CellSizes s = cell_sizes(c->N);
         ca.pre_nodes = c->prenodes.as<int2>();
@@ -1389,6 +1404,7 @@ asicp_status asicp_step(asicp_ctx *ctx, int k)
         if (!ctx->inputs_ready() || !ctx->theta_set) fail(ASICP_ERR_STATE, "step: inputs and poses must be set first");
         if (ctx->layout_dirty) fail(ASICP_ERR_STATE, "step: inputs changed since the poses were set");
         if (k < 0 || k >= ctx->cfg.k_max) fail(ASICP_ERR_INVALID_ARG, "step: k out of [0, k_max)");
+        note_capture(ctx);
         ensure_cells(ctx, ctx->fwd_variant, 1);
         ensure_pre_cells(ctx, 1);
         ensure_sorted(ctx);
@@ -1415,6 +1431,7 @@ asicp_status asicp_run(asicp_ctx *ctx, const float *theta0)
                "initial poses");
         }
         ctx->theta_set = true;
+        note_capture(ctx);
         if (ctx->cfg.autotune && !ctx->tuned) autotune_impl(ctx, nullptr);
         ensure_cells(ctx, ctx->fwd_variant, ctx->cfg.k_max + 1);
         ensure_pre_cells(ctx, ctx->cfg.k_max + 1);
@@ -1508,6 +1525,7 @@ asicp_status asicp_autotune(asicp_ctx *ctx, int *chosen, float *ms)
             ctx->theta_set = true;
             ctx->stepped = false;
         }
+        note_capture(ctx);
         autotune_impl(ctx, ms);
         if (chosen) *chosen = ctx->fwd_variant;
     });
