@@ -77,7 +77,9 @@ typedef enum {
  *                  tensor-core screening with its exact-choice kernel (not with mini-batches),
  *                  which clouds of 1024 to 2^18 points replace, once the passes so far would
  *                  have paid for the build, by cells around the object that keep the points
- *                  which can be nearest in them (same results).
+ *                  which can be nearest in them (same results).  Cells take 9.7 MB and
+ *                  1.15 KB per point of every object, at most an eighth of the free
+ *                  device memory in all; without room the screening goes on.
  *                  Every shape returns the lowest-index minimum of the exact-form float32
  *                  distance over the points that can be nearest; they can differ only where
  *                  several points' float32 distances tie within rounding (near-ties)
@@ -193,7 +195,9 @@ asicp_status asicp_set_particle_counts(asicp_ctx *ctx, const int *K, int n);
  * (1 <= N <= 6144).  The context keeps a copy of the grid, a corner-packed
  * copy for the lookups (32 bytes per cell: 8 (nx-1)(ny-1)(nz-1) floats) and a byte
  * per cell for its distance to the gripper; for N >= 512 also cells around S for
- * the reverse matching.
+ * the reverse matching (9.7 MB and 1.15 KB per point each and one int per particle and
+ * collision point, at most an eighth of the free device memory; built once the passes
+ * so far would have paid for it).
  * Errors: INVALID_ARG (index, N out of range, a grid dimension < 2, voxel <= 0, N differing
  * from an earlier preshape, non-finite value). */
 asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_xyz, int N,
@@ -340,6 +344,12 @@ asicp_status asicp_test_expire_waits(asicp_ctx *ctx, int on);
  * stays usable.  Errors: none beyond a NULL handle. */
 struct asicp_prop;
 asicp_status asicp_test_expire_proposal_waits(struct asicp_prop *prop, int on);
+
+/* Testing aid for the fallback without cells: after `after` more successful
+ * allocations for cells the next one fails as if the device had no memory left
+ * (after < 0: off).  The context then gives the cells' memory back and goes on
+ * without them.  Errors: none beyond a NULL context. */
+asicp_status asicp_test_fail_cell_memory(asicp_ctx *ctx, int after);
 
 /* Message of the last failing call on ctx (owned by ctx, valid until its next call). */
 const char *asicp_last_error(const asicp_ctx *ctx);

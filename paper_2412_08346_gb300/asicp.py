@@ -29,7 +29,7 @@ EXPORTED = ("asicp_config_default", "asicp_create", "asicp_destroy", "asicp_set_
             "asicp_get_state", "asicp_kernel_times", "asicp_last_error", "asicp_match_noalloc",
             "asicp_set_object_at", "asicp_set_particle_counts", "asicp_best_grasps_at", "asicp_autotune",
             "asicp_set_minibatch", "asicp_set_convergence", "asicp_test_expire_waits",
-            "asicp_test_expire_proposal_waits")
+            "asicp_test_expire_proposal_waits", "asicp_test_fail_cell_memory")
 
 
 class AsicpError(RuntimeError):
@@ -83,6 +83,7 @@ def load(build_if_missing: bool = True):
     lib.asicp_set_convergence.argtypes = [vp, vp, vp]
     lib.asicp_test_expire_waits.argtypes = [vp, ip]
     lib.asicp_test_expire_proposal_waits.argtypes = [vp, ip]
+    lib.asicp_test_fail_cell_memory.argtypes = [vp, ip]
     lib.asicp_step.argtypes = [vp, ip]
     lib.asicp_run.argtypes = [vp, vp]
     lib.asicp_best_grasps.argtypes = [vp, ip, vp, vp, vp, C.POINTER(C.c_int)]
@@ -192,6 +193,10 @@ def asicp_set_convergence(ctx, prev_cost=None, frozen=None) -> None:
 
 def asicp_test_expire_waits(ctx, on: bool) -> None:
     _check(ctx, load().asicp_test_expire_waits(ctx, int(bool(on))))
+
+
+def asicp_test_fail_cell_memory(ctx, after: int) -> None:
+    _check(ctx, load().asicp_test_fail_cell_memory(ctx, int(after)))
 
 
 def asicp_step(ctx, k: int) -> None:

@@ -162,6 +162,7 @@ struct asicp_ctx {
     bool cells_on = false;            // the passes being launched match through the cells
     double cells_owed = 0.0;          // microseconds of screening on the present objects so far
     bool pre_oom = false;             // no room for the gripper clouds' cells
+    int fail_cells = -1;              // this many more allocations for cells succeed, the next fails (testing; < 0: off)
     bool pre_built = false;           // the gripper clouds' cells are built (all preshapes together)
     double pre_owed = 0.0;            // microseconds of reverse matching without them so far
     bool recording = false;           // the caller's stream is being captured (see note_capture)
@@ -498,7 +499,6 @@ void build_layout(asicp_ctx *c)
     c->tccand.ensure(sizeof(int4) * (size_t)T * N, "tensor-core candidate chunks");
     c->ncol.ensure(sizeof(int) * T, "ncol");
     c->colidx.ensure(sizeof(int) * std::max<long long>(1, colidx_total), "colidx");
-    c->colsrt.ensure(sizeof(int) * std::max<long long>(1, colidx_total), "colsrt");
     c->colnn.ensure(sizeof(int) * std::max<long long>(1, colidx_total), "colnn");
     c->cost.ensure(sizeof(double) * T, "cost");
     c->grad.ensure(sizeof(double) * T * 8, "grad");
@@ -621,16 +621,16 @@ void drop_minibatches(asicp_ctx *c)
 size_t cell_scratch(const CellSizes &s) { return 2 * sizeof(int) * (size_t)s.list_cap + s.rec_bytes; }
 constexpr size_t kCellCtrBytes = sizeof(int) * kCellCounters * kCellBatch;
 
-void ensure_cell_scratch(asicp_ctx *c, const std::vector<CellBuild> &todo)
+size_t scratch_bytes(const std::vector<int> &sizes)
 {
     size_t need = 0, sum = 0;
-    for (size_t i = 0, first = 0; i < todo.size(); ++i) {
-        const size_t w = cell_scratch(cell_sizes(todo[i].M));
+    for (size_t i = 0, first = 0; i < sizes.size(); ++i) {
+        const size_t w = cell_scratch(cell_sizes(sizes[i]));
         if (i > first && (sum + w > kCellScratch || i - first == kCellBatch)) { sum = 0; first = i; }
         sum += w;
         need = std::max(need, sum);
     }
-    c->cellwork.ensure(kCellCtrBytes + need, "matching cells' scratch");
+    return kCellCtrBytes + need;
 }
 
 void build_cells(asicp_ctx *c, const std::vector<CellBuild> &todo)
@@ -654,6 +654,24 @@ void build_cells(asicp_ctx *c, const std::vector<CellBuild> &todo)
         ck(cudaMemsetAsync(c->cellwork.p, 0, kCellCtrBytes, c->st), "matching cells");
         ck(launch_cells_build(batch, n, c->st), "matching cells");
     }
+}
+
+// Memory for cells.  They only make passes faster, so they take at most an eighth of what is free on the device
+// (their size is a bound for any cloud, 9.7 MB and 1.15 KB per point of an object, and a few MB of it are used);
+// without room the kernels that need none run.
+void need_room(const std::vector<std::pair<const DevMem *, size_t>> &wants)
+{
+    size_t more = 0, avail = 0, total = 0;
+    for (const auto &w : wants) more += w.second > w.first->bytes ? w.second - w.first->bytes : 0;
+    if (more == 0) return;
+    ck(cudaMemGetInfo(&avail, &total), "free memory");
+    if (more > avail / 8) fail(ASICP_ERR_OOM, "cells would take more than an eighth of the free memory");
+}
+
+void cell_memory(asicp_ctx *c, DevMem &m, size_t bytes, const char *what)
+{
+    if (c->fail_cells >= 0 && c->fail_cells-- == 0) fail(ASICP_ERR_OOM, what);
+    m.ensure(bytes, what);
 }
 
 // Decide whether the next `passes` passes of kernel shape v match through the cells, and build
@@ -683,12 +701,23 @@ void ensure_cells(asicp_ctx *c, int v, int passes)
     std::vector<CellBuild> builds;
     bool moved = false;
     try {
+        std::vector<std::pair<const DevMem *, size_t>> wants;
+        std::vector<int> sizes;
+        for (int i : todo) {
+            sizes.push_back(c->objs[i].M);
+            const CellSizes s = cell_sizes(c->objs[i].M);
+            wants.push_back({&c->objs[i].nodes, sizeof(int2) * (size_t)s.node_cap});
+            wants.push_back({&c->objs[i].leaves, sizeof(int) * (size_t)s.leaf_cap});
+        }
+        wants.push_back({&c->cellwork, scratch_bytes(sizes)});
+        need_room(wants);
+        cell_memory(c, c->cellwork, scratch_bytes(sizes), "matching cells' scratch");
         for (int i : todo) {
             ObjBufs &o = c->objs[i];
             const CellSizes s = cell_sizes(o.M);
             const void *was[2] = {o.nodes.p, o.leaves.p};
-            o.nodes.ensure(sizeof(int2) * (size_t)s.node_cap, "matching cells");
-            o.leaves.ensure(sizeof(int) * (size_t)s.leaf_cap, "matching cells");
+            cell_memory(c, o.nodes, sizeof(int2) * (size_t)s.node_cap, "matching cells");
+            cell_memory(c, o.leaves, sizeof(int) * (size_t)s.leaf_cap, "matching cells");
             moved = moved || o.nodes.p != was[0] || o.leaves.p != was[1];
             CellBuild b{};
             b.R = o.R.as<float4>();
@@ -699,12 +728,18 @@ void ensure_cells(asicp_ctx *c, int v, int passes)
             b.log_factor = kObjectCells;
             builds.push_back(b);
         }
-        ensure_cell_scratch(c, builds);
     } catch (const Err &e) {
         if (e.st != ASICP_ERR_OOM) throw;
+        // nothing is kept: the memory is the caller's again, and the table holds no pointer into it
         c->cells_oom = true;
         c->cells_on = false;
         c->cellwork.release();
+        for (ObjBufs &o : c->objs) {
+            o.nodes.release();
+            o.leaves.release();
+            o.cells_built = false;
+        }
+        moved = true;
     }
     if (moved) {
         for (int o = 0; o < c->nobj; ++o) {
@@ -765,37 +800,52 @@ constexpr double kPreRate = 5.7e6;
 
 void ensure_pre_cells(asicp_ctx *c, int passes)
 {
-    if (c->pre_built || c->pre_oom || c->N < kPreMinN || c->recording) return;
-    double tests = 0.0;
-    for (const ObjMeta &m : c->objmeta_h) tests += (double)m.np * m.Mc;
-    c->pre_owed += passes * (5.0 + tests / 32.0 * c->N / kPreRate);
+    if (c->pre_oom || c->N < kPreMinN || c->recording) return;
     const int P = c->cfg.P;
-    if (c->pre_owed <= 150.0 + (double)P * c->N / kCellRatePts) return;
+    const size_t list = sizeof(int) * (size_t)std::max<long long>(1, c->colidx_total);
+    if (c->pre_built) {
+        if (list <= c->colsrt.bytes) return;
+    } else {
+        double tests = 0.0;
+        for (const ObjMeta &m : c->objmeta_h) tests += (double)m.np * m.Mc;
+        c->pre_owed += passes * (5.0 + tests / 32.0 * c->N / kPreRate);
+        if (c->pre_owed <= 150.0 + (double)P * c->N / kCellRatePts) return;
+    }
     std::vector<CellBuild> builds;
     const CellSizes s = cell_sizes(c->N);
+    const size_t nodes = sizeof(int2) * (size_t)s.node_cap * P, leaves = sizeof(int) * (size_t)s.leaf_cap * P;
     try {
-        c->prenodes.ensure(sizeof(int2) * (size_t)s.node_cap * P, "gripper cells");
-        c->preleaves.ensure(sizeof(int) * (size_t)s.leaf_cap * P, "gripper cells");
-        for (int p = 0; p < P; ++p) {
-            CellBuild b{};
-            b.R = c->S.as<float4>() + (size_t)p * c->N;
-            b.frame = c->preframe.as<float4>() + p;
-            b.nodes = c->prenodes.as<int2>() + (size_t)p * s.node_cap;
-            b.leaves = c->preleaves.as<int>() + (size_t)p * s.leaf_cap;
-            b.M = c->N;
-            b.log_factor = kGripperCells;
-            b.tol = kGripperTol;
-            b.near_only = 1;
-            builds.push_back(b);
+        const size_t scratch = c->pre_built ? 0 : scratch_bytes(std::vector<int>(P, c->N));
+        need_room({{&c->prenodes, nodes}, {&c->preleaves, leaves}, {&c->colsrt, list}, {&c->cellwork, scratch}});
+        cell_memory(c, c->colsrt, list, "colliding points in spatial order");
+        if (!c->pre_built) {
+            cell_memory(c, c->cellwork, scratch, "gripper cells' scratch");
+            cell_memory(c, c->prenodes, nodes, "gripper cells");
+            cell_memory(c, c->preleaves, leaves, "gripper cells");
+            for (int p = 0; p < P; ++p) {
+                CellBuild b{};
+                b.R = c->S.as<float4>() + (size_t)p * c->N;
+                b.frame = c->preframe.as<float4>() + p;
+                b.nodes = c->prenodes.as<int2>() + (size_t)p * s.node_cap;
+                b.leaves = c->preleaves.as<int>() + (size_t)p * s.leaf_cap;
+                b.M = c->N;
+                b.log_factor = kGripperCells;
+                b.tol = kGripperTol;
+                b.near_only = 1;
+                builds.push_back(b);
+            }
         }
-        ensure_cell_scratch(c, builds);
     } catch (const Err &e) {
         if (e.st != ASICP_ERR_OOM) throw;
         c->pre_oom = true;
+        c->pre_built = false;
         c->prenodes.release();
         c->preleaves.release();
+        c->colsrt.release();
+        c->cellwork.release();
         return;
     }
+    if (c->pre_built) return;
     build_cells(c, builds);
     c->pre_built = true;
 }
@@ -882,7 +932,6 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
     ca.S = c->S.as<float4>();
     ca.ncol = c->ncol.as<int>();
     ca.colidx = c->colidx.as<int>();
-    ca.colsrt = c->colsrt.as<int>();
     ca.colnn = c->colnn.as<int>();
     ca.colmap = c->colmap.as<int2>();
     ca.col_items = c->colitems.as<int>();
@@ -890,6 +939,7 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
     for (const ObjMeta &m : c->objmeta_h) ca.most_points = std::max(ca.most_points, m.Mc);
     ca.cells = c->pre_built && !c->recording;
     if (ca.cells) {
+        ca.colsrt = c->colsrt.as<int>();
         const CellSizes s = cell_sizes(c->N);
         ca.pre_nodes = c->prenodes.as<int2>();
         ca.pre_leaves = c->preleaves.as<int>();
@@ -1534,6 +1584,11 @@ asicp_status asicp_autotune(asicp_ctx *ctx, int *chosen, float *ms)
 asicp_status asicp_test_expire_waits(asicp_ctx *ctx, int on)
 {
     return guarded(ctx, [&] { ctx->expire_test = on != 0; });
+}
+
+asicp_status asicp_test_fail_cell_memory(asicp_ctx *ctx, int after)
+{
+    return guarded(ctx, [&] { ctx->fail_cells = after; });
 }
 
 asicp_status asicp_kernel_times(asicp_ctx *ctx, double ms[ASICP_KERNEL_KINDS], long long launches[ASICP_KERNEL_KINDS],

@@ -339,7 +339,7 @@ struct CollideArgs {
     const float4 *S;          // [P][N]
     int *ncol;                // [T]
     int *colidx;              // colliding points, ascending (see ObjMeta::colidx_base)
-    int *colsrt;              // the same points as positions in Csort, in no particular order
+    int *colsrt;              // the same points as positions in Csort, in no particular order (cells only)
     int *colnn;               // like colidx: nearest gripper point of each
     int2 *colmap;             // bit map of the colliding points: words (bits, number of earlier bits),
                               // only those with bits written (see ObjMeta::colmap_base)
