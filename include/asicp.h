@@ -79,7 +79,9 @@ typedef enum {
  *                  have paid for the build, by cells around the object that keep the points
  *                  which can be nearest in them (same results).  Cells take 9.7 MB and
  *                  1.15 KB per point of every object, at most an eighth of the free
- *                  device memory in all; without room the screening goes on.
+ *                  device memory in all; without room, and for clouds on which they
+ *                  would be slower (points on a common sphere, cylinder or plane,
+ *                  many copies of a point), the screening goes on.
  *                  Every shape returns the lowest-index minimum of the exact-form float32
  *                  distance over the points that can be nearest; they can differ only where
  *                  several points' float32 distances tie within rounding (near-ties)

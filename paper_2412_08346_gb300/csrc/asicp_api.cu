@@ -127,6 +127,12 @@ struct ObjBufs {
 // through the cells little beside either.
 constexpr int kCellMinM = 1024, kCellMaxM = 1 << 18;
 constexpr double kCellRate = 1.65e7, kCellRatePts = 50.0;
+// Clouds whose lists do not shrink (points on a common sphere or plane, many copies of a point) are matched faster by
+// the screening.  So the work of one pass is counted on a sample of the queries when cells have been built (see
+// cells_cost_kernel): a pass takes 1 us per kCellRounds rounds, or, where few warps have long lists, kCellLatency us
+// per round of the longest one.  What it saves of the screening, but at least kCellGain of it, is what the next
+// clouds' build is weighed against.
+constexpr double kCellRounds = 7.5e4, kCellLatency = 0.15, kCellGain = 1.0 / 32.0;
 constexpr size_t kCellScratch = (size_t)256 << 20;   // scratch of one build launch (at least one object)
 
 enum { kTimeMatch = 0, kTimeCollide = 1, kTimeCollideNN = 2, kTimeFinalize = 3, kTimeStein = 4, kTimeExact = 5,
@@ -160,6 +166,9 @@ struct asicp_ctx {
     bool tuned = false;
     bool cells_oom = false;           // no room for matching cells: the screening is used
     bool cells_on = false;            // the passes being launched match through the cells
+    bool cells_slow = false;          // the present objects' cells are built, but the screening is the faster
+    double cells_gain = 1.0;          // share of a screening pass that the cells save, as last seen
+    double cells_share = 0.0;         // sample of the cost count that has been enqueued (0: none)
     double cells_owed = 0.0;          // microseconds of screening on the present objects so far
     bool pre_oom = false;             // no room for the gripper clouds' cells
     int fail_cells = -1;              // this many more allocations for cells succeed, the next fails (testing; < 0: off)
@@ -201,6 +210,7 @@ struct asicp_ctx {
     // the collision test's branch of a pass and the events that part and join the two
     cudaStream_t side_st = nullptr;
     cudaEvent_t parted = nullptr, joined = nullptr;
+    cudaEvent_t counted = nullptr;    // the cells' cost count is in page-locked memory
     cudaGraphExec_t loop_exec = nullptr;
     std::vector<const void *> loop_key;
     std::vector<Ev> graph_events;     // event pairs inside the graph (profile = 1)
@@ -245,6 +255,7 @@ struct asicp_ctx {
         if (cap_st) cudaStreamDestroy(cap_st);
         if (parted) cudaEventDestroy(parted);
         if (joined) cudaEventDestroy(joined);
+        if (counted) cudaEventDestroy(counted);
         if (side_st) cudaStreamDestroy(side_st);
     }
 };
@@ -619,6 +630,7 @@ void drop_minibatches(asicp_ctx *c)
 // Build the cells of the given clouds (at most kCellBatch of them, or as many as the scratch
 // holds, per launch).
 size_t cell_scratch(const CellSizes &s) { return 2 * sizeof(int) * (size_t)s.list_cap + s.rec_bytes; }
+using CellCost = unsigned long long[4];
 constexpr size_t kCellCtrBytes = sizeof(int) * kCellCounters * kCellBatch;
 
 size_t scratch_bytes(const std::vector<int> &sizes)
@@ -680,6 +692,7 @@ void cell_memory(asicp_ctx *c, DevMem &m, size_t bytes, const char *what)
 void ensure_cells(asicp_ctx *c, int v, int passes)
 {
     c->cells_on = false;
+    c->cells_share = 0.0;
     if (v != kFwdVariants - 1 || c->cells_oom || c->recording) return;
     std::vector<int> todo;
     int most = 0;
@@ -692,12 +705,13 @@ void ensure_cells(asicp_ctx *c, int v, int passes)
         points += c->objs[o].M;
     }
     if (most < kCellMinM || most > kCellMaxM) return;
-    if (!todo.empty()) {
-        c->cells_owed += passes * pairs / kCellRate;
-        if (c->cells_owed <= 100.0 + points / kCellRatePts) return;
+    if (todo.empty()) {
+        c->cells_on = !c->cells_slow;
+        return;
     }
+    c->cells_owed += passes * pairs / kCellRate * c->cells_gain;
+    if (c->cells_owed <= 100.0 + points / kCellRatePts) return;
     c->cells_on = true;
-    if (todo.empty()) return;
     std::vector<CellBuild> builds;
     bool moved = false;
     try {
@@ -753,6 +767,40 @@ void ensure_cells(asicp_ctx *c, int v, int passes)
     if (!c->cells_on) return;
     build_cells(c, builds);
     for (int o : todo) c->objs[o].cells_built = true;
+
+    // whether they are the faster way for these clouds: weigh_cells() reads the count
+    FwdArgs fa{};
+    fa.L = c->layout();
+    fa.theta = c->theta.as<float>();
+    fa.Ssort = c->Ssort.as<float4>();
+    unsigned long long *cost = c->cellwork.as<unsigned long long>();      // (the counters' place)
+    ck(cudaMemsetAsync(cost, 0, sizeof(CellCost), c->st), "matching cells");
+    double share = 0.0;
+    ck(launch_cells_cost(fa, cost, &share, c->st), "matching cells");
+    if (!c->pin.ensure(sizeof(CellCost))) return;      // (without page-locked memory the cells are taken as they are)
+    ck(cudaMemcpyAsync(c->pin.p, cost, sizeof(CellCost), cudaMemcpyDeviceToHost, c->st), "matching cells");
+    ck(cudaEventRecord(c->counted, c->st), "matching cells");
+    c->cells_share = share;
+}
+
+// Read the count that ensure_cells() has enqueued and keep the faster way.  Called after the other preparations of the
+// call, which run meanwhile.
+void weigh_cells(asicp_ctx *c)
+{
+    if (c->cells_share == 0.0) return;
+    const double share = c->cells_share;
+    c->cells_share = 0.0;
+    ck(cudaEventSynchronize(c->counted), "matching cells");
+    CellCost cost;
+    std::memcpy(cost, c->pin.p, sizeof(cost));
+    double pairs = 0.0, us = 0.0;
+    for (const ObjMeta &m : c->objmeta_h) pairs += (double)m.np * c->N * m.M;
+    for (int k = 0; k < 4; k += 2)
+        us = std::max({us, (double)cost[k] / share / kCellRounds, (double)cost[k + 1] * kCellLatency});
+    const double gain = 1.0 - us * kCellRate / pairs;
+    c->cells_slow = gain < 0.0;
+    c->cells_gain = std::max(gain, kCellGain);
+    c->cells_on = c->cells_on && !c->cells_slow;
 }
 
 // Whether the caller's own stream is being captured: the launches of this call run when its graph is replayed,
@@ -1121,6 +1169,7 @@ void autotune_impl(asicp_ctx *c, float *ms_out)
         fa.cand = c->tccand.as<int4>();
         fa.variant = v;
         ensure_cells(c, v, c->cfg.k_max + 1);
+        weigh_cells(c);
         fa.Ssort = c->Ssort.as<float4>();
         fa.cells = c->cells_on;
         ck(launch_fwd_match(fa, c->st), "autotune warm-up");
@@ -1260,6 +1309,7 @@ asicp_status asicp_create(const asicp_config *cfg, asicp_ctx **out)
         ck(cudaStreamCreateWithFlags(&c->side_st, cudaStreamNonBlocking), "side stream");
         ck(cudaEventCreateWithFlags(&c->parted, cudaEventDisableTiming), "side stream event");
         ck(cudaEventCreateWithFlags(&c->joined, cudaEventDisableTiming), "side stream event");
+        ck(cudaEventCreateWithFlags(&c->counted, cudaEventDisableTiming), "event");
         ck(init_collision_attributes(), "collision kernel attributes");
         ck(init_update_attributes(), "update kernel attributes");
         ck(init_cells_attributes(), "cell kernel attributes");
@@ -1458,6 +1508,7 @@ asicp_status asicp_step(asicp_ctx *ctx, int k)
         ensure_cells(ctx, ctx->fwd_variant, 1);
         ensure_pre_cells(ctx, 1);
         ensure_sorted(ctx);
+        weigh_cells(ctx);
         step_impl(ctx, k);
         ctx->run_done = false;
     });
@@ -1486,6 +1537,7 @@ asicp_status asicp_run(asicp_ctx *ctx, const float *theta0)
         ensure_cells(ctx, ctx->fwd_variant, ctx->cfg.k_max + 1);
         ensure_pre_cells(ctx, ctx->cfg.k_max + 1);
         ensure_sorted(ctx);
+        weigh_cells(ctx);
         run_loop_graph(ctx);
         ctx->k_next = ctx->cfg.k_max;
         ctx->stepped = true;

@@ -313,6 +313,8 @@ struct CellSizes {
 CellSizes cell_sizes(int M);
 cudaError_t launch_cells_build(const CellBuildBatch &batch, int n, cudaStream_t st);
 cudaError_t launch_cells_match(const FwdArgs &a, cudaStream_t st);
+constexpr int kCellSample = 4096;      // warps looked at by launch_cells_cost
+cudaError_t launch_cells_cost(const FwdArgs &a, unsigned long long *cost, double *share, cudaStream_t st);
 cudaError_t launch_sort_points(const float4 *S, int N, float4 *out, float4 *frame, cudaStream_t st);
 cudaError_t init_cells_attributes();
 

@@ -615,14 +615,17 @@ __global__ void __launch_bounds__(kMatchThreads) cells_match_kernel(const FwdArg
         const float qx = __shfl_sync(0xffffffffu, o.x, src), qy = __shfl_sync(0xffffffffu, o.y, src),
                     qz = __shfl_sync(0xffffffffu, o.z, src);
         const int base = __shfl_sync(0xffffffffu, nd.x, src), len = __shfl_sync(0xffffffffu, nd.y, src);
-        const int n = len == kWhole ? om.M : len;
         float wb = __int_as_float(0x7f800000);
         int wi = 0x7fffffff;
-        for (int e = lane; e < n; e += 32) {
-            const int r = len == kWhole ? e : __ldg(om.leaves + base + e);
-            const float4 p = __ldg(R + r);
-            const float d = dist2_f32(qx, qy, qz, p.x, p.y, p.z);
-            if (d < wb || (d == wb && r < wi)) { wb = d; wi = r; }
+        if (len == kWhole) {
+            warp_exact_all(R, om.M, qx, qy, qz, wb, wi);
+        } else {
+            for (int e = lane; e < len; e += 32) {       // (index order: a lane's ties keep the lower index)
+                const int r = __ldg(om.leaves + base + e);
+                const float4 p = __ldg(R + r);
+                const float d = dist2_f32(qx, qy, qz, p.x, p.y, p.z);
+                if (d < wb) { wb = d; wi = r; }
+            }
         }
         for (int off = 16; off > 0; off >>= 1) {
             const float ob = __shfl_xor_sync(0xffffffffu, wb, off);
@@ -640,6 +643,61 @@ __global__ void __launch_bounds__(kMatchThreads) cells_match_kernel(const FwdArg
         a.dbg_sp[q * 3 + 1] = o.y;
         a.dbg_sp[q * 3 + 2] = o.z;
     }
+}
+
+// What the matching through the cells costs, counted on a sample of its warps: for the present poses, and for poses
+// that much nearer to the object's centre (kCellPull), which is where a run takes them.  The unit is a round of 32 points
+// of the whole cloud that a warp compares together; kCellList for 32 points of a long list (gathered through indices),
+// kCellStep for each four points that the lanes compare from lists of their own, kCellBase for the look-ups.  Warp i of
+// n looks at one of the i-th n-th of all warps.  Measured on GB300 (1.6 M queries, M 8192; us per pass counted at
+// kCellRounds and timed): noisy objects 37 and 42; boxes without noise 49 to 67 and 51 to 70; every point four times 166
+// and 163; an ellipsoid without noise 1158 and 1300.
+constexpr int kCellBase = 30, kCellStep = 9, kCellList = 3;
+constexpr float kCellPull = 0.25f;
+
+__global__ void __launch_bounds__(128) cells_cost_kernel(const FwdArgs a, long long warps, int n, unsigned long long *cost)
+{
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31, N = a.L.N;
+    if (i >= n) return;
+    const long long lo = warps * i / n, room = warps * (i + 1) / n - lo;
+    const long long w = lo + (long long)((i * 2654435761u) >> 8) % room;
+    const int per = (N + 31) / 32, pk = (int)(w / per), k = (int)(w % per) * 32 + lane;
+    const int grp = a.L.part_grp[pk], obj = grp / a.L.P;
+    const float4 s = a.Ssort[(size_t)(grp - obj * a.L.P) * N + min(k, N - 1)];
+    const ObjMeta &om = a.L.obj[obj];
+    const float4 fr = a.L.frame[obj];
+    const float *th = a.theta + (size_t)pk * 8;
+    float Rm[9];
+    quat_rot_f32(th[3], th[4], th[5], th[6], Rm);
+    for (int near = 0; near < 2; ++near) {
+        const float f = near ? kCellPull : 1.f;
+        const float3 o = xform_f32(Rm, fr.x + f * (th[0] - fr.x), fr.y + f * (th[1] - fr.y), fr.z + f * (th[2] - fr.z), s.x, s.y,
+                                   s.z);
+        const int2 nd = find_cell(om.nodes, cell_half(fr.w, kObjectCells), __fsub_rn(o.x, fr.x), __fsub_rn(o.y, fr.y),
+                                  __fsub_rn(o.z, fr.z));
+        const int len = nd.y == kWhole ? om.M : nd.y;
+        const bool own = nd.y != kWhole && len <= kCellOwn;
+        const unsigned steps = __reduce_max_sync(0xffffffffu, own ? (unsigned)len / 4u : 0u);
+        const unsigned mine = own || k >= N ? 0u : (unsigned)(len + 31) / 32u;
+        const unsigned whole = __reduce_add_sync(0xffffffffu, nd.y == kWhole ? mine : 0u);
+        const unsigned lists = __reduce_add_sync(0xffffffffu, nd.y == kWhole ? 0u : mine);
+        if (lane == 0) {
+            const unsigned own_work = kCellBase + kCellStep * steps;
+            atomicAdd(cost + 2 * near, (unsigned long long)(own_work + whole + kCellList * lists));
+            atomicMax(cost + 2 * near + 1, (unsigned long long)(own_work + whole + lists));
+        }
+    }
+}
+
+// The sum over the sample goes to cost[0], the most rounds of a warp, of any kind, to cost[1], those of the poses pulled
+// in to cost[2] and cost[3] (cleared before); *share: how much of all warps the sample is.
+cudaError_t launch_cells_cost(const FwdArgs &a, unsigned long long *cost, double *share, cudaStream_t st)
+{
+    const long long warps = (long long)a.L.T * ((a.L.N + 31) / 32);
+    const int n = (int)(warps < kCellSample ? warps : kCellSample);
+    *share = (double)n / (double)warps;
+    cells_cost_kernel<<<(n + 3) / 4, 128, 0, st>>>(a, warps, n, cost);
+    return cudaGetLastError();
 }
 
 CellSizes cell_sizes(int M)
