@@ -115,6 +115,7 @@ struct ObjBufs {
     DevMem nodes, leaves;     // matching cells of R
     DevMem Csort, Cball;      // the collision cloud in spatial order
     int M = 0, Mpad = 0, Mc = 0;
+    float4 frame{};           // centre and radius of R, as on the device
     bool set = false, cells_built = false, sorted = false;
 };
 
@@ -172,6 +173,8 @@ struct asicp_ctx {
     double cells_owed = 0.0;          // microseconds of screening on the present objects so far
     bool pre_oom = false;             // no room for the gripper clouds' cells
     int fail_cells = -1;              // this many more allocations for cells succeed, the next fails (testing; < 0: off)
+    bool pre_on = false;              // the passes being launched match the colliding points through them
+    std::vector<float4> preframe_h;   // the gripper clouds' centres and radii, as on the device
     bool pre_built = false;           // the gripper clouds' cells are built (all preshapes together)
     double pre_owed = 0.0;            // microseconds of reverse matching without them so far
     bool recording = false;           // the caller's stream is being captured (see note_capture)
@@ -846,13 +849,34 @@ void ensure_sorted(asicp_ctx *c)
 constexpr int kPreMinN = 512;
 constexpr double kPreRate = 5.7e6;
 
+// Whether the cells hold for colliding points of every object: collide_cells_kernel compares the whole gripper cloud for
+// a point whose position is less exact than they allow, which takes five times as long as collide_nn_kernel (4.3e5
+// points, N 2048, an object 8 m away or more, gripper radius 7 cm: 1106 us against 217).  Its bound, for a pose at
+// the farthest object's centre and any point of the distance field's grid.
+bool pre_cells_hold(const asicp_ctx *c)
+{
+    auto sum = [](float x, float y, float z) { return std::fabs(x) + std::fabs(y) + std::fabs(z); };
+    float far = 0.f;
+    for (const ObjBufs &o : c->objs) far = std::max(far, sum(o.frame.x, o.frame.y, o.frame.z));
+    for (int p = 0; p < c->cfg.P; ++p) {
+        const float4 &f = c->preframe_h[p];
+        const SdfMeta &m = c->meta[p];
+        auto end = [&](float o, int n) { return std::max(std::fabs(o), std::fabs(o + m.voxel * (float)(n - 1))); };
+        const float reach = sum(f.x, f.y, f.z) + f.w, x = end(m.ox, m.nx) + end(m.oy, m.ny) + end(m.oz, m.nz);
+        if (!(1.2e-6f * (x + reach) + 4e-7f * far <= 0.4f * kGripperTol * f.w)) return false;
+    }
+    return true;
+}
+
 void ensure_pre_cells(asicp_ctx *c, int passes)
 {
-    if (c->pre_oom || c->N < kPreMinN || c->recording) return;
+    c->pre_on = false;
+    if (c->pre_oom || c->N < kPreMinN || c->recording || !pre_cells_hold(c)) return;
     const int P = c->cfg.P;
     const size_t list = sizeof(int) * (size_t)std::max<long long>(1, c->colidx_total);
     if (c->pre_built) {
-        if (list <= c->colsrt.bytes) return;
+        c->pre_on = list <= c->colsrt.bytes;
+        if (c->pre_on) return;
     } else {
         double tests = 0.0;
         for (const ObjMeta &m : c->objmeta_h) tests += (double)m.np * m.Mc;
@@ -879,8 +903,7 @@ void ensure_pre_cells(asicp_ctx *c, int passes)
                 b.M = c->N;
                 b.log_factor = kGripperCells;
                 b.tol = kGripperTol;
-                b.near_only = 1;
-                builds.push_back(b);
+                    builds.push_back(b);
             }
         }
     } catch (const Err &e) {
@@ -893,9 +916,8 @@ void ensure_pre_cells(asicp_ctx *c, int passes)
         c->cellwork.release();
         return;
     }
-    if (c->pre_built) return;
-    build_cells(c, builds);
-    c->pre_built = true;
+    if (!c->pre_built) build_cells(c, builds);
+    c->pre_on = c->pre_built = true;
 }
 
 // The collision test and the reverse matching of a pass read the poses only, as the forward matching
@@ -985,7 +1007,7 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
     ca.col_items = c->colitems.as<int>();
     ca.col_list = c->collist.as<int>();
     for (const ObjMeta &m : c->objmeta_h) ca.most_points = std::max(ca.most_points, m.Mc);
-    ca.cells = c->pre_built && !c->recording;
+    ca.cells = c->pre_on;
     if (ca.cells) {
         ca.colsrt = c->colsrt.as<int>();
         const CellSizes s = cell_sizes(c->N);
@@ -1071,7 +1093,7 @@ std::vector<const void *> loop_key(const asicp_ctx *c)
             reinterpret_cast<const void *>((size_t)c->N), reinterpret_cast<const void *>((size_t)c->fwd_variant),
             reinterpret_cast<const void *>((size_t)c->expire_test), c->Ssort.p,
             reinterpret_cast<const void *>((size_t)c->cells_on), c->prenodes.p, c->preleaves.p, c->preframe.p,
-            reinterpret_cast<const void *>((size_t)c->pre_built), reinterpret_cast<const void *>((size_t)c->colmap_total)};
+            reinterpret_cast<const void *>((size_t)c->pre_on), reinterpret_cast<const void *>((size_t)c->colmap_total)};
 }
 
 // Replay the captured loop on the caller's stream, capturing it first when the
@@ -1231,6 +1253,7 @@ void set_object_impl(asicp_ctx *ctx, int o, const float *R_xyz, int M, const flo
     b.Rt.ensure(tc_ref_bytes(Mpad), "tensor-core object tiles");
     ck(launch_tc_ref_prep(b.R.as<float4>(), M, Mpad, ctx->frame.as<float4>() + o, b.Rt.p, ctx->st),
        "tensor-core ref prep");
+    copy_out(ctx, &b.frame, ctx->frame.as<float4>() + o, sizeof(float4));
     finish(ctx, "set_object");
     b.M = M;
     b.Mpad = Mpad;
@@ -1301,6 +1324,7 @@ asicp_status asicp_create(const asicp_config *cfg, asicp_ctx **out)
     c->grids.resize(cfg->P);
     c->cells.resize(cfg->P);
     c->clear.resize(cfg->P);
+    c->preframe_h.assign(cfg->P, float4{});
     c->objs.resize(c->nobj);
     c->Kg.assign((size_t)c->nobj * cfg->P, cfg->K);
     asicp_status s = guarded(c, [&] {
@@ -1448,6 +1472,7 @@ asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_
         ctx->clear[preshape].ensure(nc, "sdf clearances");
         ck(launch_sdf_clear(ctx->cells[preshape].as<float4>(), nx, ny, nz, ctx->clear[preshape].as<unsigned char>(),
                             ctx->stage.as<unsigned char>(), ctx->st), "sdf clearances");
+        copy_out(ctx, &ctx->preframe_h[preshape], ctx->preframe.as<float4>() + preshape, sizeof(float4));
         finish(ctx, "set_gripper_sdf");
         SdfMeta m{};
         m.grid = ctx->grids[preshape].as<float>();

@@ -297,10 +297,10 @@ struct CellBuild {
     int M, leaf_cap, list_cap, cell_cap, node_cap;
     int log_factor;           // near cells reach 2^log_factor times the power of two above the radius
     float tol;                // positions looked up may be off by 0.4 tol times the radius
-    int near_only;            // no cells beyond the near ones
 };
-// Cells of objects, and of gripper clouds in the gripper frame (colliding points lie in the
-// gripper's body, not far from its surface; see collide_cells_kernel for the tolerance).
+// Cells of objects, and of gripper clouds in the gripper frame (see collide_cells_kernel for the tolerance).  Colliding
+// points lie in the gripper's body, which may reach far beyond a cloud that covers its fingertips only: with the near
+// cells alone a cloud a fifth of the body's size took 1033 us per pass against 217 without cells.
 constexpr int kObjectCells = 2, kGripperCells = 1;     // (log_factor)
 constexpr float kGripperTol = 1.25e-4f;
 struct CellBuildBatch {

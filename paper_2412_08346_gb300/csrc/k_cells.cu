@@ -200,8 +200,8 @@ __global__ void __launch_bounds__(256) cells_start_kernel(const CellBuildBatch b
         r.c.w = 0.25f * H;
         r.c.x = (2 * x + 1) * r.c.w - H; r.c.y = (2 * y + 1) * r.c.w - H; r.c.z = (2 * z + 1) * r.c.w - H;
         r.at = kFarBase + cell;
-        // inside (the near grid or a smaller shell covers it), or no far cells wanted
-        if ((x % 3 != 0 && y % 3 != 0 && z % 3 != 0) || b.near_only) {
+        // inside: the near grid or a smaller shell covers it
+        if (x % 3 != 0 && y % 3 != 0 && z % 3 != 0) {
             if (threadIdx.x == 0) b.nodes[r.at] = make_int2(0, kWhole);
             return;
         }
