@@ -1457,8 +1457,10 @@ asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_
         ck(launch_pack_points(ctx->stage.as<float>(), N, Sp, ctx->errw.as<int>(), ctx->st), "pack S");
         ctx->Ssort.ensure(sizeof(float4) * (size_t)ctx->cfg.P * N, "gripper clouds, sorted");
         ctx->preframe.ensure(sizeof(float4) * ctx->cfg.P, "gripper frames");
+        // (one CTA each, the sort and the preshape sums: beside each other)
+        Branch side(ctx, true);
         ck(launch_sort_points(Sp, N, ctx->Ssort.as<float4>() + (size_t)preshape * N, ctx->preframe.as<float4>() + preshape,
-                              ctx->st), "sort S");
+                              side.stream()), "sort S");
         ctx->pre_built = false;
         ctx->pre_owed = 0.0;
         ck(launch_preshape_consts(Sp, N, ctx->pconst.as<double>() + 12 * preshape, ctx->st), "preshape sums");
@@ -1467,11 +1469,13 @@ asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_
         ck(cudaMemcpyAsync(ctx->grids[preshape].p, sdf, sizeof(float) * nv, cudaMemcpyDefault, ctx->st), "copy sdf");
         ck(launch_check_finite(ctx->grids[preshape].as<float>(), (long long)nv, ctx->errw.as<int>(), ctx->st), "check sdf");
         ctx->cells[preshape].ensure(sdf_cells_bytes(nx, ny, nz), "corner-packed sdf grid");
-        ck(launch_sdf_pack_cells(ctx->grids[preshape].as<float>(), nx, ny, nz, ctx->cells[preshape].as<float4>(), ctx->st),
-           "pack sdf cells");
+        // (S has been packed: the staging buffer is free again)
+        ck(launch_sdf_pack_cells(ctx->grids[preshape].as<float>(), nx, ny, nz, ctx->cells[preshape].as<float4>(),
+                                 ctx->stage.as<unsigned char>(), ctx->st), "pack sdf cells");
         ctx->clear[preshape].ensure(nc, "sdf clearances");
-        ck(launch_sdf_clear(ctx->cells[preshape].as<float4>(), nx, ny, nz, ctx->clear[preshape].as<unsigned char>(),
-                            ctx->stage.as<unsigned char>(), ctx->st), "sdf clearances");
+        ck(launch_sdf_clear(nx, ny, nz, ctx->stage.as<unsigned char>(), ctx->clear[preshape].as<unsigned char>(), ctx->st),
+           "sdf clearances");
+        side.join();
         copy_out(ctx, &ctx->preframe_h[preshape], ctx->preframe.as<float4>() + preshape, sizeof(float4));
         finish(ctx, "set_gripper_sdf");
         SdfMeta m{};

@@ -393,9 +393,9 @@ cudaError_t launch_preshape_consts(const float4 *S, int N, double *out12, cudaSt
 cudaError_t launch_fibonacci(const Layout &L, float radius, int mode, float *theta, cudaStream_t st);
 cudaError_t launch_store_meta(ObjMeta *dst, const ObjMeta &v, cudaStream_t st);
 cudaError_t launch_set_theta(const float *theta7, int T, float *theta8, int *err, cudaStream_t st);
-cudaError_t launch_sdf_clear(const float4 *cells, int nx, int ny, int nz, unsigned char *clear, unsigned char *tmp,
-                             cudaStream_t st);
-cudaError_t launch_sdf_pack_cells(const float *grid, int nx, int ny, int nz, float4 *cells, cudaStream_t st);
+cudaError_t launch_sdf_clear(int nx, int ny, int nz, unsigned char *away, unsigned char *clear, cudaStream_t st);
+cudaError_t launch_sdf_pack_cells(const float *grid, int nx, int ny, int nz, float4 *cells, unsigned char *away,
+                                  cudaStream_t st);
 size_t sdf_cells_bytes(int nx, int ny, int nz);
 cudaError_t launch_select(const Layout &L, const double *cost, const int *ncol, int *order, cudaStream_t st);
 cudaError_t launch_uniform_groups(int *part_grp, int *grp_off, int P, int K, cudaStream_t st);
