@@ -11,6 +11,7 @@
 #include "asicp_internal.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cmath>
 #include <cstdio>
@@ -131,9 +132,10 @@ constexpr double kCellRate = 1.65e7, kCellRatePts = 50.0;
 // Clouds whose lists do not shrink (points on a common sphere or plane, many copies of a point) are matched faster by
 // the screening.  So the work of one pass is counted on a sample of the queries when cells have been built (see
 // cells_cost_kernel): a pass takes 1 us per kCellRounds rounds, or, where few warps have long lists, kCellLatency us
-// per round of the longest one.  What it saves of the screening, but at least kCellGain of it, is what the next
-// clouds' build is weighed against.
-constexpr double kCellRounds = 7.5e4, kCellLatency = 0.15, kCellGain = 1.0 / 32.0;
+// per round of the longest one.  Screening and exact choice take kScreenLeast us (two kernels) and at least
+// kScreenPoint us per object point (one CTA's chain over the tiles: 6144 queries on 200000 points 363 us).
+constexpr double kCellRounds = 7.5e4, kCellLatency = 0.15, kScreenLeast = 15.0, kScreenPoint = 1.8e-3;
+constexpr double kCellDoubt = 1.0 / 32.0;            // after such clouds the next ones' build is held against this much
 constexpr size_t kCellScratch = (size_t)256 << 20;   // scratch of one build launch (at least one object)
 
 enum { kTimeMatch = 0, kTimeCollide = 1, kTimeCollideNN = 2, kTimeFinalize = 3, kTimeStein = 4, kTimeExact = 5,
@@ -168,8 +170,9 @@ struct asicp_ctx {
     bool cells_oom = false;           // no room for matching cells: the screening is used
     bool cells_on = false;            // the passes being launched match through the cells
     bool cells_slow = false;          // the present objects' cells are built, but the screening is the faster
-    double cells_gain = 1.0;          // share of a screening pass that the cells save, as last seen
+    double cells_worth = 1.0;         // share of the screening's time that the next clouds' build is weighed against
     double cells_share = 0.0;         // sample of the cost count that has been enqueued (0: none)
+    unsigned weight_seq = 0;          // number of that count
     double cells_owed = 0.0;          // microseconds of screening on the present objects so far
     bool pre_oom = false;             // no room for the gripper clouds' cells
     int fail_cells = -1;              // this many more allocations for cells succeed, the next fails (testing; < 0: off)
@@ -202,6 +205,7 @@ struct asicp_ctx {
     struct Out { void *dst; const void *src; size_t bytes; };
     std::vector<Out> outs;
     PinMem pin, pin_in;
+    PinMem weights;                   // the cells' cost count, written by the device
     bool pin_busy = false;
     size_t pin_used = 0;              // bytes of pin_in taken by copies in flight
     DevMem outp, outg;                // phi and gradient as they are returned
@@ -213,7 +217,6 @@ struct asicp_ctx {
     // the collision test's branch of a pass and the events that part and join the two
     cudaStream_t side_st = nullptr;
     cudaEvent_t parted = nullptr, joined = nullptr;
-    cudaEvent_t counted = nullptr;    // the cells' cost count is in page-locked memory
     cudaGraphExec_t loop_exec = nullptr;
     std::vector<const void *> loop_key;
     std::vector<Ev> graph_events;     // event pairs inside the graph (profile = 1)
@@ -258,7 +261,6 @@ struct asicp_ctx {
         if (cap_st) cudaStreamDestroy(cap_st);
         if (parted) cudaEventDestroy(parted);
         if (joined) cudaEventDestroy(joined);
-        if (counted) cudaEventDestroy(counted);
         if (side_st) cudaStreamDestroy(side_st);
     }
 };
@@ -633,7 +635,6 @@ void drop_minibatches(asicp_ctx *c)
 // Build the cells of the given clouds (at most kCellBatch of them, or as many as the scratch
 // holds, per launch).
 size_t cell_scratch(const CellSizes &s) { return 2 * sizeof(int) * (size_t)s.list_cap + s.rec_bytes; }
-using CellCost = unsigned long long[4];
 constexpr size_t kCellCtrBytes = sizeof(int) * kCellCounters * kCellBatch;
 
 size_t scratch_bytes(const std::vector<int> &sizes)
@@ -712,7 +713,7 @@ void ensure_cells(asicp_ctx *c, int v, int passes)
         c->cells_on = !c->cells_slow;
         return;
     }
-    c->cells_owed += passes * pairs / kCellRate * c->cells_gain;
+    c->cells_owed += passes * pairs / kCellRate * c->cells_worth;
     if (c->cells_owed <= 100.0 + points / kCellRatePts) return;
     c->cells_on = true;
     std::vector<CellBuild> builds;
@@ -776,14 +777,13 @@ void ensure_cells(asicp_ctx *c, int v, int passes)
     fa.L = c->layout();
     fa.theta = c->theta.as<float>();
     fa.Ssort = c->Ssort.as<float4>();
-    unsigned long long *cost = c->cellwork.as<unsigned long long>();      // (the counters' place)
-    ck(cudaMemsetAsync(cost, 0, sizeof(CellCost), c->st), "matching cells");
-    double share = 0.0;
-    ck(launch_cells_cost(fa, cost, &share, c->st), "matching cells");
-    if (!c->pin.ensure(sizeof(CellCost))) return;      // (without page-locked memory the cells are taken as they are)
-    ck(cudaMemcpyAsync(c->pin.p, cost, sizeof(CellCost), cudaMemcpyDeviceToHost, c->st), "matching cells");
-    ck(cudaEventRecord(c->counted, c->st), "matching cells");
-    c->cells_share = share;
+    if (!c->weights.p) {
+        if (!c->weights.ensure(sizeof(CellCost))) return;      // (the cells are taken as they are)
+        std::memset(c->weights.p, 0, sizeof(CellCost));
+    }
+    ck(launch_cells_cost(fa, reinterpret_cast<CellCost *>(c->cellwork.as<int>() + kCellCounters / 2),
+                         reinterpret_cast<CellCost *>(c->weights.p), ++c->weight_seq, &c->cells_share, c->st),
+       "matching cells");
 }
 
 // Read the count that ensure_cells() has enqueued and keep the faster way.  Called after the other preparations of the
@@ -793,16 +793,24 @@ void weigh_cells(asicp_ctx *c)
     if (c->cells_share == 0.0) return;
     const double share = c->cells_share;
     c->cells_share = 0.0;
-    ck(cudaEventSynchronize(c->counted), "matching cells");
-    CellCost cost;
-    std::memcpy(cost, c->pin.p, sizeof(cost));
-    double pairs = 0.0, us = 0.0;
-    for (const ObjMeta &m : c->objmeta_h) pairs += (double)m.np * c->N * m.M;
-    for (int k = 0; k < 4; k += 2)
-        us = std::max({us, (double)cost[k] / share / kCellRounds, (double)cost[k + 1] * kCellLatency});
-    const double gain = 1.0 - us * kCellRate / pairs;
-    c->cells_slow = gain < 0.0;
-    c->cells_gain = std::max(gain, kCellGain);
+    const volatile CellCost *v = reinterpret_cast<const CellCost *>(c->weights.p);
+    for (int n = 1; v->seq != c->weight_seq; ++n)
+        if (n % 1024 == 0) {               // (an error would leave it unwritten)
+            const cudaError_t e = cudaStreamQuery(c->st);
+            if (e == cudaErrorNotReady) continue;
+            ck(e, "matching cells");
+            if (v->seq != c->weight_seq) fail(ASICP_ERR_CUDA, "matching cells: no count");
+        }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    double pairs = 0.0, most = 0.0, us = 0.0;
+    for (const ObjMeta &m : c->objmeta_h) {
+        pairs += (double)m.np * c->N * m.M;
+        most = std::max(most, (double)m.M);
+    }
+    for (int k = 0; k < 2; ++k)
+        us = std::max({us, (double)v->sum[k] / share / kCellRounds, (double)v->most[k] * kCellLatency});
+    c->cells_slow = us > kScreenLeast + std::max(pairs / kCellRate, most * kScreenPoint);
+    c->cells_worth = c->cells_slow ? kCellDoubt : 1.0;
     c->cells_on = c->cells_on && !c->cells_slow;
 }
 
@@ -812,7 +820,8 @@ void weigh_cells(asicp_ctx *c)
 void note_capture(asicp_ctx *c)
 {
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->st, &s) != cudaSuccess) {
+    // (the default stream cannot be captured)
+    if (c->st != nullptr && c->st != cudaStreamLegacy && cudaStreamIsCapturing(c->st, &s) != cudaSuccess) {
         cudaGetLastError();
         s = cudaStreamCaptureStatusNone;
     }
@@ -1008,8 +1017,8 @@ void iterate(asicp_ctx *c, int mode, float gamma, int k)
     ca.col_list = c->collist.as<int>();
     for (const ObjMeta &m : c->objmeta_h) ca.most_points = std::max(ca.most_points, m.Mc);
     ca.cells = c->pre_on;
+    ca.colsrt = ca.cells ? c->colsrt.as<int>() : ca.colnn;
     if (ca.cells) {
-        ca.colsrt = c->colsrt.as<int>();
         const CellSizes s = cell_sizes(c->N);
         ca.pre_nodes = c->prenodes.as<int2>();
         ca.pre_leaves = c->preleaves.as<int>();
@@ -1333,7 +1342,6 @@ asicp_status asicp_create(const asicp_config *cfg, asicp_ctx **out)
         ck(cudaStreamCreateWithFlags(&c->side_st, cudaStreamNonBlocking), "side stream");
         ck(cudaEventCreateWithFlags(&c->parted, cudaEventDisableTiming), "side stream event");
         ck(cudaEventCreateWithFlags(&c->joined, cudaEventDisableTiming), "side stream event");
-        ck(cudaEventCreateWithFlags(&c->counted, cudaEventDisableTiming), "event");
         ck(init_collision_attributes(), "collision kernel attributes");
         ck(init_update_attributes(), "update kernel attributes");
         ck(init_cells_attributes(), "cell kernel attributes");

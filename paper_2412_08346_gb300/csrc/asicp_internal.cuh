@@ -313,8 +313,12 @@ struct CellSizes {
 CellSizes cell_sizes(int M);
 cudaError_t launch_cells_build(const CellBuildBatch &batch, int n, cudaStream_t st);
 cudaError_t launch_cells_match(const FwdArgs &a, cudaStream_t st);
-constexpr int kCellSample = 4096;      // warps looked at by launch_cells_cost
-cudaError_t launch_cells_cost(const FwdArgs &a, unsigned long long *cost, double *share, cudaStream_t st);
+constexpr int kCellSample = 1024;      // warps looked at by launch_cells_cost
+struct CellCost {
+    unsigned long long sum[2];
+    unsigned most[2], seq, pad;
+};
+cudaError_t launch_cells_cost(const FwdArgs &a, CellCost *cost, CellCost *host, unsigned seq, double *share, cudaStream_t st);
 cudaError_t launch_sort_points(const float4 *S, int N, float4 *out, float4 *frame, cudaStream_t st);
 cudaError_t init_cells_attributes();
 
@@ -341,7 +345,8 @@ struct CollideArgs {
     const float4 *S;          // [P][N]
     int *ncol;                // [T]
     int *colidx;              // colliding points, ascending (see ObjMeta::colidx_base)
-    int *colsrt;              // the same points as positions in Csort, in no particular order (cells only)
+    int *colsrt;              // the same points as positions in Csort, in no particular order (without cells colnn, which
+                              // the reverse matching overwrites)
     int *colnn;               // like colidx: nearest gripper point of each
     int2 *colmap;             // bit map of the colliding points: words (bits, number of earlier bits),
                               // only those with bits written (see ObjMeta::colmap_base)

@@ -648,17 +648,21 @@ __global__ void __launch_bounds__(kMatchThreads) cells_match_kernel(const FwdArg
 // What the matching through the cells costs, counted on a sample of its warps: for the present poses, and for poses
 // that much nearer to the object's centre (kCellPull), which is where a run takes them.  The unit is a round of 32 points
 // of the whole cloud that a warp compares together; kCellList for 32 points of a long list (gathered through indices),
-// kCellStep for each four points that the lanes compare from lists of their own, kCellBase for the look-ups.  Warp i of
-// n looks at one of the i-th n-th of all warps.  Measured on GB300 (1.6 M queries, M 8192; us per pass counted at
-// kCellRounds and timed): noisy objects 37 and 42; boxes without noise 49 to 67 and 51 to 70; every point four times 166
-// and 163; an ellipsoid without noise 1158 and 1300.
-constexpr int kCellBase = 30, kCellStep = 9, kCellList = 3;
+// kCellStep for each four points that the lanes compare from lists of their own (kCellWait where one warp's latency
+// counts), kCellBase for the look-ups.  Warp i of n looks at one of the i-th n-th of all warps.  Measured on GB300 (1.6 M
+// queries, M 8192; us per pass counted at kCellRounds and timed): noisy objects 37 and 42; boxes without noise 49 to 67
+// and 51 to 70; every point four times 166 and 163; an ellipsoid without noise 1158 and 1300.
+constexpr int kCellBase = 30, kCellStep = 9, kCellList = 3, kCellWait = 3;
 constexpr float kCellPull = 0.25f;
 
-__global__ void __launch_bounds__(128) cells_cost_kernel(const FwdArgs a, long long warps, int n, unsigned long long *cost)
+constexpr int kCostThreads = 256;
+
+__global__ void __launch_bounds__(kCostThreads) cells_cost_kernel(const FwdArgs a, long long warps, int n, CellCost *cost,
+                                                                  CellCost *host, unsigned seq)
 {
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31, N = a.L.N;
-    if (i >= n) return;
+    __shared__ unsigned s_sum[2][kCostThreads / 32], s_most[2][kCostThreads / 32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, N = a.L.N;
+    const int at = blockIdx.x * (kCostThreads / 32) + warp, i = min(at, n - 1);
     const long long lo = warps * i / n, room = warps * (i + 1) / n - lo;
     const long long w = lo + (long long)((i * 2654435761u) >> 8) % room;
     const int per = (N + 31) / 32, pk = (int)(w / per), k = (int)(w % per) * 32 + lane;
@@ -682,21 +686,46 @@ __global__ void __launch_bounds__(128) cells_cost_kernel(const FwdArgs a, long l
         const unsigned whole = __reduce_add_sync(0xffffffffu, nd.y == kWhole ? mine : 0u);
         const unsigned lists = __reduce_add_sync(0xffffffffu, nd.y == kWhole ? 0u : mine);
         if (lane == 0) {
-            const unsigned own_work = kCellBase + kCellStep * steps;
-            atomicAdd(cost + 2 * near, (unsigned long long)(own_work + whole + kCellList * lists));
-            atomicMax(cost + 2 * near + 1, (unsigned long long)(own_work + whole + lists));
+            s_sum[near][warp] = at == i ? kCellBase + kCellStep * steps + whole + kCellList * lists : 0u;
+            s_most[near][warp] = kCellBase + kCellWait * steps + whole + lists;
         }
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int k = 0; k < 2; ++k) {
+        unsigned long long sum = 0;
+        unsigned most = 0u;
+        for (int w = 0; w < kCostThreads / 32; ++w) {
+            sum += s_sum[k][w];
+            most = max(most, s_most[k][w]);
+        }
+        atomicAdd(&cost->sum[k], sum);
+        atomicMax(&cost->most[k], most);
+    }
+    // the last CTA hands the counts over
+    __threadfence();
+    if (atomicAdd(&cost->seq, 1u) == gridDim.x - 1) {
+        __threadfence();
+        volatile CellCost *h = host;
+        for (int k = 0; k < 2; ++k) {
+            h->sum[k] = atomicAdd(&cost->sum[k], 0ull);
+            h->most[k] = atomicAdd(&cost->most[k], 0u);
+        }
+        __threadfence_system();
+        h->seq = seq;
     }
 }
 
-// The sum over the sample goes to cost[0], the most rounds of a warp, of any kind, to cost[1], those of the poses pulled
-// in to cost[2] and cost[3] (cleared before); *share: how much of all warps the sample is.
-cudaError_t launch_cells_cost(const FwdArgs &a, unsigned long long *cost, double *share, cudaStream_t st)
+// The sum over the sample and the most rounds of a warp, of any kind, for the present poses and those pulled in, go to *cost
+// (cleared before) and from there to *host, page-locked memory, whose seq is written last; *share: how much of all warps
+// the sample is.
+cudaError_t launch_cells_cost(const FwdArgs &a, CellCost *cost, CellCost *host, unsigned seq, double *share, cudaStream_t st)
 {
     const long long warps = (long long)a.L.T * ((a.L.N + 31) / 32);
     const int n = (int)(warps < kCellSample ? warps : kCellSample);
     *share = (double)n / (double)warps;
-    cells_cost_kernel<<<(n + 3) / 4, 128, 0, st>>>(a, warps, n, cost);
+    constexpr int kWarps = kCostThreads / 32;
+    cells_cost_kernel<<<(n + kWarps - 1) / kWarps, kCostThreads, 0, st>>>(a, warps, n, cost, host, seq);
     return cudaGetLastError();
 }
 

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kTestThreads, 1280 / kTestThreads) collide_ker
         lz = __fmaf_rn(Rm[2], dx, __fmaf_rn(Rm[5], dy, __fmul_rn(Rm[8], dz)));
     };
     const long long first = om.colidx_base + (long long)(pk - om.pfirst) * Mc;
-    int *colidx = a.colidx + first, *colsrt = a.cells ? a.colsrt + first : nullptr;
+    int *colidx = a.colidx + first, *colsrt = a.colsrt + first;
     int2 *colmap = a.colmap + om.colmap_base + (long long)(pk - om.pfirst) * ((Mc + 31) / 32);
     int count = 0;
     if (threadIdx.x == 0) s_hits = 0;
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kTestThreads, 1280 / kTestThreads) collide_ker
                 if (hit) {
                     const int own = __float_as_int(c[u].w);
                     atomicOr(&s_bits[own >> 5], 1u << (own & 31));
-                    if (colsrt) colsrt[base + __popc(bal & ((1u << lane) - 1u))] = seg + at[u];
+                    colsrt[base + __popc(bal & ((1u << lane) - 1u))] = seg + at[u];
                 }
             }
         }
