@@ -1465,13 +1465,10 @@ asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_
         ck(launch_pack_points(ctx->stage.as<float>(), N, Sp, ctx->errw.as<int>(), ctx->st), "pack S");
         ctx->Ssort.ensure(sizeof(float4) * (size_t)ctx->cfg.P * N, "gripper clouds, sorted");
         ctx->preframe.ensure(sizeof(float4) * ctx->cfg.P, "gripper frames");
-        // (one CTA each, the sort and the preshape sums: beside each other)
-        Branch side(ctx, true);
-        ck(launch_sort_points(Sp, N, ctx->Ssort.as<float4>() + (size_t)preshape * N, ctx->preframe.as<float4>() + preshape,
-                              side.stream()), "sort S");
+        ck(launch_gripper_cloud(Sp, N, ctx->Ssort.as<float4>() + (size_t)preshape * N, ctx->preframe.as<float4>() + preshape,
+                                ctx->pconst.as<double>() + 12 * preshape, ctx->st), "gripper cloud");
         ctx->pre_built = false;
         ctx->pre_owed = 0.0;
-        ck(launch_preshape_consts(Sp, N, ctx->pconst.as<double>() + 12 * preshape, ctx->st), "preshape sums");
         const size_t nv = (size_t)nx * ny * nz;
         ctx->grids[preshape].ensure(sizeof(float) * nv, "sdf grid");
         ck(cudaMemcpyAsync(ctx->grids[preshape].p, sdf, sizeof(float) * nv, cudaMemcpyDefault, ctx->st), "copy sdf");
@@ -1483,7 +1480,6 @@ asicp_status asicp_set_gripper_sdf(asicp_ctx *ctx, int preshape, const float *S_
         ctx->clear[preshape].ensure(nc, "sdf clearances");
         ck(launch_sdf_clear(nx, ny, nz, ctx->stage.as<unsigned char>(), ctx->clear[preshape].as<unsigned char>(), ctx->st),
            "sdf clearances");
-        side.join();
         copy_out(ctx, &ctx->preframe_h[preshape], ctx->preframe.as<float4>() + preshape, sizeof(float4));
         finish(ctx, "set_gripper_sdf");
         SdfMeta m{};

@@ -319,7 +319,7 @@ struct CellCost {
     unsigned most[2], seq, pad;
 };
 cudaError_t launch_cells_cost(const FwdArgs &a, CellCost *cost, CellCost *host, unsigned seq, double *share, cudaStream_t st);
-cudaError_t launch_sort_points(const float4 *S, int N, float4 *out, float4 *frame, cudaStream_t st);
+cudaError_t launch_gripper_cloud(const float4 *S, int N, float4 *out, float4 *frame, double *out12, cudaStream_t st);
 cudaError_t init_cells_attributes();
 
 constexpr int kColChunk = 64;          // colliding points per partial sum, and per work item of collide_nn_kernel
@@ -394,7 +394,6 @@ cudaError_t launch_stein(const UpdateArgs &a, cudaStream_t st);      // SVGD ste
 
 cudaError_t launch_pack_points(const float *xyz, int n, float4 *out, int *err, cudaStream_t st);
 cudaError_t launch_check_finite(const float *v, long long n, int *err, cudaStream_t st);
-cudaError_t launch_preshape_consts(const float4 *S, int N, double *out12, cudaStream_t st);
 cudaError_t launch_fibonacci(const Layout &L, float radius, int mode, float *theta, cudaStream_t st);
 cudaError_t launch_store_meta(ObjMeta *dst, const ObjMeta &v, cudaStream_t st);
 cudaError_t launch_set_theta(const float *theta7, int T, float *theta8, int *err, cudaStream_t st);

@@ -755,13 +755,43 @@ cudaError_t launch_cells_match(const FwdArgs &a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// Spatial order of a gripper cloud (one CTA): a bitonic sort of (Morton code, index) keys,
-// then the points in that order with their own index in w.  *frame: the centre of the bounding
-// box and the largest distance from it, rounded up.
-__global__ void __launch_bounds__(1024) sort_points_kernel(const float4 *S, int N, int Npow, float4 *out, float4 *frame)
+// sum s and sum s s^T (upper triangle) of a gripper cloud in float64, for one CTA: fixed thread striding and tree.
+__device__ __forceinline__ void preshape_sums(const float4 *S, int N, double *out12)
+{
+    __shared__ double red[32][9];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double acc[9] = {};
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+        const float4 s = S[i];
+        const double x = s.x, y = s.y, z = s.z;
+        acc[0] += x; acc[1] += y; acc[2] += z;
+        acc[3] = fma(x, x, acc[3]); acc[4] = fma(x, y, acc[4]); acc[5] = fma(x, z, acc[5]);
+        acc[6] = fma(y, y, acc[6]); acc[7] = fma(y, z, acc[7]); acc[8] = fma(z, z, acc[8]);
+    }
+    warp_sum_f64(acc);
+    if (lane == 0)
+        for (int c = 0; c < 9; ++c) red[warp][c] = acc[c];
+    __syncthreads();
+    if (threadIdx.x < 12) {
+        double s = 0.0;
+        if (threadIdx.x < 9)
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w][threadIdx.x];
+        out12[threadIdx.x] = s;
+    }
+}
+
+// Preparation of a gripper cloud, two CTAs of 25 us each side by side.  CTA 1: its sums.  CTA 0: its spatial order, a
+// bitonic sort of (Morton code, index) keys, then the points in that order with their own index in w.  *frame: the centre
+// of the bounding box and the largest distance from it, rounded up.
+__global__ void __launch_bounds__(1024) gripper_cloud_kernel(const float4 *S, int N, int Npow, float4 *out, float4 *frame,
+                                                             double *out12)
 {
     extern __shared__ unsigned long long s_key[];
     __shared__ float s_lo[3][32], s_hi[3][32];
+    if (blockIdx.x == 1) {
+        preshape_sums(S, N, out12);
+        return;
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float lo[3], hi[3];
     for (int k = 0; k < 3; ++k) { lo[k] = __int_as_float(0x7f800000); hi[k] = -lo[k]; }
@@ -833,16 +863,16 @@ __global__ void __launch_bounds__(1024) sort_points_kernel(const float4 *S, int 
 
 cudaError_t init_cells_attributes()
 {
-    return cudaFuncSetAttribute(sort_points_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(gripper_cloud_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 8192 * (int)sizeof(unsigned long long));
 }
 
-cudaError_t launch_sort_points(const float4 *S, int N, float4 *out, float4 *frame, cudaStream_t st)
+cudaError_t launch_gripper_cloud(const float4 *S, int N, float4 *out, float4 *frame, double *out12, cudaStream_t st)
 {
     static_assert(kMaxN <= 8192, "shared-memory sort");
     int Npow = 2;
     while (Npow < N) Npow <<= 1;
-    sort_points_kernel<<<1, 1024, (size_t)Npow * sizeof(unsigned long long), st>>>(S, N, Npow, out, frame);
+    gripper_cloud_kernel<<<2, 1024, (size_t)Npow * sizeof(unsigned long long), st>>>(S, N, Npow, out, frame, out12);
     return cudaGetLastError();
 }
 

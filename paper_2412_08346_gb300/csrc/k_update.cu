@@ -613,47 +613,6 @@ cudaError_t launch_check_finite(const float *v, long long n, int *err, cudaStrea
     return cudaGetLastError();
 }
 
-// Deterministic single-CTA float64 reductions (fixed thread striding + fixed tree).
-template <int NV, class F>
-__device__ void block_sum_f64(int n, F term, double *out)
-{
-    __shared__ double red[32][NV];
-    double acc[NV];
-    for (int c = 0; c < NV; ++c) acc[c] = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) term(i, acc);
-    warp_sum_f64(acc);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0)
-        for (int c = 0; c < NV; ++c) red[warp][c] = acc[c];
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w][threadIdx.x];
-        out[threadIdx.x] = s;
-    }
-}
-
-__global__ void preshape_consts_kernel(const float4 *S, int N, double *out12)
-{
-    __shared__ double tmp[9];
-    block_sum_f64<9>(N, [&](int i, double *acc) {
-        const float4 s = S[i];
-        const double x = s.x, y = s.y, z = s.z;
-        acc[0] += x; acc[1] += y; acc[2] += z;
-        acc[3] = fma(x, x, acc[3]); acc[4] = fma(x, y, acc[4]); acc[5] = fma(x, z, acc[5]);
-        acc[6] = fma(y, y, acc[6]); acc[7] = fma(y, z, acc[7]); acc[8] = fma(z, z, acc[8]);
-    }, tmp);
-    __syncthreads();
-    if (threadIdx.x < 9) out12[threadIdx.x] = tmp[threadIdx.x];
-    if (threadIdx.x >= 9 && threadIdx.x < 12) out12[threadIdx.x] = 0.0;
-}
-
-cudaError_t launch_preshape_consts(const float4 *S, int N, double *out12, cudaStream_t st)
-{
-    preshape_consts_kernel<<<1, 1024, 0, st>>>(S, N, out12);
-    return cudaGetLastError();
-}
-
 // Fibonacci sphere of K directions around the CoM (Section V); the same set for
 // every preshape.  u_j: z = 1 - (2j+1)/K, azimuth j * pi * (3 - sqrt 5);
 // t_j = CoM + radius u_j; q_j the smallest rotation taking +z (the approach
