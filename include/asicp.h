@@ -63,8 +63,9 @@ typedef enum {
  *   profile       1: time the main kernels with CUDA events (asicp_kernel_times);
  *                  2: time the forward-matching (screening) kernel only.  The events
  *                  are nodes of the captured iteration loop and add a few
- *                  microseconds each to a pass (profile 1: ~5 % of a paper-scale
- *                  grasp set on GB300)
+ *                  microseconds each to a pass, and with 1 the collision test no longer
+ *                  runs beside the matching (a paper-scale grasp set on GB300: 9.6 ms
+ *                  untimed, 10.8 with 2, 13.5 with 1)
  *   cuda_stream   cudaStream_t for all work, NULL for the default stream
  *   n_objects     objects optimised together in one pass (one grasp set each, default 1);
  *                  every kernel covers all of them, each particle matched against its
@@ -77,7 +78,10 @@ typedef enum {
  *                  tensor-core screening with its exact-choice kernel (not with mini-batches),
  *                  which clouds of 1024 to 2^18 points replace, once the passes so far would
  *                  have paid for the build, by cells around the object that keep the points
- *                  which can be nearest in them (same results).  Cells take 9.7 MB and
+ *                  which can be nearest in them (same results but for near-ties: which of
+ *                  the two decides depends on the passes so far, so for poses about a metre
+ *                  and more from the object equal steps may differ in near-ties and what
+ *                  follows from them).  Cells take 9.7 MB and
  *                  1.15 KB per point of every object, at most an eighth of the free
  *                  device memory in all; without room, and for clouds on which they
  *                  would be slower (points on a common sphere, cylinder or plane,

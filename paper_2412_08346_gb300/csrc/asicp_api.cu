@@ -120,13 +120,15 @@ struct ObjBufs {
     bool set = false, cells_built = false, sorted = false;
 };
 
-// Matching through cells (k_cells.cu): for clouds of kCellMinM points and more (the screening
-// reads the same eight tiles for any smaller one) up to kCellMaxM (the build's 32-bit
-// counters cannot overflow below it), once the passes known of on the present objects (those of
-// an asicp_run, or the asicp_step calls so far) would take longer through the screening than
-// the build: screening and exact choice take 1 us per kCellRate pairs, the build 100 us + 1 us
-// per kCellRatePts points (measured: 0.27 ms at 8192 points, 1.4 ms at 65536), the matching
-// through the cells little beside either.
+// Matching through cells (k_cells.cu): for clouds of kCellMinM points and more up to kCellMaxM
+// (the build's 32-bit counters cannot overflow below it), once the passes known of on the
+// present objects (those of an asicp_run, or the asicp_step calls so far) would take longer
+// through the screening than the build: screening and exact choice take 1 us per kCellRate
+// pairs, the build 100 us + 1 us per kCellRatePts points (measured: 0.27 ms at 8192 points,
+// 1.4 ms at 65536), the matching through the cells little beside either.  kCellMinM keeps the
+// tables (9.7 MB for the smallest cloud) from batches of many small clouds; it is not where the
+// cells stop paying: 1.6 M queries on 256 / 512 / 1000 points take 160 / 181 / 230 us through
+// the screening and 29 / 30 / 32 through cells (on 128 points the screening stays the cheaper).
 constexpr int kCellMinM = 1024, kCellMaxM = 1 << 18;
 constexpr double kCellRate = 1.65e7, kCellRatePts = 50.0;
 // Clouds whose lists do not shrink (points on a common sphere or plane, many copies of a point) are matched faster by

@@ -25,8 +25,8 @@ int per_device_value(int (&cache)[kDeviceSlots], std::mutex &mu, F compute)
 }
 
 constexpr int kRefTilePts = 2048;      // object points per shared-memory tile of the matching kernel
-constexpr int kFwdSums = 13;           // per-particle matching sums (see match kernel)
-constexpr int kColSums = 22;           // per-particle collision sums (see collision kernel)
+constexpr int kFwdSums = 13;           // per-particle matching sums (see finalize_kernel)
+constexpr int kColSums = 22;           // per-particle collision sums (see finalize_kernel)
 constexpr int kMaxK = 1024;            // particles per preshape (one update CTA per preshape)
 constexpr int kMaxN = 6144;            // gripper points per preshape (reverse matching keeps 32 B per point in shared memory)
 

@@ -379,12 +379,10 @@ __global__ void __launch_bounds__(kColThreads) collide_nn_kernel(const CollideAr
     __shared__ float s_smax[kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int slots = Npad / 64;                 // point pairs per lane
-    // Two barriers per item.  Thread 0 takes the next item right after the first
-    // (its index is read at the top of the loop, after the second).  After the
-    // second barrier the transformed cloud and sC are no longer read, so the
-    // next item may overwrite them while slower threads still add this item's
-    // sums; those read only sRec, which the next item writes after its own
-    // first barrier.
+    // Two barriers per item.  The first parts the writes of the transformed cloud, sC and
+    // s_smax from their reads; thread 0 takes the next item right after it (every thread has
+    // read s_item at the top of the loop by then).  After the second nothing of this item is
+    // read any more, and s_item holds the next one.
     if (threadIdx.x == 0) s_item = atomicAdd(&a.col_items[1], 1);
     __syncthreads();
     for (;;) {
@@ -445,7 +443,7 @@ __global__ void __launch_bounds__(kColThreads) collide_nn_kernel(const CollideAr
         const float smax = sqrtf(sm2) * 1.0001f;
 
         // colliding points of this warp (warp-uniform): a warp whose eight slots are all past the
-        // particle's count (the padding of its last item) skips the matching; its records are zeros
+        // particle's count (the padding of its last item) skips the matching
         const int g = lane >> 2, gs = lane & 3;       // lane group g works on colliding point g
         const float4 cq = sC[warp * kQW + g];
         float best = __int_as_float(0x7f800000);

@@ -1,4 +1,4 @@
-// Forward matching: transform + brute-force nearest neighbour + per-particle sums.
+// Forward matching: transform + brute-force nearest neighbour.
 //
 // For particle (p, j) and gripper point i the kernel forms s'_i = R_j s_i + t_j
 // (Algorithm 1, "transform the source cloud") and finds the object point with
