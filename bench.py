@@ -54,6 +54,7 @@ EPILOGUE_OPS_PER_PAIR = 1   # the tensor-core shape's epilogue: one compare per 
 # cells_match_kernel, of the committed ncu capture of a paper-scale launch
 # (profiles/pass_kernels_paper-scale-P3-K256-N2048-M8192.md): executed lane instructions per gripper point
 # (transform, cell look-up, about 12 exact distances; 19.97 M warp instructions for 1.573 M points) and DRAM bytes
+CELLS_CAPTURED = (3, 256, 2048, 8192)      # (P, K, N, M) of that launch
 CELLS_LANE_INST_PER_QUERY = 406
 CELLS_DRAM_BYTES_PER_LAUNCH = 3054848
 TC_SHAPE = "tc-f16x3-m128-n256"
@@ -406,7 +407,7 @@ def run_gpu(args, rank, world, local_rank):
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     cells = tc and launches[5] == 0       # no exact choice after the matching: it went through the cells
     if cells:
-        roofline = cells_roofline_entry(P * K * N, M, match_avg_s, ms, sms, clk)
+        roofline = cells_roofline_entry((P, K, N, M), match_avg_s, ms, sms, clk)
     else:
         roofline = roofline_entry(tc, pairs_per_launch, match_avg_s, exact_avg_s, ms, sms, clk)
     # match, collide, collide_nn, finalize per pass (+ the exact choice after the tensor-core screening),
@@ -517,23 +518,30 @@ def roofline_entry(tc, pairs_per_launch, match_avg_s, exact_avg_s, ms, sms, clk)
             "sms": sms, "sm_mhz": mhz}
 
 
-def cells_roofline_entry(queries, M, match_avg_s, ms, sms, clk):
+def cells_roofline_entry(sizes, match_avg_s, ms, sms, clk):
     """Roofline of cells_match_kernel in gripper points (queries) per second: the issue rate, SMs x 128
-    lane instructions per clock over the instructions a query executes (counted once by ncu).  The
-    rate of brute-force pairs that the search stands for is reported beside it."""
-    mhz = clk.get("sm_mhz") or SM_MAX_MHZ_NOMINAL
-    peak = sms * FP32_LANES_PER_SM * mhz * 1e6 / CELLS_LANE_INST_PER_QUERY
+    lane instructions per clock over the instructions a query executes, counted once by ncu for the
+    paper-scale sizes (P, K, N, M); for other sizes neither that peak nor the DRAM traffic is known and both are
+    null.  The rate of brute-force pairs that the search stands for is reported beside it."""
+    P, K, N, M = sizes
+    queries = P * K * N
     achieved = queries / match_avg_s
-    return {"bound": "alu", "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Gqueries/s",
-            "frac": achieved / peak, "kernel": "cells_match_kernel",
-            "peak_basis": f"{sms} SMs x {FP32_LANES_PER_SM} lane instructions per clock x {mhz:.0f} MHz / "
-                          f"{CELLS_LANE_INST_PER_QUERY} executed lane instructions per query (ncu)",
-            "traffic": CELLS_DRAM_BYTES_PER_LAUNCH,
-            "traffic_basis": "dram__bytes_read+write of one paper-scale launch from cold caches (ncu); cells, points "
-                             "and poses are L2-resident between the passes",
-            "launch_ms": match_avg_s * 1e3, "queries_per_launch": queries, "pairs_per_launch": queries * M,
-            "matching_pairs_per_s": queries * M / match_avg_s, "kernel_share": ms[0] / max(1e-9, sum(ms)),
-            "sms": sms, "sm_mhz": mhz}
+    entry = {"bound": "alu", "achieved": achieved / 1e9, "peak": None, "unit": "Gqueries/s", "frac": None,
+             "kernel": "cells_match_kernel", "peak_basis": "no capture of this workload", "traffic": None,
+             "traffic_basis": "no capture of this workload",
+             "launch_ms": match_avg_s * 1e3, "queries_per_launch": queries, "pairs_per_launch": queries * M,
+             "matching_pairs_per_s": queries * M / match_avg_s, "kernel_share": ms[0] / max(1e-9, sum(ms)),
+             "sms": sms, "sm_mhz": clk.get("sm_mhz") or SM_MAX_MHZ_NOMINAL}
+    if sizes == CELLS_CAPTURED:
+        mhz = entry["sm_mhz"]
+        peak = sms * FP32_LANES_PER_SM * mhz * 1e6 / CELLS_LANE_INST_PER_QUERY
+        entry.update(peak=peak / 1e9, frac=achieved / peak,
+                     peak_basis=f"{sms} SMs x {FP32_LANES_PER_SM} lane instructions per clock x {mhz:.0f} MHz / "
+                                f"{CELLS_LANE_INST_PER_QUERY} executed lane instructions per query (ncu)",
+                     traffic=CELLS_DRAM_BYTES_PER_LAUNCH,
+                     traffic_basis="dram__bytes_read+write of one paper-scale launch from cold caches (ncu); cells, "
+                                   "points and poses are L2-resident between the passes")
+    return entry
 
 
 def measured_peaks():
