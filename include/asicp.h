@@ -244,7 +244,10 @@ asicp_status asicp_step(asicp_ctx *ctx, int k);
  * K_g poses of radius init_radius around its object's CoM (Section V); k_max steps;
  * a final evaluation of cost and collisions at the last poses; and the per-object
  * ranking used by asicp_best_grasps (Algorithm 1's argmin).  The loop is replayed
- * from a captured CUDA graph.  Errors: STATE, INVALID_ARG, CUDA. */
+ * from a captured CUDA graph.  The call returns once the loop is enqueued; with
+ * theta0 it waits for their check first, and with new clouds whose cells are due (see
+ * config.fwd_shape) for the count that decides whether they are used (about the time
+ * of their build, 0.1 to 3 ms).  Errors: STATE, INVALID_ARG, CUDA. */
 asicp_status asicp_run(asicp_ctx *ctx, const float *theta0);
 
 /* The topk best particles of object 0 in the last asicp_run: non-colliding first,

@@ -914,7 +914,7 @@ void ensure_pre_cells(asicp_ctx *c, int passes)
                 b.M = c->N;
                 b.log_factor = kGripperCells;
                 b.tol = kGripperTol;
-                    builds.push_back(b);
+                builds.push_back(b);
             }
         }
     } catch (const Err &e) {
